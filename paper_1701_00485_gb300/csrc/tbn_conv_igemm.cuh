@@ -1036,7 +1036,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     const uint32_t lane_off = static_cast<uint32_t>(sub * 32) << 16;
     const int Po = kPoolBW ? a.P / 2 : a.P;
     const int Qo = kPoolBW ? a.Q / 2 : a.Q;
-    const uint32_t res_bytes = static_cast<uint32_t>(a.bw * a.bh * a.bn * kBM * 2);
+    const uint32_t res_half_bytes = static_cast<uint32_t>(a.bw * a.bh * a.bn * (kBM / 2) * 2);
     __nv_bfloat16* stage = reinterpret_cast<__nv_bfloat16*>(out_stage);
     grid_dependency_wait();   // the residual may come from the previous kernel
     uint32_t tiles_done = 0;
@@ -1058,13 +1058,14 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         if (elected) bulk_wait_group_read<0>();
         named_barrier_sync(1, 32 * kEpiWarps);
         if (ok && a.residual && elected) {
-          mbar_arrive_expect_tx(&ctl->res_full, res_bytes);
-          asm volatile(
-              "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-              " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_addr(stage)),
-              "l"(&tmap_res), "r"(smem_addr(&ctl->res_full)), "r"(tc.ktile * kBM),
-              "r"(tc.q0), "r"(tc.p0), "r"(tc.n0)
-              : "memory");
+          // the residual box, in the staging tile's own layout (two swizzled
+          // halves of 64 filters), lands where the outputs will be staged
+          const bool both = tc.ktile * kBM + kBM / 2 < a.K;
+          mbar_arrive_expect_tx(&ctl->res_full, both ? 2 * res_half_bytes : res_half_bytes);
+          tma_load_4d(stage, &tmap_res, &ctl->res_full, tc.ktile * kBM, tc.q0, tc.p0, tc.n0);
+          if (both)
+            tma_load_4d(reinterpret_cast<uint8_t*>(stage) + 32768, &tmap_res, &ctl->res_full,
+                        tc.ktile * kBM + kBM / 2, tc.q0, tc.p0, tc.n0);
         }
       }
       if (ok)
@@ -1076,11 +1077,16 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       if (ok) tc_fence_after_sync();
       if (!ok) {
         // skip the work, keep the barrier schedule
-      } else if (kPoolBW == 0 && kTmaStore && a.residual == nullptr) {
+      } else if constexpr (kPoolBW == 0 && kTmaStore) {
         // Fragment epilogue: 16x256b loads (lane = filter, column = pixel),
-        // scale / ReLU / bf16 pairs, transposed 8x8 stores into the staging
-        // tile [pixel][filter] as two 128-byte-swizzled halves of 64
-        // filters (chunk c of pixel row px at c ^ (px & 7)).
+        // scale / residual / ReLU / bf16 pairs, transposed 8x8 stores into
+        // the staging tile [pixel][filter] as two 128-byte-swizzled halves of
+        // 64 filters (chunk c of pixel row px at c ^ (px & 7)).  The residual
+        // sits at the very addresses its outputs go to, and the transposed
+        // 8x8 loads deliver it in the fragment's own register layout, so it
+        // costs one ldmatrix per stmatrix.  (One 2-byte shared load and store
+        // per value took a 64-filter 56x56 layer at batch 128 from 49 to
+        // 103 us; this way the residual costs 51.4 MB more of reads, no more.)
         const int nchunks = (a.tile_n + 31) / 32;
         const int c_begin = half ? (nchunks + 1) / 2 : 0;
         const int c_end = half ? nchunks : (nchunks + 1) / 2;
@@ -1112,12 +1118,33 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
 #pragma unroll
           for (int lg = 0; lg < 2; ++lg) {
             uint32_t pk[8];
+            uint32_t addr[2];
+#pragma unroll
+            for (int bp = 0; bp < 2; ++bp) {
+              // matrices: (filters +0, block 2bp), (+8, 2bp), (+0, 2bp+1), (+8, 2bp+1)
+              const int px = 32 * j + 8 * (2 * bp + (mi >> 1)) + mrow;
+              const int chunk = 4 * sub + 2 * lg + (mi & 1);           // 8-filter chunk 0..15
+              addr[bp] = stage_s + static_cast<uint32_t>((chunk >> 3) * 32768 + px * 128 +
+                                                         (((chunk & 7) ^ (px & 7)) << 4));
+            }
+            if (a.residual) {
+#pragma unroll
+              for (int bp = 0; bp < 2; ++bp)
+                ldmatrix_x4_trans(addr[bp], pk[4 * bp + 0], pk[4 * bp + 1], pk[4 * bp + 2],
+                                  pk[4 * bp + 3]);
+            }
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
               float y0 = a2f[lg][0] * __uint_as_float(v[lg][4 * b + 0]);
               float y1 = a2f[lg][0] * __uint_as_float(v[lg][4 * b + 1]);
               float y2 = a2f[lg][1] * __uint_as_float(v[lg][4 * b + 2]);
               float y3 = a2f[lg][1] * __uint_as_float(v[lg][4 * b + 3]);
+              if (a.residual) {   // bf16 pairs, low half first
+                y0 += __uint_as_float(pk[2 * b] << 16);
+                y1 += __uint_as_float(pk[2 * b] & 0xFFFF0000u);
+                y2 += __uint_as_float(pk[2 * b + 1] << 16);
+                y3 += __uint_as_float(pk[2 * b + 1] & 0xFFFF0000u);
+              }
               if (a.relu) {
                 y0 = fmaxf(y0, 0.0f);
                 y1 = fmaxf(y1, 0.0f);
@@ -1128,15 +1155,9 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
               pk[2 * b + 1] = pack_bf16x2(y2, y3);   // filters fr + 8
             }
 #pragma unroll
-            for (int bp = 0; bp < 2; ++bp) {
-              // matrices: (filters +0, block 2bp), (+8, 2bp), (+0, 2bp+1), (+8, 2bp+1)
-              const int px = 32 * j + 8 * (2 * bp + (mi >> 1)) + mrow;
-              const int chunk = 4 * sub + 2 * lg + (mi & 1);           // 8-filter chunk 0..15
-              const uint32_t addr = stage_s + static_cast<uint32_t>((chunk >> 3) * 32768 + px * 128 +
-                                                                    (((chunk & 7) ^ (px & 7)) << 4));
-              stmatrix_x4_trans(addr, pk[4 * bp + 0], pk[4 * bp + 1], pk[4 * bp + 2],
+            for (int bp = 0; bp < 2; ++bp)
+              stmatrix_x4_trans(addr[bp], pk[4 * bp + 0], pk[4 * bp + 1], pk[4 * bp + 2],
                                 pk[4 * bp + 3]);
-            }
           }
         }
         if (c_begin >= c_end) {
@@ -1160,7 +1181,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
             tc_fence_before_sync();
             mbar_arrive(&ctl->acc_empty[ab]);
           }
-          if (!kTmaStore && a.partial != nullptr) {
+          if (a.partial != nullptr) {
             // split K (1x1 image): pixel px is image n0 + px; the raw sum of
             // this K range goes to partial[split][n][k]
             float* dst = a.partial + (static_cast<size_t>(tc.split) * a.N + tc.n0 + 32 * j) * a.K + k;
@@ -1168,18 +1189,6 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
             for (int i = 0; i < 32; ++i)
               if (kvalid && 32 * j + i < T && tc.n0 + 32 * j + i < a.N)
                 dst[static_cast<size_t>(i) * a.K] = __uint_as_float(v[i]);
-          } else if (kTmaStore) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const int px = 32 * j + i;
-              if (px < T) {
-                float y = a2 * __uint_as_float(v[i]);
-                __nv_bfloat16* sp = stage + px * kBM + m;
-                if (a.residual) y += __bfloat162float(*sp);
-                if (a.relu) y = fmaxf(y, 0.0f);
-                *sp = __float2bfloat16_rn(y);
-              }
-            }
           } else {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
@@ -1259,13 +1268,11 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         if (elected && ok) {
           if (kPoolBW) {
             tma_store_4d(&tmap_y, stage, tc.ktile * kBM, 0, tc.p0 / 2, tc.n0);
-          } else if (a.residual == nullptr) {
+          } else {
             tma_store_4d(&tmap_y, stage, tc.ktile * kBM, tc.q0, tc.p0, tc.n0);
             if (tc.ktile * kBM + kBM / 2 < a.K)
               tma_store_4d(&tmap_y, reinterpret_cast<uint8_t*>(stage) + 32768,
                            tc.ktile * kBM + kBM / 2, tc.q0, tc.p0, tc.n0);
-          } else {
-            tma_store_4d(&tmap_y, stage, tc.ktile * kBM, tc.q0, tc.p0, tc.n0);
           }
           bulk_commit_group();
         }
@@ -1384,12 +1391,12 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
     if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "cuTensorMapEncodeTiled(x) failed (%d)", (int)cr);
   }
   if (kTmaStore) {
-    // the fragment epilogue (no pool, no residual) stages two swizzled halves
-    const bool halves = kPoolBW == 0 && p.residual == nullptr;
+    // the fragment epilogue (no pool) stages two swizzled halves
+    const bool halves = kPoolBW == 0;
     CUresult cr = encode_out_map(&tmap_y, p.y, p, t, kPoolBW ? 1 : 0, halves);
     if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "cuTensorMapEncodeTiled(y) failed (%d)", (int)cr);
     if (p.residual) {
-      cr = encode_out_map(&tmap_res, p.residual, p, t, 0);
+      cr = encode_out_map(&tmap_res, p.residual, p, t, 0, true);
       if (cr != CUDA_SUCCESS)
         return fail(TBN_ERR_CUDA, "cuTensorMapEncodeTiled(residual) failed (%d)", (int)cr);
     }
