@@ -159,11 +159,12 @@ const char* conv_igemm_unsupported_reason(const ConvProblem& p) {
 tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const bool s2d = p0.layout == TBN_S2D_NHWC;
   const ConvProblem p = s2d ? s2d_problem(p0) : p0;
-  const TilePlan t = plan_tiles(p);
+  const TilePlan t = plan_conv(p, s2d);
   IgArgs a{};
-  a.N = (int)p.N; a.C = (int)p.C; a.H = (int)p.H; a.W = (int)p.W; a.K = (int)p.K;
+  a.N = (int)t.oN; a.C = (int)p.C; a.H = (int)p.H; a.W = (int)p.W; a.K = (int)p.K;
   a.R = (int)p.R; a.S = (int)p.S; a.sh = (int)p.sh; a.sw = (int)p.sw;
-  a.ph = (int)p.ph; a.pw = (int)p.pw; a.P = (int)p.P; a.Q = (int)p.Q;
+  a.ph = (int)p.ph; a.pw = (int)p.pw; a.P = (int)t.oP; a.Q = (int)t.oQ;
+  a.im2col = t.im2col ? 1 : 0; a.iP = (int)p.P; a.iQ = (int)p.Q;
   a.bw = t.bw; a.bh = t.bh; a.bn = t.bn; a.tile_n = t.tile_n;
   a.tiles_q = t.tiles_q; a.tiles_p = t.tiles_p;
   a.tiles_k = ceil_div(p.K, kBM);

@@ -25,6 +25,9 @@
 //                   64 channels and one TMA box load fetches it (the box is
 //                   the tile's output pixels shifted by the tap; zero fill
 //                   supplies the padding, element strides the conv stride).
+//                   A tile is a run of consecutive output pixels of the
+//                   whole batch, fetched in im2col mode, or whole output
+//                   rows, fetched as a tiled box (see plan_conv).
 //                   When C % 32 == 0 (e.g. 96 channels) a K block is two
 //                   boxes of 32 channels, each from its own tap, into two
 //                   64-byte-row halves of the stage with the 64-byte swizzle
@@ -104,6 +107,10 @@ struct IgArgs {
   const void* residual;
   int relu, y_bf16;
   uint32_t* err;
+  // im2col tiles: N, P and Q above are the extents that the tiles walk (the
+  // batch as one row of N P Q pixels, or as one image of N P rows when
+  // pooling); an image's output is iP x iQ
+  int im2col, iP, iQ;
   // patch mode: the patch is rows [p0 sh - ph, + PR) x columns [-pw, W + pw)
   int PR, PW;              // patch rows, patch columns (W + 2 pw)
   int patch_cap;           // bytes per patch buffer (multiple of 16)
@@ -134,6 +141,8 @@ struct IgArgs {
 
 struct TilePlan {
   int bw, bh, bn, T, tile_n, tiles_q, tiles_p, tiles_n;
+  bool im2col;             // tiles of consecutive pixels over the whole batch
+  int64_t oN, oP, oQ;      // output extents that the tiles walk
 };
 
 namespace {
@@ -505,6 +514,15 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     bool ok = true;
     for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
       const TileCoord tc = tile_coord(a, t);
+      // base input position of the tile's first pixel
+      int w0 = tc.q0 * a.sw - a.pw, h0 = tc.p0 * a.sh - a.ph, n0 = tc.n0;
+      if (a.im2col) {
+        const int f = tc.p0 * a.Q + tc.q0;
+        const int row = f / a.iQ;
+        n0 = row / a.iP;
+        w0 = (f - row * a.iQ) * a.sw - a.pw;
+        h0 = (row - n0 * a.iP) * a.sh - a.ph;
+      }
       // (tap, channel box) of the next box
       int tap = (tc.kb0 * kBoxes) / cblocks, cb = (tc.kb0 * kBoxes) % cblocks;
       for (int kb = tc.kb0; kb < tc.kb1; ++kb, ++g) {
@@ -529,9 +547,12 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
             const bool past = tap >= a.R * a.S;
             const int tp = past ? 0 : tap;
             const int r = tp / a.S, s = tp - r * a.S;
-            tma_load_4d(ring + sb * kStageBytes + bx * (kStageBytes / kBoxes), &tmap_x,
-                        &ctl->full[sb], past ? a.C : cb * kBoxCh, tc.q0 * a.sw - a.pw + s,
-                        tc.p0 * a.sh - a.ph + r, tc.n0);
+            uint8_t* dst = ring + sb * kStageBytes + bx * (kStageBytes / kBoxes);
+            const int c0 = past ? a.C : cb * kBoxCh;
+            if (a.im2col)
+              tma_load_im2col_4d(dst, &tmap_x, &ctl->full[sb], c0, w0, h0, n0, s, r);
+            else
+              tma_load_4d(dst, &tmap_x, &ctl->full[sb], c0, w0 + s, h0 + r, n0);
             if (++cb == cblocks) { cb = 0; ++tap; }
           }
         } else {
@@ -1331,6 +1352,10 @@ inline TilePlan plan_tiles(const ConvProblem& p) {
   t.tiles_n = ceil_div(p.N, t.bn);
   t.T = t.bw * t.bh * t.bn;
   t.tile_n = ((t.T + 15) / 16) * 16;
+  t.im2col = false;
+  t.oN = p.N;
+  t.oP = p.P;
+  t.oQ = p.Q;
   return t;
 }
 
@@ -1339,6 +1364,95 @@ inline int pool_width(const ConvProblem& p, const TilePlan& t) {
   if (t.tiles_q != 1 || t.T > kMaxTileN || (t.bh & 1)) return -1;
   if (t.bw == 8 || t.bw == 16 || t.bw == 32) return t.bw;
   return -1;
+}
+
+// Estimated time (ns) of a TMA-mode plan.  A K block of a T-pixel tile takes
+// about 215 + 0.25 T ns on a CTA (fitted to the AlexNet and ResNet-18 layers:
+// 256 ns at 176 pixels, 264 at 224, 285 at 256: supplying the operands costs
+// nearly the same whatever the width), a tile about 0.9 us more, with a
+// single accumulator, which its epilogue holds, 1.7 us.  CTAs take whole
+// tiles, so what counts is the largest number any of them gets.
+inline double plan_cost(const ConvProblem& p, const TilePlan& t, bool resident, int sms) {
+  const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n *
+                        ((p.K + kBM - 1) / kBM);
+  const double waves = static_cast<double>((tiles + sms - 1) / sms);
+  const double kb = static_cast<double>((p.C * p.R * p.S + kBK - 1) / kBK);
+  const bool acc2 = !resident && t.tile_n <= kAcc2Cols;
+  return waves * (kb * (215.0 + 0.25 * t.tile_n) + (acc2 ? 900.0 : 1700.0));
+}
+
+// Whether the activations can be fetched in im2col mode: the limits of the
+// tensor map (corner offsets of a 4-D map are 8 bits, tap offsets unsigned),
+// 32-bit pixel indices, and at least 128 KiB of input (smaller tensors are
+// left to tiled boxes, which is where the one-image layers are).
+inline bool im2col_ok(const ConvProblem& p) {
+  return use_tma(p) && p.R <= 128 && p.S <= 128 && p.ph <= 127 && p.pw <= 127 &&
+         p.N * p.P * p.Q <= (int64_t(1) << 30) && p.N * p.H * p.W * p.C * 2 >= 131072 &&
+         get_encode_im2col() != nullptr;
+}
+
+// The tile plan of a launch.  Gathering modes and split K: plan_tiles.  TMA
+// modes: the cheapest (plan_cost) of plan_tiles, of runs of T consecutive
+// pixels of the whole batch where im2col mode can fetch them (T a multiple
+// of 16, or of two output rows when pooling), and otherwise of fewer rows per
+// tile.  Whole-image tiles leave the last wave nearly empty (13 x 13 images,
+// 384 filters, batch 256: 768 tiles on 152 SMs, six waves for 5.05) or their
+// columns short of 256; runs of pixels are cut to the machine instead:
+// four waves of 224 (that layer at 1152 codes per filter: 63.9 -> 50.6 us,
+// at 3456: 91.4 -> 69.7; the AlexNet step at batch 256: 680 -> 627 us).  `resident`: the space-to-depth mode, whose K blocks
+// stay beside the accumulator.
+inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
+  TilePlan best = plan_tiles(p);
+  if (!use_tma(p) || p.ksplit > 1) return best;
+  const int sms = device_sm_count();
+  double cost = plan_cost(p, best, resident, sms);
+  const auto consider = [&](const TilePlan& t) {
+    const double c = plan_cost(p, t, resident, sms);
+    if (c < cost) {
+      cost = c;
+      best = t;
+    }
+  };
+  const int kb = ceil_div(p.C * p.R * p.S, kBK);
+  const int t_max = resident ? std::min(kMaxTileN, kTmemCols - 32 * kb) : kMaxTileN;
+  if (im2col_ok(p)) {
+    TilePlan t = best;
+    t.im2col = true;
+    t.oN = 1;
+    t.tiles_n = t.bn = 1;
+    if (!p.pool) {
+      t.oP = 1;
+      t.oQ = p.N * p.P * p.Q;
+      t.tiles_p = t.bh = 1;
+      for (int T = 16; T <= t_max; T += 16) {
+        t.T = t.bw = t.tile_n = T;
+        t.tiles_q = ceil_div(t.oQ, T);
+        consider(t);
+      }
+    } else if (p.P % 2 == 0 && (p.Q == 8 || p.Q == 16 || p.Q == 32)) {
+      // row pairs of all images in sequence (P even: none crosses images)
+      t.oP = p.N * p.P;
+      t.oQ = p.Q;
+      t.bw = static_cast<int>(p.Q);
+      t.tiles_q = 1;
+      for (int rows = 2; rows * t.bw <= t_max; rows += 2) {
+        t.bh = rows;
+        t.T = t.tile_n = rows * t.bw;
+        t.tiles_p = ceil_div(t.oP, rows);
+        consider(t);
+      }
+    }
+  } else if (!p.pool && best.tiles_q == 1 && best.bn == 1) {
+    TilePlan t = best;
+    for (int rows = 1; rows < best.bh; ++rows) {
+      t.bh = rows;
+      t.T = t.bw * rows;
+      t.tile_n = ((t.T + 15) / 16) * 16;
+      t.tiles_p = ceil_div(p.P, rows);
+      consider(t);
+    }
+  }
+  return best;
 }
 
 inline bool use_tma_store(const ConvProblem& p) {
@@ -1351,8 +1465,8 @@ inline bool use_tma_store(const ConvProblem& p) {
 // staging layout of the fragment epilogue, two stores per tile).
 inline CUresult encode_out_map(CUtensorMap* m, const void* base, const ConvProblem& p, const TilePlan& t,
                         int pool, bool halves = false) {
-  const int64_t Po = pool ? p.P / 2 : p.P, Qo = pool ? p.Q / 2 : p.Q;
-  const cuuint64_t gdim[4] = {(cuuint64_t)p.K, (cuuint64_t)Qo, (cuuint64_t)Po, (cuuint64_t)p.N};
+  const int64_t Po = pool ? t.oP / 2 : t.oP, Qo = pool ? t.oQ / 2 : t.oQ;
+  const cuuint64_t gdim[4] = {(cuuint64_t)p.K, (cuuint64_t)Qo, (cuuint64_t)Po, (cuuint64_t)t.oN};
   const cuuint64_t gstride[3] = {(cuuint64_t)(p.K * 2), (cuuint64_t)(Qo * p.K * 2),
                                  (cuuint64_t)(Po * Qo * p.K * 2)};
   const cuuint32_t box[4] = {(cuuint32_t)(halves ? kBM / 2 : kBM), (cuuint32_t)(pool ? t.bw / 2 : t.bw),
@@ -1376,19 +1490,31 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
     const cuuint64_t gdim[4] = {(cuuint64_t)p.C, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.N};
     const cuuint64_t gstride[3] = {(cuuint64_t)(p.C * 2), (cuuint64_t)(p.W * p.C * 2),
                                    (cuuint64_t)(p.H * p.W * p.C * 2)};
-    const cuuint32_t box[4] = {(cuuint32_t)(kCh32 ? kBK / 2 : kBK), (cuuint32_t)(t.bw * p.sw),
-                               (cuuint32_t)(t.bh * p.sh), (cuuint32_t)t.bn};
     const cuuint32_t estr[4] = {1u, (cuuint32_t)p.sw, (cuuint32_t)p.sh, 1u};
-    if (box[1] > 256 || box[2] > 256 || box[3] > 256)
-      return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: TMA box too large");
-    const CUresult cr = get_encode_tiled()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
-                                           const_cast<void*>(p.x), gdim, gstride, box, estr,
-                                           CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                           kCh32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                                 : CU_TENSOR_MAP_SWIZZLE_128B,
-                                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "cuTensorMapEncodeTiled(x) failed (%d)", (int)cr);
+    const cuuint32_t channels = kCh32 ? kBK / 2 : kBK;
+    const CUtensorMapSwizzle swizzle = kCh32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+    CUresult cr;
+    if (t.im2col) {
+      // base positions [-pad, size - 1 + pad - (kernel - 1)] in steps of the stride
+      const int lower[2] = {-(int)p.pw, -(int)p.ph};
+      const int upper[2] = {(int)(p.pw - (p.S - 1)), (int)(p.ph - (p.R - 1))};
+      cr = get_encode_im2col()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
+                               const_cast<void*>(p.x), gdim, gstride, lower, upper, channels,
+                               (cuuint32_t)t.T, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {
+      const cuuint32_t box[4] = {channels, (cuuint32_t)(t.bw * p.sw), (cuuint32_t)(t.bh * p.sh),
+                                 (cuuint32_t)t.bn};
+      if (box[1] > 256 || box[2] > 256 || box[3] > 256)
+        return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: TMA box too large");
+      cr = get_encode_tiled()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
+                              const_cast<void*>(p.x), gdim, gstride, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "tensor map of x failed (%d)", (int)cr);
   }
   if (kTmaStore) {
     // the fragment epilogue (no pool) stages two swizzled halves

@@ -187,6 +187,20 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const void* tmap, uint64_
       : "memory");
 }
 
+// 4-D im2col bulk tensor load global -> shared: the map's pixel count of
+// consecutive base positions (over columns, then rows, then images) from
+// (c0, w, h, n) on, each shifted by (off_w, off_h); completion on an mbarrier.
+__device__ __forceinline__ void tma_load_im2col_4d(void* dst, const void* tmap, uint64_t* bar,
+                                                   int c0, int w, int h, int n, int off_w,
+                                                   int off_h) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};" ::"r"(smem_addr(dst)),
+      "l"(tmap), "r"(smem_addr(bar)), "r"(c0), "r"(w), "r"(h), "r"(n),
+      "h"(static_cast<uint16_t>(off_w)), "h"(static_cast<uint16_t>(off_h))
+      : "memory");
+}
+
 // 4-D tiled bulk tensor store shared -> global (out-of-range box elements
 // are clipped), tracked by this thread's bulk async-group.
 __device__ __forceinline__ void tma_store_4d(const void* tmap, const void* src, int c0, int c1,

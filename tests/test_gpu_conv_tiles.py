@@ -32,3 +32,48 @@ def test_residual_epilogue_filter_boxes(K, N, hw):
                       algo=tbn.TBN_CONV_IMPLICIT_GEMM, relu=relu, residual=res)
         assert_within(y, want, bound, out_bf16=True, epilogue=True,
                       what="residual K=%d N=%d %d" % (K, N, hw))
+
+
+RUNS = [
+    # N, C, H, W, K, R, S, stride, pad: inputs of at least 128 KiB, whose
+    # tiles are runs of pixels that cross rows and images
+    (9, 64, 13, 13, 136, 3, 3, (1, 1), (1, 1)),
+    (5, 64, 23, 21, 72, 3, 3, (2, 2), (1, 1)),      # odd sizes, stride 2
+    (3, 96, 27, 29, 64, 5, 5, (1, 1), (2, 2)),      # 32-channel boxes, ragged last block
+    (7, 128, 15, 15, 128, 1, 1, (2, 2), (0, 0)),    # projection shortcut
+    (3, 64, 40, 30, 40, 2, 3, (1, 2), (1, 0)),      # R != S, stride and pad differ by axis
+    (2, 128, 3, 300, 128, 3, 3, (1, 1), (1, 1)),    # rows longer than a tile
+    (300, 64, 2, 2, 64, 3, 3, (1, 1), (1, 1)),      # a tile holds many images
+]
+
+
+@pytest.mark.parametrize("case", RUNS)
+def test_pixel_run_tiles(case):
+    c = _case(*case, seed=sum(case[:7]))
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.float32,
+                  algo=tbn.TBN_CONV_IMPLICIT_GEMM)
+    assert_within(y, y_orc, bound, out_bf16=False, what="runs %s" % (case,))
+    res = torch.randn(*y_orc.shape, generator=inputs.generator(3)).to(torch.bfloat16)
+    want = oracle.epilogue(y_orc, res.float().numpy(), relu=True)
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16,
+                  algo=tbn.TBN_CONV_IMPLICIT_GEMM, relu=True, residual=res)
+    assert_within(y, want, bound, out_bf16=True, epilogue=True, what="runs epi %s" % (case,))
+
+
+@pytest.mark.parametrize("N,C,hw", [(5, 128, 16), (21, 64, 8), (3, 96, 32)])
+def test_pixel_run_tiles_pooled(N, C, hw):
+    """Fused 2x2 pool over runs of row pairs that cross images."""
+    c = _case(N, C, hw, hw, 72, 3, 3, (1, 1), (1, 1), seed=N)
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    want = oracle.maxpool2d_nchw(oracle.epilogue(y_orc, None, relu=True), (2, 2), (2, 2))
+    P = hw // 2
+    bound = bound.reshape(N, 72, P, 2, P, 2).max(axis=(3, 5))
+    Wl, codes, alpha = c.quantize_gpu(tbn.TBN_NHWC)
+    x = c.x.to(torch.bfloat16).permute(0, 2, 3, 1).contiguous().cuda()
+    for dt in (torch.float32, torch.bfloat16):
+        y = tbn.tbn_conv2d_fwd(x, codes, alpha, 72, 3, 3, (1, 1), (1, 1), out_dtype=dt, relu=True,
+                               pool=2, algo=tbn.TBN_CONV_IMPLICIT_GEMM)
+        y = y.float().cpu().permute(0, 3, 1, 2).numpy()
+        assert_within(y, want, bound, out_bf16=dt == torch.bfloat16, epilogue=True,
+                      what="pooled runs %d %d" % (N, hw))
