@@ -474,8 +474,8 @@ tbn_status tbn_nchw_to_nhwc(const void *x, tbn_dtype dt, int64_t N, int64_t C, i
 /* ---- full-precision layers (network glue, not the paper's method) -------
  * Two-bit networks keep their first convolution and last fully-connected
  * layer in full precision (the ResNet-18 workload).  These calls compute
- * them on the CUDA cores in fp32: products x * w rounded to fp32 and added
- * in fp32. */
+ * them with fp32 weights and fp32 sums: products x * w rounded to fp32 (or
+ * exact) and added in fp32. */
 
 /* Dense convolution with fp32 weights w [K][C][R][S] (PyTorch order, any
  * activation layout): y = x cross-correlated with w, zero padding, no bias,

@@ -2,9 +2,11 @@
 // its TBN layers (network glue, not the paper's method): the first
 // convolution with fp32 weights, the global average pool and the last
 // fully-connected layer with fp32 weights (the ResNet-18 workload keeps
-// both ends in full precision).  All arithmetic is fp32 on the CUDA cores:
-// x * w products are rounded to fp32 and accumulated in fp32, which is what
-// "kept in fp32" means for these layers.
+// both ends in full precision).  All arithmetic here is fp32 on the CUDA
+// cores: x * w products are rounded to fp32 and accumulated in fp32, which is
+// what "kept in fp32" means for these layers.  The first convolution of a
+// bf16 network runs on the tensor cores instead where tbn_dense_tc.cu takes
+// it.
 //
 // Dense convolution: a persistent CTA takes tiles of 4 output rows x 32
 // output columns of one image for 64 filters.  Per chunk of input channels it
@@ -337,6 +339,7 @@ __global__ void __launch_bounds__(256) dense_linear_kernel(const float* __restri
 }  // namespace
 
 tbn_status launch_dense_conv(const ConvProblem& p, const float* w, cudaStream_t s) {
+  if (dense_conv_tc_takes(p)) return launch_dense_conv_tc(p, w, s);
   DenseConvArgs a{};
   a.N = (int)p.N; a.C = (int)p.C; a.H = (int)p.H; a.W = (int)p.W; a.K = (int)p.K;
   a.R = (int)p.R; a.S = (int)p.S; a.sh = (int)p.sh; a.sw = (int)p.sw;

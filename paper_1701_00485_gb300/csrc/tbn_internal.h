@@ -184,6 +184,9 @@ tbn_status launch_repack(const uint32_t* in, int64_t words, uint32_t* out, bool 
 
 // Full-precision layers around the two-bit ones (tbn_dense.cu).
 tbn_status launch_dense_conv(const ConvProblem& p, const float* w, cudaStream_t s);
+// Its tensor-core form (tbn_dense_tc.cu), for the shapes that it takes.
+bool dense_conv_tc_takes(const ConvProblem& p);
+tbn_status launch_dense_conv_tc(const ConvProblem& p, const float* w, cudaStream_t s);
 tbn_status launch_avgpool_global_nhwc(const void* x, tbn_dtype xdt, int64_t N, int64_t H,
                                       int64_t W, int64_t C, void* y, tbn_dtype ydt,
                                       cudaStream_t s);

@@ -1,0 +1,78 @@
+"""The tensor-core form of the full-precision first convolution (fp32 weights
+as three bf16 terms) against the oracle, at the edges of its tiles, filter
+groups and weight blocks, and with infinities and NaN.
+
+Tolerance: the products are exact and at most n = C*R*S sums of each of the
+three terms round in fp32, so |err| <= n * 2^-24 * sum|x w| as for the
+CUDA-core kernel, plus the bf16 rounding of the output."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1701_00485_gb300 as tbn
+from paper_1701_00485_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # N, C, H, W, K, R, S, stride, pad
+    (2, 3, 32, 32, 64, 7, 7, (2, 2), (3, 3)),     # two whole tiles per image
+    (3, 3, 30, 40, 72, 7, 7, (2, 2), (3, 3)),     # ragged last tile, second filter group
+    (1, 1, 8, 8, 8, 3, 3, (2, 2), (1, 1)),        # one partial tile, one block
+    (2, 4, 16, 24, 16, 5, 8, (1, 2), (0, 0)),     # 8 taps, even padding, row stride 1
+    (1, 5, 33, 64, 64, 8, 4, (4, 4), (2, 1)),     # all five weight blocks
+    (200, 3, 16, 16, 64, 7, 7, (2, 2), (3, 3)),   # several tiles per CTA
+    (1, 3, 9, 224, 8, 7, 7, (2, 2), (3, 3)),      # the widest rows of the workload
+]
+
+
+def _run(x, w, st, pd, relu=False):
+    y = tbn.tbn_dense_conv2d_fwd(x.cuda(), w.cuda(), st, pd, layout=tbn.TBN_NCHW_NHWC,
+                                 out_dtype=torch.bfloat16, relu=relu)
+    torch.cuda.synchronize()
+    assert tbn.tbn_device_error() == 0
+    return y.float().cpu().permute(0, 3, 1, 2).numpy()
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_dense_tc_matches_oracle(case):
+    N, C, H, W, K, R, S, st, pd = case
+    g = inputs.generator(sum(case[:7]))
+    x = torch.randn(N, C, H, W, generator=g).to(torch.bfloat16)
+    w = inputs.he_normal(K, C, R, S, g)
+    want, bound = oracle.dense_conv2d_nchw(x.float().numpy(), w.numpy(), st, pd)
+    for relu in (False, True):
+        ref = np.maximum(want, 0.0) if relu else want
+        err = np.abs(_run(x, w, st, pd, relu).astype(np.float64) - ref)
+        tol = C * R * S * 2.0 ** -24 * bound + 2.0 ** -8 * np.abs(ref)
+        assert np.all(err <= tol), float(np.max(err - tol))
+
+
+def test_dense_tc_weight_terms():
+    """Weights that need all three terms: one tap, so each output is a single
+    product rounded once to bf16, at most half an ulp away."""
+    g = inputs.generator(9)
+    x = torch.ones(1, 1, 8, 8, dtype=torch.bfloat16)
+    w = (torch.rand(64, 1, 1, 1, generator=g) + 1) * (1 + 2.0 ** -23)
+    y = _run(x, w, (1, 2), (0, 0))
+    want = w.reshape(1, 64, 1, 1).double().numpy() * np.ones(y.shape)
+    assert np.array_equal(y, torch.from_numpy(want).to(torch.bfloat16).float().numpy())
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.3e38])
+def test_dense_tc_not_finite(value):
+    """An infinite, NaN or overflowing input touches the outputs whose taps
+    read it, as in fp32 arithmetic, and no other."""
+    g = inputs.generator(4)
+    x = torch.randn(2, 3, 24, 24, generator=g)
+    x[0, 1, 7, 9] = value
+    x = x.to(torch.bfloat16)
+    w = inputs.he_normal(16, 3, 7, 7, g)
+    y = _run(x, w, (2, 2), (3, 3))
+    ref = torch.nn.functional.conv2d(x.double(), w.double(), stride=2, padding=3)
+    ref = ref.float().to(torch.bfloat16).float().numpy()   # fp32 range, then bf16
+    fin = np.isfinite(ref)
+    assert np.array_equal(np.isnan(y), np.isnan(ref))
+    assert np.array_equal(y[~fin & ~np.isnan(ref)], ref[~fin & ~np.isnan(ref)])
+    assert np.all(np.abs(y[fin] - ref[fin]) <= 2.0 ** -6 * np.abs(ref[fin]) + 1e-4)
