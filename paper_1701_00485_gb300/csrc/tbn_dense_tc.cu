@@ -31,8 +31,17 @@
 // A tile is 128 consecutive pixels of an image's output map; its input rows
 // arrive by one TMA box, zero-filled outside the image.
 //
-// Bound: the MMAs, 96 cycles per 16 codes (11 steps for 7x7 over 3 channels:
-// 1056 cycles per tile; shared memory is read for 528 + 336 of them).
+// Bound and measured (7x7/2 over 3 x 224 x 224, batch 128): 83 us, where the
+// CUDA-core kernel takes 871.  The MMAs need 96 cycles per 16 codes, 1056 per
+// tile (46 us; shared memory is read for 528 + 336 of those cycles, the output
+// write is 30 us of memory time), a tile takes about 1650.  What is left is
+// the roles' serial instruction paths: with some 20 warps on an SM a warp
+// issues about one instruction in ten cycles, so a hundred of them per block
+// or tile is a thousand cycles.  That is why the coordinates are divided by
+// multiplication, the chunk offsets come from a table, three groups of
+// builders take turns (two: 103 us), the three terms are added two filters at
+// a time, and the MMA warp issues a block as one predicated statement
+// (before all that: 120 us).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -54,7 +63,8 @@ constexpr int kSlotCols = 32;
 constexpr int kRingCol = 2 * kCols;       // accumulators [0, 192) and [192, 384)
 constexpr int kTmemAll = 512;
 constexpr int kPatches = 3;               // input patches in flight
-constexpr int kBuildWarps = 8;            // two groups of four (128 lanes) take blocks in turn
+constexpr int kBuildGroups = 3;           // groups of four warps (128 lanes) take blocks in turn
+constexpr int kBuildWarps = 4 * kBuildGroups;
 constexpr int kEpWarps = 8;               // two groups of four, 32 filters each
 constexpr int kTmaWarp = kBuildWarps + kEpWarps;
 constexpr int kMmaWarp = kTmaWarp + 1;
@@ -67,6 +77,7 @@ constexpr uint64_t kLimitNs = 1000000000ull;
 static_assert(kRingCol + kSlots * kSlotCols <= kTmemAll, "tensor memory");
 
 struct Args {
+  FastDiv by_img, by_q;   // tiles_img, Q
   int C, H, W, K, R, S, sh, sw, ph, pw, Q, PQ;
   int tiles_img, tiles;   // tiles per image, in all
   int nch, blocks;        // (channel, row) chunks of 8 codes; 64-code blocks
@@ -81,7 +92,10 @@ struct Args {
   uint32_t* err;
 };
 
-struct Ctl {
+struct alignas(16) Ctl {
+  // byte offsets in the patch of each (channel, row) chunk; those past the
+  // last repeat it (their weights are zero)
+  int chunk_off[8 * kMaxBlocks];
   uint64_t pfull[kPatches], pempty[kPatches];
   uint64_t full[kSlots], empty[kSlots];
   uint64_t dfull[2], dempty[2];
@@ -99,6 +113,22 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&v)
         "=r"(v[14]), "=r"(v[15])
       : "r"(taddr)
       : "memory");
+}
+
+// Two fp32 additions / multiply-adds in one instruction, each rounded as by
+// itself.
+__device__ __forceinline__ uint64_t f32x2(uint32_t lo, uint32_t hi) {
+  return static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
 // One output tap by tap, for results that are not finite.
@@ -138,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&ctl->pempty[i], 32 * kBuildWarps);
     }
     for (int i = 0; i < kSlots; ++i) {
-      mbar_init(&ctl->full[i], 32 * kBuildWarps / 2);
+      mbar_init(&ctl->full[i], kPix);
       mbar_init(&ctl->empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -154,6 +184,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == kMmaWarp) {
     tmem_alloc(&ctl->tmem_base, kTmemAll);
     tmem_relinquish();
+  }
+  for (int i = threadIdx.x; i < 8 * a.blocks; i += kThreads) {
+    const int ch = min(i, a.nch - 1), c = ch / a.R;
+    ctl->chunk_off[i] = 2 * (c * a.pplane_elems + (ch - c * a.R) * a.prow_elems);
   }
   // the weights' three terms: row f + 64 t of block b holds term t of filter
   // k0 + f, codes [64 b, + 64): chunk of 8 per (channel, row), tap s at
@@ -207,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       ok = mbar_wait(&ctl->pempty[b], (static_cast<uint32_t>(i / kPatches) & 1u) ^ 1u, abort_flag,
                      a.err, kLimitNs);
       if (!__all_sync(0xffffffffu, ok)) break;
-      const int n = t / a.tiles_img, p0 = ((t - n * a.tiles_img) * kPix) / a.Q;
+      const int n = a.by_img(t), p0 = a.by_q((t - n * a.tiles_img) * kPix);
       if (elect_one()) {
         mbar_arrive_expect_tx(&ctl->pfull[b], static_cast<uint32_t>(a.box_bytes));
         tma_load_4d(patch_s + b * a.patch_bytes, &tmap_x, &ctl->pfull[b], -8,
@@ -222,34 +256,27 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == kMmaWarp) {
     // ---------------- MMA issue
     const uint32_t idesc = idesc_bf16_f32(kPix, kCols);
-    int g = 0, issued = 0;
-    uint32_t i = 0;
+    const uint64_t wdesc = smem_desc_sw128_kmajor(smem_addr(w_s));
+    int issued = 0;
+    uint32_t i = 0, sl = 0, ph = 0;   // ring slot and the parity of its fill
     bool ok = true;
     for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++i) {
       const uint32_t db = i & 1u;
-      ok = mbar_wait(&ctl->dempty[db], ((i >> 1) & 1u) ^ 1u, abort_flag, a.err, kLimitNs);
-      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      tc_fence_after_sync();
-      for (int b = 0; b < a.blocks; ++b, ++g) {
-        const int sl = g % kSlots;
-        ok = mbar_wait(&ctl->full[sl], static_cast<uint32_t>(g / kSlots) & 1u, abort_flag, a.err,
-                       kLimitNs);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      ok = mbar_wait_warp(&ctl->dempty[db], ((i >> 1) & 1u) ^ 1u, abort_flag, a.err, kLimitNs);
+      if (!ok) break;
+      for (int b = 0; b < a.blocks; ++b) {
+        ok = mbar_wait_warp(&ctl->full[sl], ph, abort_flag, a.err, kLimitNs);
+        if (!ok) break;
         tc_fence_after_sync();
-        const int steps = min(4, (a.nch - 8 * b + 1) / 2);
-        if (elect_one()) {
-          const uint64_t bdesc = smem_desc_sw128_kmajor(smem_addr(w_s + b * kWBlockBytes));
-          for (int kk = 0; kk < steps; ++kk)
-            tc_mma_ts(db * kCols, static_cast<uint32_t>(kRingCol + sl * kSlotCols + 8 * kk),
-                      bdesc + static_cast<uint64_t>(2 * kk), idesc, (b | kk) != 0 ? 1u : 0u);
-          tc_commit(&ctl->empty[sl]);
-        }
-        __syncwarp();
+        tc_mma_ts_block<2, 4, 6>(db * kCols, kRingCol + sl * kSlotCols,
+                        wdesc + static_cast<uint64_t>(b * (kWBlockBytes >> 4)), idesc,
+                        b != 0 ? 1u : 0u, (a.nch - 8 * b + 1) / 2, &ctl->empty[sl],
+                        b == a.blocks - 1 ? &ctl->dfull[db] : nullptr);
         ++issued;
-      }
-      if (ok) {
-        if (elect_one()) tc_commit(&ctl->dfull[db]);
-        __syncwarp();
+        if (++sl == kSlots) {
+          sl = 0;
+          ph ^= 1u;
+        }
       }
     }
     if (!ok && issued > 0) {
@@ -259,55 +286,48 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_wait(&ctl->drain, 0u, nullptr, a.err, kLimitNs);
     }
   } else if (warp < kBuildWarps) {
-    // ---------------- A rows: this thread's pixel, blocks g % 2 == group
+    // ---------------- A rows: this thread's pixel, blocks g % kBuildGroups == group
     const int group = warp >> 2, px = (warp & 3) * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    const int row_b = a.prow_elems * 2, plane_b = a.pplane_elems * 2;
-    int g = 0;
-    uint32_t i = 0;
+    const int row_b = a.prow_elems * 2;
+    const int col0 = 2 * (8 - a.pw - a.lead);
+    uint32_t g = static_cast<uint32_t>(group), pb = 0, pph = 0;
+    int b = group;   // this group's next block within the tile
     bool ok = true;
-    for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++i) {
-      const int pb = static_cast<int>(i % kPatches);
-      ok = mbar_wait(&ctl->pfull[pb], (i / kPatches) & 1u, abort_flag, a.err, kLimitNs);
+    for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+      ok = mbar_wait(&ctl->pfull[pb], pph, abort_flag, a.err, kLimitNs);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      const int f0 = (t % a.tiles_img) * kPix;
+      const int f0 = (t - a.by_img(t) * a.tiles_img) * kPix;
       const int pix = min(f0 + px, a.PQ - 1);   // pixels past the map repeat its last one
-      const int p = pix / a.Q, q = pix - p * a.Q;
+      const int p = a.by_q(pix), q = pix - p * a.Q;
       const uint32_t base = smem_addr(patch_s + pb * a.patch_bytes) +
-                            static_cast<uint32_t>((p - f0 / a.Q) * a.sh * row_b +
-                                                  2 * (q * a.sw + 8 - a.pw - a.lead));
-      for (int b = 0; b < a.blocks; ++b, ++g) {
-        if ((g & 1) != group) continue;
+                            static_cast<uint32_t>((p - a.by_q(f0)) * a.sh * row_b +
+                                                  2 * q * a.sw + col0);
+      for (; b < a.blocks; b += kBuildGroups, g += kBuildGroups) {
+        int off[8];
+        *reinterpret_cast<int4*>(off) = *reinterpret_cast<const int4*>(&ctl->chunk_off[8 * b]);
+        *reinterpret_cast<int4*>(off + 4) = *reinterpret_cast<const int4*>(&ctl->chunk_off[8 * b + 4]);
         uint32_t v[32];
-        int c = (8 * b) / a.R, r = 8 * b - c * a.R;
-        uint32_t addr = base + static_cast<uint32_t>(c * plane_b + r * row_b);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const bool in = 8 * b + j < a.nch;
+        for (int j = 0; j < 8; ++j)
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            v[4 * j + u] = 0u;
-            if (in)
-              asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v[4 * j + u]) : "r"(addr + 4 * u));
-          }
-          if (++r == a.R) {
-            r = 0;
-            addr += static_cast<uint32_t>(plane_b - (a.R - 1) * row_b);
-          } else {
-            addr += static_cast<uint32_t>(row_b);
-          }
-        }
-        const int sl = g % kSlots;
-        ok = mbar_wait(&ctl->empty[sl], (static_cast<uint32_t>(g / kSlots) & 1u) ^ 1u, abort_flag,
-                       a.err, kLimitNs);
+          for (int u = 0; u < 4; ++u)
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v[4 * j + u]) : "r"(base + off[j] + 4 * u));
+        const uint32_t sl = g % kSlots;
+        ok = mbar_wait(&ctl->empty[sl], ((g / kSlots) & 1u) ^ 1u, abort_flag, a.err, kLimitNs);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         tc_fence_after_sync();
-        tmem_st_32x32b_x32(lane_off + static_cast<uint32_t>(kRingCol + sl * kSlotCols), v);
+        tmem_st_32x32b_x32(lane_off + kRingCol + sl * kSlotCols, v);
         tmem_wait_st();
         tc_fence_before_sync();
         mbar_arrive(&ctl->full[sl]);
       }
+      b -= a.blocks;
       if (ok) mbar_arrive(&ctl->pempty[pb]);
+      if (++pb == kPatches) {
+        pb = 0;
+        pph ^= 1u;
+      }
     }
   } else {
     // ---------------- epilogue: this thread's pixel, filters [32 half, + 32)
@@ -326,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       named_barrier_sync(1, 32 * kEpWarps);
       if (ok) ok = mbar_wait(&ctl->dfull[db], (i >> 1) & 1u, abort_flag, a.err, kLimitNs);
       ok = __all_sync(0xffffffffu, ok);
-      const int n = t / a.tiles_img, f0 = (t - n * a.tiles_img) * kPix;
+      const int n = a.by_img(t), f0 = (t - n * a.tiles_img) * kPix;
       if (ok) {
         tc_fence_after_sync();
 #pragma unroll
@@ -341,28 +361,39 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_before_sync();
             mbar_arrive(&ctl->dempty[db]);
           }
-          float o[16];
-          bool finite = true;
+          // (l + m) + h; zero times the results sums to zero unless one of
+          // them is infinite or NaN
+          uint64_t o2[8], zero = 0;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            o[j] = (__uint_as_float(vl[j]) + __uint_as_float(vm[j])) + __uint_as_float(vh[j]);
-            finite = finite && fabsf(o[j]) <= 3.402823466e38f;
+          for (int j = 0; j < 8; ++j) {
+            o2[j] = add_f32x2(add_f32x2(f32x2(vl[2 * j], vl[2 * j + 1]),
+                                        f32x2(vm[2 * j], vm[2 * j + 1])),
+                              f32x2(vh[2 * j], vh[2 * j + 1]));
+            zero = fma_f32x2(o2[j], 0ull, zero);
           }
-          if (!finite && f0 + row < a.PQ) {
+          float o[16];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            o[2 * j] = __uint_as_float(static_cast<uint32_t>(o2[j]));
+            o[2 * j + 1] = __uint_as_float(static_cast<uint32_t>(o2[j] >> 32));
+          }
+          const float z = __uint_as_float(static_cast<uint32_t>(zero)) +
+                          __uint_as_float(static_cast<uint32_t>(zero >> 32));
+          if (z != 0.0f && f0 + row < a.PQ) {   // NaN != 0
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int k = k0 + 32 * half + 16 * cc + j;
-              if (k < a.K && !(fabsf(o[j]) <= 3.402823466e38f))
+              if (k < a.K && !(fabsf(o[j]) <= 3.402823466e38f)) {
                 o[j] = dense_by_taps(a, n, k, f0 + row);
+                if (a.relu) o[j] = fmaxf(o[j], 0.0f);   // NaN gives 0 there too
+              }
             }
           }
           uint32_t pk[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float y0 = a.relu ? fmaxf(o[2 * j], 0.0f) : o[2 * j];
-            const float y1 = a.relu ? fmaxf(o[2 * j + 1], 0.0f) : o[2 * j + 1];
-            pk[j] = pack_bf16x2(y0, y1);
-          }
+          for (int j = 0; j < 8; ++j)
+            pk[j] = a.relu ? pack_bf16x2_relu(o[2 * j], o[2 * j + 1])
+                           : pack_bf16x2(o[2 * j], o[2 * j + 1]);
 #pragma unroll
           for (int u = 0; u < 2; ++u)
             *reinterpret_cast<uint4*>(stage + row * 128 +
@@ -406,6 +437,8 @@ bool plan(const ConvProblem& p, Args* out, size_t* smem) {
   a.sh = (int)p.sh; a.sw = (int)p.sw; a.ph = (int)p.ph; a.pw = (int)p.pw;
   a.Q = (int)p.Q; a.PQ = (int)(p.P * p.Q);
   a.tiles_img = (a.PQ + kPix - 1) / kPix;
+  a.by_img = fast_div(a.tiles_img);
+  a.by_q = fast_div(a.Q);
   if (p.N * a.tiles_img > 0x7fffffffLL) return false;
   a.tiles = (int)(p.N * a.tiles_img);
   a.nch = (int)(p.C * p.R);

@@ -47,6 +47,26 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// Division by a launch constant as one multiplication: exact for 0 <= n < 2^31
+// (with 2^(s-1) < d <= 2^s and m = floor(2^(31+s) / d) + 1, m d - 2^(31+s) is
+// in (0, d], and n times it stays below 2^(31+s)).  A runtime integer division
+// is some 35 dependent instructions, about 350 cycles on a busy SM, and every
+// role needs several per tile.
+struct FastDiv {
+  uint32_t m;
+  int shift;
+  __device__ __forceinline__ int operator()(int n) const {
+    return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(n)) * m) >> shift);
+  }
+};
+
+inline FastDiv fast_div(int d) {
+  int s = 0;
+  while ((int64_t(1) << s) < d) ++s;
+  return FastDiv{static_cast<uint32_t>((uint64_t(1) << (31 + s)) / static_cast<uint64_t>(d) + 1),
+                 31 + s};
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count)
@@ -135,6 +155,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
       }
     }
   }
+}
+
+// mbar_wait by a whole converged warp, with one warp-uniform answer: a wait
+// that has already ended costs one poll and one vote.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
+                                               volatile int* abort, uint32_t* err,
+                                               uint64_t limit_ns) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, limit_ns));
 }
 
 // Named barrier over `nthreads` threads (a multiple of 32) of the CTA.
@@ -289,6 +318,37 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// One 64-code block by a whole converged warp: min(steps, 4) MMAs of 16 codes
+// (A 8 columns apart in tensor memory; B at b_desc and, in its 16-byte units,
+// kB1, kB2, kB3 beyond), then a commit to `done` and, if not null, to `done2`, all from one
+// elected lane.  Predicated in one statement instead of a branch around
+// five: the issuing warp's instructions per block are what paces the kernels
+// whose other warps load its scheduler.
+template <uint32_t kB1, uint32_t kB2, uint32_t kB3>
+__device__ __forceinline__ void tc_mma_ts_block(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                                uint32_t idesc, uint32_t accumulate, int steps,
+                                                uint64_t* done, uint64_t* done2) {
+  asm volatile(
+      "{\n\t.reg .pred e, e1, e2, e3, ec, p, t;\n\t"
+      ".reg .b32 a1, a2, a3;\n\t.reg .b64 b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "setp.gt.and.s32 e1, %5, 1, e;\n\tsetp.gt.and.s32 e2, %5, 2, e;\n\t"
+      "setp.gt.and.s32 e3, %5, 3, e;\n\tsetp.ne.and.b32 ec, %7, 0, e;\n\t"
+      "add.u32 a1, %1, 8;\n\tadd.u32 a2, %1, 16;\n\tadd.u32 a3, %1, 24;\n\t"
+      "add.u64 b1, %2, %8;\n\tadd.u64 b2, %2, %9;\n\tadd.u64 b3, %2, %10;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t"
+      "@e1 tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, t;\n\t"
+      "@e2 tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, t;\n\t"
+      "@e3 tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, t;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%6];\n\t"
+      "@ec tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n\t}" ::"r"(
+          d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(steps), "r"(smem_addr(done)),
+      "r"(done2 != nullptr ? smem_addr(done2) : 0u), "n"(kB1), "n"(kB2), "n"(kB3)
       : "memory");
 }
 
