@@ -181,6 +181,12 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   a.base_tiles = static_cast<int>(tiles);
   a.tiles = static_cast<int>(tiles * a.ksplit);
   a.partial = split ? p.partial : nullptr;
+  a.by_base = fast_div(a.base_tiles);
+  a.by_k = fast_div(a.tiles_k);
+  a.by_tq = fast_div(a.tiles_q);
+  a.by_tp = fast_div(a.tiles_p);
+  a.by_iq = fast_div(a.iQ);
+  a.by_ip = fast_div(a.iP);
   a.wpf = (a.ncodes + 15) / 16;
   if (s2d) {
     // codes of the original (r, s, c) filter

@@ -111,6 +111,8 @@ struct IgArgs {
   // batch as one row of N P Q pixels, or as one image of N P rows when
   // pooling); an image's output is iP x iQ
   int im2col, iP, iQ;
+  // divisors of the tile and pixel coordinates
+  FastDiv by_base, by_k, by_tq, by_tp, by_iq, by_ip;
   // patch mode: the patch is rows [p0 sh - ph, + PR) x columns [-pw, W + pw)
   int PR, PW;              // patch rows, patch columns (W + 2 pw)
   int patch_cap;           // bytes per patch buffer (multiple of 16)
@@ -250,15 +252,16 @@ struct TileCoord {
 
 __device__ __forceinline__ TileCoord tile_coord(const IgArgs& a, int t) {
   TileCoord c;
-  c.split = t / a.base_tiles;
+  c.split = a.by_base(t);
   t -= c.split * a.base_tiles;
   c.kb0 = c.split * a.kb_per;
   c.kb1 = min(a.kblocks, c.kb0 + a.kb_per);
-  c.ktile = t % a.tiles_k;
-  const int pt_lin = t / a.tiles_k;
-  const int qt = pt_lin % a.tiles_q;
-  const int pt = (pt_lin / a.tiles_q) % a.tiles_p;
-  const int nt = pt_lin / (a.tiles_q * a.tiles_p);
+  const int pt_lin = a.by_k(t);
+  c.ktile = t - pt_lin * a.tiles_k;
+  const int np = a.by_tq(pt_lin);
+  const int qt = pt_lin - np * a.tiles_q;
+  const int nt = a.by_tp(np);
+  const int pt = np - nt * a.tiles_p;
   c.q0 = qt * a.bw;
   c.p0 = pt * a.bh;
   c.n0 = nt * a.bn;
@@ -511,6 +514,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     const uint32_t box_bytes = static_cast<uint32_t>(a.bw * a.bh * a.bn * kBoxCh * 2);
     const int cblocks = a.C / kBoxCh;                // boxes per tap
     int g = 0;  // global K-block counter of this CTA
+    int st = 0;          // its ring stage
+    uint32_t par = 0;    // and the parity of the stage's fill
     bool ok = true;
     for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
       const TileCoord tc = tile_coord(a, t);
@@ -518,49 +523,63 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       int w0 = tc.q0 * a.sw - a.pw, h0 = tc.p0 * a.sh - a.ph, n0 = tc.n0;
       if (a.im2col) {
         const int f = tc.p0 * a.Q + tc.q0;
-        const int row = f / a.iQ;
-        n0 = row / a.iP;
+        const int row = a.by_iq(f);
+        n0 = a.by_ip(row);
         w0 = (f - row * a.iQ) * a.sw - a.pw;
         h0 = (row - n0 * a.iP) * a.sh - a.ph;
       }
-      // (tap, channel box) of the next box
-      int tap = (tc.kb0 * kBoxes) / cblocks, cb = (tc.kb0 * kBoxes) % cblocks;
+      // (filter row, filter column, channel box) of the next box
+      const int tap0 = (tc.kb0 * kBoxes) / cblocks;
+      int cb = tc.kb0 * kBoxes - tap0 * cblocks, r = tap0 / a.S, q = tap0 - r * a.S;
+      const auto next_box = [&]() {
+        if (++cb == cblocks) {
+          cb = 0;
+          if (++q == a.S) {
+            q = 0;
+            ++r;
+          }
+        }
+      };
       for (int kb = tc.kb0; kb < tc.kb1; ++kb, ++g) {
+        const int sb = st;
+        const uint32_t ph = par;
+        if (++st == kSt) {
+          st = 0;
+          par ^= 1u;
+        }
         const bool mine = turn == pid;
         if (++turn == kTmaProducers) turn = 0;
-        if (!mine) {
+        if (mine) {
+          ok = mbar_wait_warp(&ctl->empty[sb], ph ^ 1u, abort_flag, a.err, kWaitLimitNs);
+          if (!ok) break;
+          if (elect_one()) {
+            mbar_arrive_expect_tx(&ctl->full[sb], box_bytes * kBoxes);
+            int cb_ = cb, r_ = r, q_ = q;
 #pragma unroll
-          for (int bx = 0; bx < kBoxes; ++bx)
-            if (++cb == cblocks) { cb = 0; ++tap; }
-          continue;
-        }
-        const int sb = g % kSt;
-        const uint32_t it = static_cast<uint32_t>(g / kSt);
-        ok = mbar_wait(&ctl->empty[sb], (it & 1u) ^ 1u, abort_flag, a.err, kWaitLimitNs);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-        if (elect_one()) {
-          mbar_arrive_expect_tx(&ctl->full[sb], box_bytes * kBoxes);
-#pragma unroll
-          for (int bx = 0; bx < kBoxes; ++bx) {
-            // a box past the filter's last tap is requested at channel C:
-            // entirely out of range, it arrives zero-filled
-            const bool past = tap >= a.R * a.S;
-            const int tp = past ? 0 : tap;
-            const int r = tp / a.S, s = tp - r * a.S;
-            uint8_t* dst = ring + sb * kStageBytes + bx * (kStageBytes / kBoxes);
-            const int c0 = past ? a.C : cb * kBoxCh;
-            if (a.im2col)
-              tma_load_im2col_4d(dst, &tmap_x, &ctl->full[sb], c0, w0, h0, n0, s, r);
-            else
-              tma_load_4d(dst, &tmap_x, &ctl->full[sb], c0, w0 + s, h0 + r, n0);
-            if (++cb == cblocks) { cb = 0; ++tap; }
+            for (int bx = 0; bx < kBoxes; ++bx) {
+              // a box past the filter's last tap is requested at channel C:
+              // entirely out of range, it arrives zero-filled
+              const bool past = r_ >= a.R;
+              uint8_t* dst = ring + sb * kStageBytes + bx * (kStageBytes / kBoxes);
+              const int c0 = past ? a.C : cb_ * kBoxCh;
+              const int dr = past ? 0 : r_, dq = past ? 0 : q_;
+              if (a.im2col)
+                tma_load_im2col_4d(dst, &tmap_x, &ctl->full[sb], c0, w0, h0, n0, dq, dr);
+              else
+                tma_load_4d(dst, &tmap_x, &ctl->full[sb], c0, w0 + dq, h0 + dr, n0);
+              if (++cb_ == cblocks) {
+                cb_ = 0;
+                if (++q_ == a.S) {
+                  q_ = 0;
+                  ++r_;
+                }
+              }
+            }
           }
-        } else {
-#pragma unroll
-          for (int bx = 0; bx < kBoxes; ++bx)
-            if (++cb == cblocks) { cb = 0; ++tap; }
+          __syncwarp();
         }
-        __syncwarp();
+#pragma unroll
+        for (int bx = 0; bx < kBoxes; ++bx) next_box();
       }
     }
     // drain: every copy this warp issued must land before the CTA may exit
@@ -876,8 +895,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
   } else if (warp == 1) {
     // ================= MMA issuer =================
     const uint32_t idesc = idesc_bf16_f32(kBM, static_cast<uint32_t>(a.tile_n));
-    int g = 0, issued = 0;
-    uint32_t tiles_done = 0;
+    int issued = 0, st = 0;
+    uint32_t tiles_done = 0, par = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++tiles_done) {
       const TileCoord tc = tile_coord(a, t);
@@ -885,47 +904,30 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const uint32_t ab = a.acc2 ? (tiles_done & 1u) : 0u;
       const uint32_t use = a.acc2 ? (tiles_done >> 1) : tiles_done;   // uses of accumulator ab
       const uint32_t acc_t = acc_tmem + ab * kAcc2Cols;
-      ok = mbar_wait(&ctl->acc_empty[ab], (use & 1u) ^ 1u, abort_flag, a.err, kWaitLimitNs);
-      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      tc_fence_after_sync();
-      for (int kb = tc.kb0; kb < tc.kb1; ++kb, ++g) {
-        const int st = g % kSt;
-        ok = mbar_wait(&ctl->full[st], static_cast<uint32_t>(g / kSt) & 1u, abort_flag, a.err,
-                       kWaitLimitNs);
+      ok = mbar_wait_warp(&ctl->acc_empty[ab], (use & 1u) ^ 1u, abort_flag, a.err, kWaitLimitNs);
+      if (!ok) break;
+      for (int kb = tc.kb0; kb < tc.kb1; ++kb) {
+        ok = mbar_wait_warp(&ctl->full[st], par, abort_flag, a.err, kWaitLimitNs);
         if (kS2d && tiles_done == 0 && ok)   // first use of a resident K block
-          ok = mbar_wait(&ctl->wready[kb], 0u, abort_flag, a.err, kWaitLimitNs);
-        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+          ok = mbar_wait_warp(&ctl->wready[kb], 0u, abort_flag, a.err, kWaitLimitNs);
+        if (!ok) break;
         tc_fence_after_sync();
         const uint32_t a_col =
             kS2d ? static_cast<uint32_t>(kTmemCols - 32 * KB + 32 * kb)
                  : a_tmem0 + static_cast<uint32_t>(st * kAColsPerStage);
-        if (elect_one()) {
-          if constexpr (kCh32) {
-            // two halves of 32 codes, 64-byte rows with the 64-byte swizzle
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              const uint64_t bdesc = smem_desc_sw64_kmajor(
-                  smem_addr(ring + st * kStageBytes + (kk >> 1) * (kStageBytes / 2)));
-              tc_mma_ts(acc_t, a_col + 8u * kk, bdesc + static_cast<uint64_t>(2 * (kk & 1)),
-                        idesc, ((kb - tc.kb0) | kk) != 0 ? 1u : 0u);
-            }
-          } else {
-            const uint64_t bdesc = smem_desc_sw128_kmajor(smem_addr(ring + st * kStageBytes));
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              // K step kk: 16 codes = 8 TMEM columns of A, 32 bytes of B rows
-              tc_mma_ts(acc_t, a_col + 8u * kk, bdesc + static_cast<uint64_t>(2 * kk), idesc,
-                        ((kb - tc.kb0) | kk) != 0 ? 1u : 0u);
-            }
-          }
-          tc_commit(&ctl->empty[st]);
-        }
-        __syncwarp();
+        // K step kk: 16 codes = 8 TMEM columns of A, 32 bytes of B rows (two
+        // halves of 32 codes, 64-byte rows, with 32-channel boxes)
+        const uint32_t b_addr = smem_addr(ring) + static_cast<uint32_t>(st * kStageBytes);
+        constexpr uint32_t kHalf = kCh32 ? (kStageBytes / 2) >> 4 : 4u;
+        tc_mma_ts_block<2, kHalf, kHalf + 2>(
+            acc_t, a_col, kCh32 ? smem_desc_sw64_kmajor(b_addr) : smem_desc_sw128_kmajor(b_addr),
+            idesc, kb != tc.kb0 ? 1u : 0u, 4, &ctl->empty[st],
+            kb == tc.kb1 - 1 ? &ctl->acc_full[ab] : nullptr);
         ++issued;
-      }
-      if (ok) {
-        if (elect_one()) tc_commit(&ctl->acc_full[ab]);
-        __syncwarp();
+        if (++st == kSt) {
+          st = 0;
+          par ^= 1u;
+        }
       }
     }
     if (!ok && issued > 0) {
@@ -968,39 +970,49 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       }
     } else {
     const bool pair_ok = ((a.wpf & 1) == 0) && ((reinterpret_cast<uintptr_t>(a.codes) & 7) == 0);
-    // this CTA's K blocks, all tiles in sequence (g = tile_index * KB + kb)
-    int total = 0;   // K blocks of all this CTA's tiles
-    for (int t = blockIdx.x; t < a.tiles; t += gridDim.x) {
-      const TileCoord tc = tile_coord(a, t);
-      total += tc.kb1 - tc.kb0;
+    // this CTA's K blocks, all tiles in sequence
+    int total = 0;
+    if (a.ksplit == 1) {
+      total = (a.tiles - static_cast<int>(blockIdx.x) + static_cast<int>(gridDim.x) - 1) /
+              static_cast<int>(gridDim.x) * KB;
+    } else {
+      for (int t = blockIdx.x; t < a.tiles; t += gridDim.x) {
+        const TileCoord tc = tile_coord(a, t);
+        total += tc.kb1 - tc.kb0;
+      }
     }
     // prefetch cursor over (tile, kb): the codes of K block kb of a filter
-    // are words [4 kb, 4 kb + 4) of its row; this warp takes two of them
-    int t_ld = blockIdx.x, kb_ld = 0, kb_end = 0;
-    const uint32_t* crow_ld = nullptr;
+    // are words [4 kb, 4 kb + 4) of its row; this warp takes two of them,
+    // where the row has them (kb < kb_lim)
+    int t_ld = blockIdx.x, kb_ld = 0, kb_end = 0, kb_lim = 0;
+    const int kb_words = (a.wpf - 2 * half + 3) / 4;   // K blocks whose two words begin in the row
+    const uint32_t* cp = a.codes;
     auto set_row = [&]() {
       const TileCoord tc = tile_coord(a, t_ld < a.tiles ? t_ld : 0);
       kb_ld = tc.kb0;
       kb_end = tc.kb1;
       const int k = tc.ktile * kBM + m;
-      crow_ld = (t_ld < a.tiles && k < a.K) ? a.codes + static_cast<size_t>(k) * a.wpf : nullptr;
+      const bool in = t_ld < a.tiles && k < a.K;
+      kb_lim = in ? kb_words : 0;
+      cp = a.codes + static_cast<size_t>(in ? k : 0) * a.wpf + 4 * kb_ld + 2 * half;
     };
     set_row();
     auto next_codes = [&]() -> uint2 {
       uint2 r = make_uint2(0u, 0u);
-      const int w0 = kb_ld * 4 + half * 2;
-      if (crow_ld != nullptr && w0 < a.wpf) {
+      if (kb_ld < kb_lim) {
         // written by this launch's prologue when fused: ordinary (L1-cached,
         // coherent) loads after the grid barrier's acquire then, not the
         // read-only path, which assumes data constant for the whole launch
+        const bool two = 4 * kb_ld + 2 * half + 1 < a.wpf;
         if constexpr (kFuse) {
-          if (pair_ok) r = __ldca(reinterpret_cast<const uint2*>(crow_ld + w0));
-          else r = make_uint2(__ldca(crow_ld + w0), w0 + 1 < a.wpf ? __ldca(crow_ld + w0 + 1) : 0u);
+          if (pair_ok) r = __ldca(reinterpret_cast<const uint2*>(cp));
+          else r = make_uint2(__ldca(cp), two ? __ldca(cp + 1) : 0u);
         } else {
-          if (pair_ok) r = __ldg(reinterpret_cast<const uint2*>(crow_ld + w0));
-          else r = make_uint2(__ldg(crow_ld + w0), w0 + 1 < a.wpf ? __ldg(crow_ld + w0 + 1) : 0u);
+          if (pair_ok) r = __ldg(reinterpret_cast<const uint2*>(cp));
+          else r = make_uint2(__ldg(cp), two ? __ldg(cp + 1) : 0u);
         }
       }
+      cp += 4;
       if (++kb_ld == kb_end) {
         t_ld += gridDim.x;
         set_row();
@@ -1012,6 +1024,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     const uint32_t col = a_tmem0 + lane_off + static_cast<uint32_t>(16 * half);
     // two K blocks per iteration: their tensor-memory stores share one
     // tcgen05.wait::st
+    int st = 0;         // ring stage of the next K block
+    uint32_t par = 0;   // parity of its fill
     for (int g = 0; g < total; g += 2) {
       const bool two = g + 1 < total;   // warp-uniform
       uint32_t v0[16], v1[16];
@@ -1023,19 +1037,19 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       q1 = q3;
       q2 = next_codes();
       q3 = next_codes();
-      const int s0 = g % kSt, s1 = (g + 1) % kSt;
+      const int s0 = st;
+      const uint32_t p0 = par ^ 1u;
+      if (++st == kSt) { st = 0; par ^= 1u; }
+      const int s1 = st;
+      const uint32_t p1 = par ^ 1u;
+      if (++st == kSt) { st = 0; par ^= 1u; }
       // in patch mode the operand builders are the bottleneck: waiting
       // expanders park instead of spinning, leaving the issue slots to them
-      bool ok = kPatch ? mbar_wait_sleep(&ctl->empty[s0], (static_cast<uint32_t>(g / kSt) & 1u) ^ 1u,
-                                         abort_flag, a.err, kWaitLimitNs)
-                       : mbar_wait(&ctl->empty[s0], (static_cast<uint32_t>(g / kSt) & 1u) ^ 1u,
-                                   abort_flag, a.err, kWaitLimitNs);
+      bool ok = kPatch ? mbar_wait_sleep(&ctl->empty[s0], p0, abort_flag, a.err, kWaitLimitNs)
+                       : mbar_wait(&ctl->empty[s0], p0, abort_flag, a.err, kWaitLimitNs);
       if (ok && two)
-        ok = kPatch ? mbar_wait_sleep(&ctl->empty[s1],
-                                      (static_cast<uint32_t>((g + 1) / kSt) & 1u) ^ 1u, abort_flag,
-                                      a.err, kWaitLimitNs)
-                    : mbar_wait(&ctl->empty[s1], (static_cast<uint32_t>((g + 1) / kSt) & 1u) ^ 1u,
-                                abort_flag, a.err, kWaitLimitNs);
+        ok = kPatch ? mbar_wait_sleep(&ctl->empty[s1], p1, abort_flag, a.err, kWaitLimitNs)
+                    : mbar_wait(&ctl->empty[s1], p1, abort_flag, a.err, kWaitLimitNs);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after_sync();
       tmem_st_32x32b_x16(col + static_cast<uint32_t>(s0 * kAColsPerStage), v0);
