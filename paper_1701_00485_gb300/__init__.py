@@ -15,6 +15,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 import torch
@@ -152,10 +153,26 @@ def lib():
             fn = getattr(L, name)
             fn.argtypes = args
             fn.restype = res
+        L.tbn_packed_call.argtypes = [I32, ctypes.c_char_p]
+        L.tbn_packed_call.restype = I32
         if L.tbn_abi_version() != ABI_VERSION:
             raise RuntimeError("libtbn ABI version mismatch")
         _lib = L
         return L
+
+
+# The calls that a program issues once per layer pass their arguments as one
+# block of 64-bit integers (tbn_packed_call, a private export that unpacks
+# them and calls the C entry point of the same name): converting some twenty
+# arguments one by one took ctypes longer than the launch itself.
+_OP_QUANTIZE, _OP_CONV, _OP_LINEAR, _OP_BWD_DATA, _OP_BWD_FILTER = range(5)
+_PACK = {n: struct.Struct("%dq" % n).pack for n in (6, 14, 17, 19, 23)}
+
+
+def _call(op: int, where: str, *args):
+    status = (_lib or lib()).tbn_packed_call(op, _PACK[len(args)](*args))
+    if status != TBN_OK:
+        _check(status, where)
 
 
 def _status_name(s: int) -> str:
@@ -191,9 +208,22 @@ def _cuda(t: torch.Tensor, name: str) -> torch.Tensor:
     return t
 
 
+def _raw_stream(stream) -> int:
+    """The cudaStream_t of `stream`, or of the current device's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_raw_stream is not None:
+        return _current_raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
+# torch's own accessor without the Stream object that current_stream() builds
+# (3 us a call); absent in some builds
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return ctypes.c_void_p(_raw_stream(stream))
 
 
 def _epi(relu: bool, residual, pool: int = 0) -> Epilogue | None:
@@ -205,7 +235,8 @@ def _epi(relu: bool, residual, pool: int = 0) -> Epilogue | None:
 
 def packed_words(n: int) -> int:
     """ceil(n / 16): uint32 words per filter of n two-bit codes."""
-    return int(lib().tbn_packed_words(int(n)))
+    n = int(n)
+    return -1 if n < 1 else (n + 15) // 16
 
 
 def conv_out_hw(H, W, R, S, stride=(1, 1), pad=(0, 0)):
@@ -226,8 +257,8 @@ def tbn_quantize_pack(W: torch.Tensor, codes: torch.Tensor | None = None,
     if alpha is None:
         alpha = torch.empty((K,), dtype=torch.float32, device=W.device)
     _cuda(codes, "codes"), _cuda(alpha, "alpha")
-    _check(lib().tbn_quantize_pack(W.data_ptr(), K, n, codes.data_ptr(), alpha.data_ptr(),
-                                   _stream(stream)), "tbn_quantize_pack")
+    _call(_OP_QUANTIZE, "tbn_quantize_pack", W.data_ptr(), K, n, codes.data_ptr(),
+          alpha.data_ptr(), _raw_stream(stream))
     return codes, alpha
 
 
@@ -292,11 +323,10 @@ def tbn_conv2d_fwd(x: torch.Tensor, codes: torch.Tensor, alpha: torch.Tensor, K:
         _cuda(residual, "residual")
         if tuple(residual.shape) != shape or _dt(residual) != ydt:
             raise ValueError("residual must match y's shape and dtype")
-    e = _epi(relu, residual, pool)
-    _check(lib().tbn_conv2d_fwd_algo(
-        x.data_ptr(), _dt(x), layout, N, C, H, W, codes.data_ptr(), alpha.data_ptr(), K, R, S,
-        stride[0], stride[1], pad[0], pad[1], out.data_ptr(), ydt,
-        ctypes.byref(e) if e is not None else None, algo, _stream(stream)), "tbn_conv2d_fwd")
+    _call(_OP_CONV, "tbn_conv2d_fwd", x.data_ptr(), _dt(x), layout, N, C, H, W, codes.data_ptr(),
+          alpha.data_ptr(), K, R, S, stride[0], stride[1], pad[0], pad[1], out.data_ptr(), ydt,
+          1 if relu else 0, residual.data_ptr() if residual is not None else 0, int(pool), algo,
+          _raw_stream(stream))
     return out
 
 
@@ -389,11 +419,9 @@ def tbn_conv2d_bwd_data(dy: torch.Tensor, codes: torch.Tensor, alpha: torch.Tens
         workspace = torch.empty(max(n, 256), dtype=torch.uint8, device=dy.device)
     ydt = TBN_BF16 if out_dtype in (None, torch.bfloat16) else TBN_F32
     dx = torch.empty((N, H, W, C), dtype=_torch_dt(ydt), device=dy.device)
-    _check(lib().tbn_conv2d_bwd_data(dy.data_ptr(), N, C, H, W, codes.data_ptr(),
-                                     alpha.data_ptr(), K, R, S, stride[0], stride[1], pad[0],
-                                     pad[1], dx.data_ptr(), ydt, workspace.data_ptr(),
-                                     workspace.numel() * workspace.element_size(),
-                                     _stream(stream)), "tbn_conv2d_bwd_data")
+    _call(_OP_BWD_DATA, "tbn_conv2d_bwd_data", dy.data_ptr(), N, C, H, W, codes.data_ptr(),
+          alpha.data_ptr(), K, R, S, stride[0], stride[1], pad[0], pad[1], dx.data_ptr(), ydt,
+          workspace.data_ptr(), workspace.numel() * workspace.element_size(), _raw_stream(stream))
     return dx
 
 
@@ -410,10 +438,9 @@ def tbn_conv2d_bwd_filter(x: torch.Tensor, dy: torch.Tensor, R: int, S: int, str
     if workspace is None:
         workspace = torch.empty(max(n, 256), dtype=torch.uint8, device=x.device)
     dw = torch.empty((K, R * S * C), dtype=torch.float32, device=x.device)
-    _check(lib().tbn_conv2d_bwd_filter(x.data_ptr(), dy.data_ptr(), *shape, dw.data_ptr(),
-                                       workspace.data_ptr(),
-                                       workspace.numel() * workspace.element_size(),
-                                       _stream(stream)), "tbn_conv2d_bwd_filter")
+    _call(_OP_BWD_FILTER, "tbn_conv2d_bwd_filter", x.data_ptr(), dy.data_ptr(), *shape,
+          dw.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
+          _raw_stream(stream))
     return dw
 
 
@@ -432,11 +459,7 @@ def tbn_linear_fwd(x: torch.Tensor, codes: torch.Tensor, alpha: torch.Tensor, K_
     ydt = _dt(x) if out_dtype is None else (TBN_F32 if out_dtype == torch.float32 else TBN_BF16)
     if out is None:
         out = torch.empty((B, K_out), dtype=_torch_dt(ydt), device=x.device)
-    e = _epi(relu, residual)
-    _check(lib().tbn_linear_fwd(x.data_ptr(), _dt(x), B, K_in, codes.data_ptr(), alpha.data_ptr(),
-                                K_out, out.data_ptr(), ydt,
-                                ctypes.byref(e) if e is not None else None, _stream(stream)),
-           "tbn_linear_fwd")
+    _linear("tbn_linear_fwd", x, codes, alpha, K_out, out, ydt, relu, residual, 0, 0, stream)
     return out
 
 
@@ -458,17 +481,21 @@ def tbn_linear_fwd_ws(x: torch.Tensor, codes: torch.Tensor, alpha: torch.Tensor,
     ydt = _dt(x) if out_dtype is None else (TBN_F32 if out_dtype == torch.float32 else TBN_BF16)
     if out is None:
         out = torch.empty((B, K_out), dtype=_torch_dt(ydt), device=x.device)
-    ws_ptr, ws_bytes = None, 0
+    ws_ptr, ws_bytes = 0, 0
     if workspace is not None:
         _cuda(workspace, "workspace")
         ws_ptr, ws_bytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-    e = _epi(relu, residual)
-    _check(lib().tbn_linear_fwd_ws(x.data_ptr(), _dt(x), B, K_in, codes.data_ptr(),
-                                   alpha.data_ptr(), K_out, out.data_ptr(), ydt,
-                                   ctypes.byref(e) if e is not None else None, ws_ptr, ws_bytes,
-                                   _stream(stream)),
-           "tbn_linear_fwd_ws")
+    _linear("tbn_linear_fwd_ws", x, codes, alpha, K_out, out, ydt, relu, residual, ws_ptr,
+            ws_bytes, stream)
     return out
+
+
+def _linear(where, x, codes, alpha, K_out, out, ydt, relu, residual, ws_ptr, ws_bytes, stream):
+    B, K_in = x.shape
+    _call(_OP_LINEAR, where, x.data_ptr(), _dt(x), B, K_in, codes.data_ptr(), alpha.data_ptr(),
+          K_out, out.data_ptr(), ydt, 1 if relu else 0,
+          residual.data_ptr() if residual is not None else 0, ws_ptr, ws_bytes,
+          _raw_stream(stream))
 
 
 def tbn_linear_f8_prepared_words(K_out: int, K_in: int) -> int:

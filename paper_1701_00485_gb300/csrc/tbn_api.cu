@@ -791,3 +791,42 @@ tbn_status tbn_dense_linear_fwd(const float* x, int64_t B, int64_t K_in, const f
 }
 
 }  // extern "C"
+
+// The Python binding's calls with their arguments as one block of 64-bit
+// integers in the order of the C entry point (pointers as integers; an
+// epilogue as its relu, residual and pool).  Not declared in tbn.h: the
+// binding's own, versioned with it.
+extern "C" tbn_status tbn_packed_call(int op, const int64_t* v) {
+  const auto ptr = [&](int i) { return reinterpret_cast<void*>(static_cast<uintptr_t>(v[i])); };
+  const auto f32 = [&](int i) { return static_cast<float*>(ptr(i)); };
+  const auto u32 = [&](int i) { return static_cast<uint32_t*>(ptr(i)); };
+  const auto dt = [&](int i) { return static_cast<tbn_dtype>(v[i]); };
+  if (v == nullptr) return fail(TBN_ERR_INVALID_ARG, "packed call: null arguments");
+  switch (op) {
+    case 0:
+      return tbn_quantize_pack(f32(0), v[1], v[2], u32(3), f32(4), ptr(5));
+    case 1: {
+      const tbn_epilogue e{static_cast<int>(v[18]), ptr(19), static_cast<int>(v[20])};
+      return tbn_conv2d_fwd_algo(ptr(0), dt(1), static_cast<tbn_layout>(v[2]), v[3], v[4], v[5],
+                                 v[6], u32(7), f32(8), v[9], v[10], v[11], v[12], v[13], v[14],
+                                 v[15], ptr(16), dt(17),
+                                 e.relu || e.residual || e.pool ? &e : nullptr,
+                                 static_cast<tbn_conv_algo>(v[21]), ptr(22));
+    }
+    case 2: {
+      const tbn_epilogue e{static_cast<int>(v[9]), ptr(10), 0};
+      return tbn_linear_fwd_ws(ptr(0), dt(1), v[2], v[3], u32(4), f32(5), v[6], ptr(7), dt(8),
+                               e.relu || e.residual ? &e : nullptr, ptr(11),
+                               static_cast<size_t>(v[12]), ptr(13));
+    }
+    case 3:
+      return tbn_conv2d_bwd_data(ptr(0), v[1], v[2], v[3], v[4], u32(5), f32(6), v[7], v[8], v[9],
+                                 v[10], v[11], v[12], v[13], ptr(14), dt(15), ptr(16),
+                                 static_cast<size_t>(v[17]), ptr(18));
+    case 4:
+      return tbn_conv2d_bwd_filter(ptr(0), ptr(1), v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[9],
+                                   v[10], v[11], v[12], f32(13), ptr(14),
+                                   static_cast<size_t>(v[15]), ptr(16));
+  }
+  return fail(TBN_ERR_INVALID_ARG, "packed call: unknown operation %d", op);
+}

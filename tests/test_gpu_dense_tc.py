@@ -76,3 +76,28 @@ def test_dense_tc_not_finite(value):
     assert np.array_equal(np.isnan(y), np.isnan(ref))
     assert np.array_equal(y[~fin & ~np.isnan(ref)], ref[~fin & ~np.isnan(ref)])
     assert np.all(np.abs(y[fin] - ref[fin]) <= 2.0 ** -6 * np.abs(ref[fin]) + 1e-4)
+
+
+@pytest.mark.parametrize("B,K_in,K_out", [(33, 128, 31), (1, 4, 1), (32, 129, 32), (65, 516, 100),
+                                          (31, 252, 1000)])
+def test_dense_linear_tile_edges(B, K_in, K_out):
+    """Rows, columns and input chunks at the edges of their tiles, with
+    vector (K_in % 4 == 0) and scalar loads.  fp32 sums: K_in 2^-24 sum|x w|."""
+    g = inputs.generator(B * K_in)
+    x = torch.randn(B, K_in, generator=g)
+    w = torch.randn(K_out, K_in, generator=g)
+    y = tbn.tbn_dense_linear_fwd(x.cuda(), w.cuda())
+    torch.cuda.synchronize()
+    want, bound = oracle.dense_linear(x.numpy(), w.numpy())
+    assert np.all(np.abs(y.cpu().numpy() - want) <= K_in * 2.0 ** -24 * bound)
+
+
+@pytest.mark.parametrize("N,H,W,C", [(3, 4, 4, 64), (2, 1, 17, 6), (5, 3, 11, 7)])
+def test_avgpool_pixel_batches(N, H, W, C):
+    """Pixel counts at and off the 16 loads kept in flight, odd channels."""
+    x = torch.randn(N, H, W, C, generator=inputs.generator(C)).to(torch.bfloat16)
+    y = tbn.tbn_avgpool2d_global_nhwc(x.cuda())
+    torch.cuda.synchronize()
+    want = x.double().mean((1, 2))
+    tol = H * W * 2.0 ** -24 * x.double().abs().mean((1, 2)) + 2.0 ** -24 * want.abs()
+    assert torch.all((y.cpu().double() - want).abs() <= tol)
