@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 #include <mutex>
 
 #include "tbn_device.cuh"
@@ -40,22 +41,22 @@ __device__ __forceinline__ uint32_t field_of_code(const uint32_t* row, int64_t i
 }
 
 // codes [K][R][S][C] -> codes_t [C][R][S][K] with the taps mirrored:
-// W'[c, r, s, k] = W~[k, R-1-r, S-1-s, c].  One thread per output word.
-__global__ void __launch_bounds__(256) transpose_codes_kernel(
-    const uint32_t* __restrict__ codes, int64_t wpf_in, uint32_t* __restrict__ out,
-    int64_t wpf_out, int K, int C, int R, int S) {
+// W'[c, r, s, k] = W~[k, R-1-r, S-1-s, c].  Thread `tid` of `nthreads` takes
+// output words in a grid stride.
+__device__ void transpose_codes(const uint32_t* __restrict__ codes, int64_t wpf_in,
+                                uint32_t* __restrict__ out, int64_t wpf_out, int K, int C, int R,
+                                int S, int64_t tid, int64_t nthreads) {
   const int64_t n_out = static_cast<int64_t>(R) * S * K;
   const int64_t total = static_cast<int64_t>(C) * wpf_out;
-  for (int64_t wi = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; wi < total;
-       wi += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+  for (int64_t wi = tid; wi < total; wi += nthreads) {
     const int c = static_cast<int>(wi / wpf_out);
     const int64_t j = wi - static_cast<int64_t>(c) * wpf_out;
     uint32_t o = 0u;
     if (K % 16 == 0) {
       // the word's 16 codes share the tap (r, s); input channels k0 .. k0+15
       const int64_t i0 = 16 * j;
-      const int k0 = static_cast<int>(i0 % K);
       const int64_t rs = i0 / K;
+      const int k0 = static_cast<int>(i0 - rs * K);
       const int s = static_cast<int>(rs % S), r = static_cast<int>(rs / S);
       const int64_t src = (static_cast<int64_t>(R - 1 - r) * S + (S - 1 - s)) * C + c;
 #pragma unroll
@@ -82,53 +83,117 @@ __global__ void __launch_bounds__(256) transpose_codes_kernel(
   }
 }
 
-// dyd [N][Hd][Wd][K] bf16 = alpha_k dy at (u / sh, v / sw) where both divide,
-// zero elsewhere; also ones[c] = 1 for the transposed filters' scales.  One
-// thread per output pixel, eight channels per step (16-byte loads and
-// stores when K % 8 == 0 and dy, dyd are 16-byte aligned).
-__global__ void __launch_bounds__(256) dilate_scale_kernel(
-    const __nv_bfloat16* __restrict__ dy, const float* __restrict__ alpha, int N, int P, int Q,
-    int K, int Hd, int Wd, int sh, int sw, __nv_bfloat16* __restrict__ dyd,
-    float* __restrict__ ones, int C, int vec) {
-  const int64_t npix = static_cast<int64_t>(N) * Hd * Wd;
-  const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t nthreads = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t c = tid; c < C; c += nthreads) ones[c] = 1.0f;
-  // one item = 8 channels of one pixel (vec) or one pixel (scalar path)
-  const int per_pix = vec ? K / 8 : 1;
-  for (int64_t e = tid; e < npix * per_pix; e += nthreads) {
+struct PrepArgs {
+  // codes
+  const uint32_t* codes;
+  uint32_t* codes_t;
+  int64_t wpf_in, wpf_out;
+  int K, C, R, S;
+  int code_blocks;         // blocks [0, code_blocks) transpose, the rest dilate
+  // dy
+  const __nv_bfloat16* dy;
+  const float* alpha;
+  __nv_bfloat16* dyd;
+  float* ones;
+  int N, P, Q, Hd, Wd, sh, sw;
+  int vec;                 // K % 8 == 0, dy and alpha 16-byte aligned
+  int small;               // fewer than 2^31 items: 32-bit indices
+  FastDiv by_pix, by_w, by_h, by_sh, by_sw;   // items per pixel, Wd, Hd, strides
+};
+
+__device__ __forceinline__ uint4 scale8(uint4 i4, const float* __restrict__ alpha) {
+  const float4 a0 = __ldg(reinterpret_cast<const float4*>(alpha));
+  const float4 a1 = __ldg(reinterpret_cast<const float4*>(alpha + 4));
+  const float al[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+  const uint32_t iw[4] = {i4.x, i4.y, i4.z, i4.w};
+  uint32_t ow[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&iw[q]));
+    ow[q] = pack_bf16x2(al[2 * q] * f.x, al[2 * q + 1] * f.y);
+  }
+  return make_uint4(ow[0], ow[1], ow[2], ow[3]);
+}
+
+// One launch before the convolution: the transposed codes, and dyd
+// [N][Hd][Wd][K] bf16 = alpha_k dy at (u / sh, v / sw) where both divide, zero
+// elsewhere; also ones[c] = 1 for the transposed filters' scales.  A thread
+// takes eight channels of one pixel per step (16-byte loads and stores), or
+// one whole pixel where those do not apply.  Bound: the bytes of dy and dyd;
+// with three 64-bit divisions per item the scaling ran at a third of their
+// rate (17.7 us with the transposition as a launch of its own, 128 x 16 x 16 x
+// 256), so 32-bit items divide by multiplication, and stride 1 needs only the
+// channel.
+template <bool kUnit>
+__global__ void __launch_bounds__(256) bwd_data_prep_kernel(const __grid_constant__ PrepArgs a) {
+  if (static_cast<int>(blockIdx.x) < a.code_blocks) {
+    transpose_codes(a.codes, a.wpf_in, a.codes_t, a.wpf_out, a.K, a.C, a.R, a.S,
+                    static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x,
+                    static_cast<int64_t>(a.code_blocks) * blockDim.x);
+    return;
+  }
+  const int64_t tid =
+      static_cast<int64_t>(blockIdx.x - a.code_blocks) * blockDim.x + threadIdx.x;
+  const int64_t nthreads = static_cast<int64_t>(gridDim.x - a.code_blocks) * blockDim.x;
+  for (int64_t c = tid; c < a.C; c += nthreads) a.ones[c] = 1.0f;
+  const int per_pix = a.vec ? a.K / 8 : 1;
+  const int64_t items = static_cast<int64_t>(a.N) * a.Hd * a.Wd * per_pix;
+  if (a.vec && a.small) {
+    const uint4* src = reinterpret_cast<const uint4*>(a.dy);
+    uint4* dst = reinterpret_cast<uint4*>(a.dyd);
+    const int n = static_cast<int>(items), step = static_cast<int>(min(nthreads, items));
+    if constexpr (kUnit) {
+      // dyd has dy's shape: item e scales the 16 bytes e, four in flight
+      for (int64_t e0 = tid; e0 < n; e0 += 4ll * step) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int64_t e = e0 + static_cast<int64_t>(u) * step;
+          if (e < n) v[u] = __ldg(src + e);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int64_t e = e0 + static_cast<int64_t>(u) * step;
+          if (e < n) {
+            const int i = static_cast<int>(e);
+            dst[i] = scale8(v[u], a.alpha + 8 * (i - a.by_pix(i) * per_pix));
+          }
+        }
+      }
+    } else {
+      for (int64_t e64 = tid; e64 < n; e64 += step) {
+        const int e = static_cast<int>(e64);
+        const int pix = a.by_pix(e), kv = e - pix * per_pix;
+        const int t = a.by_w(pix), v = pix - t * a.Wd;
+        const int im = a.by_h(t), u = t - im * a.Hd;
+        const int p = a.by_sh(u), q = a.by_sw(v);
+        uint4 o = make_uint4(0u, 0u, 0u, 0u);
+        if (p * a.sh == u && q * a.sw == v && p < a.P && q < a.Q)
+          o = scale8(__ldg(src + ((static_cast<int64_t>(im) * a.P + p) * a.Q + q) * per_pix + kv),
+                     a.alpha + 8 * kv);
+        dst[e] = o;
+      }
+    }
+    return;
+  }
+  for (int64_t e = tid; e < items; e += nthreads) {
     const int64_t pix = e / per_pix;
     const int kv = static_cast<int>(e - pix * per_pix);
-    const int v = static_cast<int>(pix % Wd);
-    const int64_t t = pix / Wd;
-    const int u = static_cast<int>(t % Hd);
-    const int n = static_cast<int>(t / Hd);
-    const bool hit = u % sh == 0 && v % sw == 0 && u / sh < P && v / sw < Q;
+    const int v = static_cast<int>(pix % a.Wd);
+    const int64_t t = pix / a.Wd;
+    const int u = static_cast<int>(t % a.Hd);
+    const int n = static_cast<int>(t / a.Hd);
+    const bool hit = u % a.sh == 0 && v % a.sw == 0 && u / a.sh < a.P && v / a.sw < a.Q;
     const __nv_bfloat16* src =
-        hit ? dy + ((static_cast<int64_t>(n) * P + u / sh) * Q + v / sw) * K : nullptr;
-    __nv_bfloat16* dst = dyd + pix * K;
-    if (vec) {
-      const int k = 8 * kv;
+        hit ? a.dy + ((static_cast<int64_t>(n) * a.P + u / a.sh) * a.Q + v / a.sw) * a.K : nullptr;
+    __nv_bfloat16* dst = a.dyd + pix * a.K;
+    if (a.vec) {
       uint4 o = make_uint4(0u, 0u, 0u, 0u);
-      if (hit) {
-        const uint4 i4 = __ldg(reinterpret_cast<const uint4*>(src + k));
-        const float4 a0 = __ldg(reinterpret_cast<const float4*>(alpha + k));
-        const float4 a1 = __ldg(reinterpret_cast<const float4*>(alpha + k + 4));
-        const float al[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-        const uint32_t iw[4] = {i4.x, i4.y, i4.z, i4.w};
-        uint32_t ow[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&iw[q]));
-          const __nv_bfloat162 r = __floats2bfloat162_rn(al[2 * q] * f.x, al[2 * q + 1] * f.y);
-          ow[q] = *reinterpret_cast<const uint32_t*>(&r);
-        }
-        o = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-      }
-      *reinterpret_cast<uint4*>(dst + k) = o;
+      if (hit) o = scale8(__ldg(reinterpret_cast<const uint4*>(src + 8 * kv)), a.alpha + 8 * kv);
+      *reinterpret_cast<uint4*>(dst + 8 * kv) = o;
     } else {
-      for (int k = 0; k < K; ++k)
-        dst[k] = __float2bfloat16_rn(hit ? __ldg(alpha + k) * __bfloat162float(src[k]) : 0.0f);
+      for (int k = 0; k < a.K; ++k)
+        dst[k] = __float2bfloat16_rn(hit ? __ldg(a.alpha + k) * __bfloat162float(src[k]) : 0.0f);
     }
   }
 }
@@ -516,6 +581,261 @@ __global__ void __launch_bounds__(kBwdThreads, 2) bwd_filter_tc_kernel(const Bwd
   }
 }
 
+// The same product fed by TMA, on tiles of 128 filters x up to 256 columns.
+// A column unit is 64 channels of one tap; a 64-pixel chunk of it is one
+// im2col-mode box (64 consecutive output pixels of the batch shifted by the
+// tap, zero-filled outside the image), 64 filters of dy one tiled box, so one
+// warp feeds the ring and no thread computes an address per element.  The
+// boxes land in the very layout described above.  Two accumulators take the
+// chunks in turn and are added at the end: half the length of each fp32 chain
+// of one accumulator per slice.  The partial tile leaves through shared
+// memory by TMA (clipped at C and K).
+//
+// Bound: the boxes' ingest, 48 KB per chunk for 512 cycles of MMAs.  Measured
+// with its reduction (3x3, batch 128): 128 -> 256 channels at 16 x 16 56.6 ->
+// 25.1 us (770 TFLOP/s), 512 -> 512 at 8 x 8 95.1 -> 41.2, 128 -> 128 at 32 x
+// 32 80.9 -> 41.7 us; the error against 64 bits about halves.
+constexpr int kTmaUnits = 4;                       // column units per tile at most
+constexpr int kTmaStages = 4;
+constexpr int kTmaStageBytes = (2 + kTmaUnits) * kHalfTile;
+constexpr int kTmaEpWarps = 8;
+constexpr int kTmaThreads = 32 * (2 + kTmaEpWarps);
+constexpr int kTmaTmem = 512;                      // two accumulators of 256 columns
+constexpr int kTmaSmem = 1024 + kTmaStages * kTmaStageBytes + 256;
+static_assert(kTmaSmem <= 232448, "shared memory budget");
+static_assert(kTmaUnits * 64 * 128 * 4 <= kTmaStages * kTmaStageBytes, "epilogue staging");
+
+struct BwdTmaArgs {
+  int units, per_cta;        // column units in all, and per tile
+  int cblocks, S, C, K;      // 64-channel blocks of C
+  int sh, sw, ph, pw;
+  FastDiv by_q, by_p;        // Q, P
+  int P, Q;
+  int chunks, chunks_per_slice;
+  uint32_t* err;
+};
+
+struct BwdTmaCtl {
+  uint64_t full[kTmaStages], empty[kTmaStages], done;
+  uint32_t tmem_base;
+  int abort;
+};
+
+// Four K = 16 steps of a 64-pixel chunk (2 KB apart in both operands) and
+// the commit to `done`, from one elected lane of a converged warp.
+__device__ __forceinline__ void tc_mma_ss_chunk(uint32_t d, uint64_t ad, uint64_t bd,
+                                                uint32_t idesc, uint32_t accumulate,
+                                                uint64_t* done) {
+  asm volatile(
+      "{\n\t.reg .pred e, p, t;\n\t.reg .b64 a1, a2, a3, b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "add.u64 a1, %1, 128;\n\tadd.u64 a2, %1, 256;\n\tadd.u64 a3, %1, 384;\n\t"
+      "add.u64 b1, %2, 128;\n\tadd.u64 b2, %2, 256;\n\tadd.u64 b3, %2, 384;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, b1, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a2, b2, %3, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a3, b3, %3, t;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}" ::"r"(
+          d),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate), "r"(smem_addr(done))
+      : "memory");
+}
+
+__global__ void __launch_bounds__(kTmaThreads, 1)
+    bwd_filter_tma_kernel(const __grid_constant__ CUtensorMap tmap_dy,
+                          const __grid_constant__ CUtensorMap tmap_x,
+                          const __grid_constant__ CUtensorMap tmap_part,
+                          const __grid_constant__ BwdTmaArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* ring = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
+  BwdTmaCtl* ctl = reinterpret_cast<BwdTmaCtl*>(ring + kTmaStages * kTmaStageBytes);
+  volatile int* abort_flag = &ctl->abort;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int k0 = blockIdx.x * 128, u0 = blockIdx.y * a.per_cta;
+  const int nu = min(a.per_cta, a.units - u0);
+  const int c_beg = blockIdx.z * a.chunks_per_slice;
+  const int n = max(0, min(a.chunks - c_beg, a.chunks_per_slice));
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kTmaStages; ++i) {
+      mbar_init(&ctl->full[i], 1);
+      mbar_init(&ctl->empty[i], 1);
+    }
+    mbar_init(&ctl->done, 1);
+    ctl->abort = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tmap_dy);
+    prefetch_tmap(&tmap_x);
+    prefetch_tmap(&tmap_part);
+  }
+  if (warp == 1) {
+    tmem_alloc(&ctl->tmem_base, kTmaTmem);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  if (ctl->tmem_base != 0u) {   // all 512 columns start at 0; else no work
+    if (threadIdx.x == 0) raise_device_error(a.err, TBN_DEVERR_BAD_LAUNCH);
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(ctl->tmem_base, kTmaTmem);
+    return;
+  }
+  bool ok = true;
+  if (warp == 0) {
+    // ---------------- producer
+    int issued = 0, st = 0;
+    uint32_t par = 1u;
+    for (int c = 0; c < n; ++c) {
+      ok = mbar_wait_warp(&ctl->empty[st], par, abort_flag, a.err, kBwdWaitLimitNs);
+      if (!ok) break;
+      const int pix = (c_beg + c) * kChunk;
+      const int row = a.by_q(pix), im = a.by_p(row);
+      const int w0 = (pix - row * a.Q) * a.sw - a.pw, h0 = (row - im * a.P) * a.sh - a.ph;
+      if (elect_one()) {
+        uint8_t* dst = ring + st * kTmaStageBytes;
+        mbar_arrive_expect_tx(&ctl->full[st], static_cast<uint32_t>((2 + nu) * kHalfTile));
+        tma_load_4d(dst, &tmap_dy, &ctl->full[st], k0, pix, 0, 0);
+        tma_load_4d(dst + kHalfTile, &tmap_dy, &ctl->full[st], k0 + 64, pix, 0, 0);
+        int tap = u0 / a.cblocks, cb = u0 - tap * a.cblocks;
+        int r = tap / a.S, q = tap - r * a.S;
+        for (int u = 0; u < nu; ++u) {
+          tma_load_im2col_4d(dst + (2 + u) * kHalfTile, &tmap_x, &ctl->full[st], 64 * cb, w0, h0,
+                             im, q, r);
+          if (++cb == a.cblocks) {
+            cb = 0;
+            if (++q == a.S) {
+              q = 0;
+              ++r;
+            }
+          }
+        }
+      }
+      __syncwarp();
+      ++issued;
+      if (++st == kTmaStages) {
+        st = 0;
+        par ^= 1u;
+      }
+    }
+    // every copy issued must land before the CTA may exit
+    for (int i = issued > kTmaStages ? issued - kTmaStages : 0; i < issued; ++i)
+      mbar_wait(&ctl->full[i % kTmaStages], static_cast<uint32_t>(i / kTmaStages) & 1u, nullptr,
+                a.err, kBwdWaitLimitNs);
+  } else if (warp == 1) {
+    // ---------------- MMA issue
+    const uint32_t idesc =
+        idesc_bf16_f32(128, static_cast<uint32_t>(64 * nu)) | (1u << 15) | (1u << 16);   // MN-major
+    const uint32_t ring_s = smem_addr(ring);
+    int st = 0;
+    uint32_t par = 0u;
+    for (int c = 0; c < n; ++c) {
+      ok = mbar_wait_warp(&ctl->full[st], par, abort_flag, a.err, kBwdWaitLimitNs);
+      if (!ok) break;
+      tc_fence_after_sync();
+      const uint32_t base = ring_s + static_cast<uint32_t>(st * kTmaStageBytes);
+      tc_mma_ss_chunk((c & 1) ? 256u : 0u, smem_desc_sw128_mn(base),
+                      smem_desc_sw128_mn(base + 2 * kHalfTile), idesc, c > 1 ? 1u : 0u,
+                      &ctl->empty[st]);
+      if (++st == kTmaStages) {
+        st = 0;
+        par ^= 1u;
+      }
+    }
+    // also after an abort: tensor memory is freed only when the MMAs are done
+    if (elect_one()) tc_commit(&ctl->done);
+    __syncwarp();
+    mbar_wait(&ctl->done, 0u, nullptr, a.err, kBwdWaitLimitNs);
+  } else {
+    // ---------------- epilogue
+    ok = mbar_wait(&ctl->done, 0u, abort_flag, a.err, kBwdWaitLimitNs);
+    ok = __all_sync(0xffffffffu, ok) && !*abort_flag;
+    tc_fence_after_sync();
+    // warp: lanes 32 (warp % 4) .. (filters), every other 32-column group;
+    // the ring is free now and holds the groups as 128-byte rows of 128 filters
+    const int sub = warp & 3, half = (warp - 2) >> 2;
+    const int row = 32 * sub + lane;
+    if (ok) {
+      for (int g = half; g < 2 * nu; g += 2) {
+        uint32_t v[32], v1[32];
+        const uint32_t col = (static_cast<uint32_t>(32 * sub) << 16) + static_cast<uint32_t>(32 * g);
+        tmem_ld_32x32b_x32(col, v);
+        tmem_ld_32x32b_x32(col + 256u, v1);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          // no chunk, or a single one: the accumulators hold nothing yet
+          const float x0 = n > 0 ? __uint_as_float(v[i]) : 0.0f;
+          const float x1 = n > 1 ? __uint_as_float(v1[i]) : 0.0f;
+          v[i] = __float_as_uint(x0 + x1);
+        }
+        uint8_t* dst = ring + g * (128 * 128) + row * 128;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          *reinterpret_cast<uint4*>(dst + ((i ^ (row & 7)) << 4)) =
+              make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+      fence_proxy_async_smem();
+    }
+    named_barrier_sync(1, 32 * kTmaEpWarps);
+    if (threadIdx.x == 64 && ok) {
+      for (int g = 0; g < 2 * nu; ++g) {
+        const int u = u0 + (g >> 1), tap = u / a.cblocks, c = 64 * (u - tap * a.cblocks) + 32 * (g & 1);
+        if (c < a.C) tma_store_4d(&tmap_part, ring + g * (128 * 128), c, tap, k0, blockIdx.z);
+      }
+      bulk_commit_group();
+      bulk_wait_group<0>();
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(0, kTmaTmem);
+  }
+}
+
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+// dw = the slices' partial values: the block's threads form `groups` (1, 2, 4
+// or 8) groups of 128 / groups; group g adds slices [8 g, 8 g + 8), [8 (g +
+// groups), ...), eight at a time in pairs and the eights in order, for four
+// values per thread (count % 4 == 0, 16-byte aligned), and group 0 adds the
+// groups in order.  Bound: the partial tiles' bytes, from L2; few weights over
+// many slices (64 -> 128, 1x1, 131 slices) need the groups: 16 blocks' loads
+// in sequence took 11 us.
+__global__ void __launch_bounds__(128) bwd_filter_reduce4_kernel(
+    const float4* __restrict__ part, int slices, int groups, int64_t count4,
+    float4* __restrict__ dw) {
+  __shared__ float4 sums[128];
+  const int per = 128 / groups;
+  const int li = threadIdx.x % per, g = threadIdx.x / per;
+  const int64_t e = static_cast<int64_t>(blockIdx.x) * per + li;
+  float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (e < count4) {
+    for (int z0 = 8 * g; z0 < slices; z0 += 8 * groups) {
+      float4 v[8];
+#pragma unroll
+      for (int z = 0; z < 8; ++z)
+        v[z] = z0 + z < slices ? __ldg(part + (z0 + z) * count4 + e)
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+      for (int w = 1; w < 8; w *= 2)
+#pragma unroll
+        for (int z = 0; z < 8; z += 2 * w) v[z] = add4(v[z], v[z + w]);
+      t = add4(t, v[0]);
+    }
+  }
+  sums[threadIdx.x] = t;
+  __syncthreads();
+  if (g == 0 && e < count4) {
+    for (int h = 1; h < groups; ++h) t = add4(t, sums[h * per + li]);
+    dw[e] = t;
+  }
+}
+
 // dw[e] = sum of the slices' partial values in a fixed order.  The block's
 // threads form `groups` (1, 2, 4 or 8, a function of the slice count) groups
 // of 256 / groups; group g sums slices g, g + groups, ... in order for one
@@ -580,6 +900,130 @@ int bwd_filter_slices(const BwdConvShape& p) {
   return static_cast<int>(std::min<int64_t>(s, 1024));
 }
 
+// The TMA-fed kernel: what limits an im2col tensor map (32-bit pixel indices,
+// 8-bit corner and tap offsets, strides up to 8), whole 16-byte rows, and at
+// least 40 channels, so that its 64-channel boxes are mostly channels.  Below
+// that, and for unaligned pointers, the kernels above (32 images of 28 x 28 x
+// 40 -> 72 at stride 2: 10.2 us against 11.7; equal at one small image).
+bool bwd_filter_tma_shape(const BwdConvShape& p) {
+  return p.K % 8 == 0 && p.C % 8 == 0 && p.C >= 40 && p.sh <= 8 && p.sw <= 8 && p.R <= 128 &&
+         p.S <= 128 && p.ph <= 127 && p.pw <= 127 && p.N * p.P * p.Q <= (int64_t(1) << 30) &&
+         p.N < (int64_t(1) << 30) && p.N * p.H * p.W * p.C * 2 >= 131072 &&
+         p.N * p.P * p.Q * p.K * 2 >= 131072;
+}
+
+// Its tiles (column units per CTA) and pixel slices, from the shape alone so
+// that the workspace query agrees with the launch.  A chunk costs a CTA about
+// 300 + 150 units cycles (its boxes' bytes); slices fill the machine once.
+struct BwdTmaPlan {
+  int units, per_cta, cblocks, chunks, per_slice, slices;
+};
+BwdTmaPlan plan_bwd_tma(const BwdConvShape& p) {
+  BwdTmaPlan t{};
+  t.cblocks = static_cast<int>((p.C + 63) / 64);
+  t.units = static_cast<int>(p.R * p.S * t.cblocks);
+  int64_t best = 0;
+  for (int u = 1; u <= kTmaUnits; ++u) {
+    const int64_t cost = static_cast<int64_t>((t.units + u - 1) / u) * (300 + 150 * u);
+    if (best == 0 || cost <= best) {
+      best = cost;
+      t.per_cta = u;
+    }
+  }
+  const int64_t tiles = ((p.K + 127) / 128) * ((t.units + t.per_cta - 1) / t.per_cta);
+  t.chunks = static_cast<int>((p.N * p.P * p.Q + kChunk - 1) / kChunk);
+  int64_t s = std::max<int64_t>(1, device_sm_count() / tiles);
+  s = std::min<int64_t>(s, std::max<int64_t>(1, t.chunks / 4));
+  s = std::min<int64_t>(s, std::max<int64_t>(1, (int64_t{16} << 20) / (p.K * p.R * p.S * p.C)));
+  t.per_slice = static_cast<int>((t.chunks + s - 1) / s);
+  t.slices = (t.chunks + t.per_slice - 1) / t.per_slice;
+  return t;
+}
+
+tbn_status launch_bwd_filter_tma(const BwdConvShape& p, const void* x, const void* dy, float* dw,
+                                 void* workspace, cudaStream_t s) {
+  const BwdTmaPlan t = plan_bwd_tma(p);
+  const int64_t rsc = p.R * p.S * p.C, count = p.K * rsc;
+  BwdTmaArgs a{};
+  a.units = t.units; a.per_cta = t.per_cta; a.cblocks = t.cblocks;
+  a.S = (int)p.S; a.C = (int)p.C; a.K = (int)p.K;
+  a.sh = (int)p.sh; a.sw = (int)p.sw; a.ph = (int)p.ph; a.pw = (int)p.pw;
+  a.P = (int)p.P; a.Q = (int)p.Q;
+  a.by_q = fast_div(a.Q);
+  a.by_p = fast_div(a.P);
+  a.chunks = t.chunks; a.chunks_per_slice = t.per_slice;
+  a.err = device_error_word();
+  // one slice: straight into dw where TMA can write it
+  const bool direct = t.slices == 1 && is_aligned(dw, 16);
+  alignas(64) CUtensorMap m_dy, m_x, m_part;
+  std::memset(&m_dy, 0, sizeof(m_dy));
+  std::memset(&m_x, 0, sizeof(m_x));
+  std::memset(&m_part, 0, sizeof(m_part));
+  const cuuint32_t one[4] = {1u, 1u, 1u, 1u};
+  const cuuint64_t npix = (cuuint64_t)(p.N * p.P * p.Q);
+  {
+    const cuuint64_t dim[4] = {(cuuint64_t)p.K, npix, 1u, 1u};
+    const cuuint64_t str[3] = {(cuuint64_t)(p.K * 2), (cuuint64_t)(p.K * 2) * npix,
+                               (cuuint64_t)(p.K * 2) * npix};
+    const cuuint32_t box[4] = {64u, (cuuint32_t)kChunk, 1u, 1u};
+    const CUresult cr = get_encode_tiled()(
+        &m_dy, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(dy), dim, str, box, one,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "backward filter: tensor map of dy failed (%d)", (int)cr);
+  }
+  {
+    const cuuint64_t dim[4] = {(cuuint64_t)p.C, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.N};
+    const cuuint64_t str[3] = {(cuuint64_t)(p.C * 2), (cuuint64_t)(p.W * p.C * 2),
+                               (cuuint64_t)(p.H * p.W * p.C * 2)};
+    const cuuint32_t estr[4] = {1u, (cuuint32_t)p.sw, (cuuint32_t)p.sh, 1u};
+    const int lower[2] = {-(int)p.pw, -(int)p.ph};
+    const int upper[2] = {(int)(p.pw - (p.S - 1)), (int)(p.ph - (p.R - 1))};
+    const CUresult cr = get_encode_im2col()(
+        &m_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dim, str, lower, upper,
+        64u, (cuuint32_t)kChunk, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "backward filter: tensor map of x failed (%d)", (int)cr);
+  }
+  {
+    const cuuint64_t dim[4] = {(cuuint64_t)p.C, (cuuint64_t)(p.R * p.S), (cuuint64_t)p.K,
+                               (cuuint64_t)t.slices};
+    const cuuint64_t str[3] = {(cuuint64_t)(p.C * 4), (cuuint64_t)(rsc * 4), (cuuint64_t)(count * 4)};
+    const cuuint32_t box[4] = {32u, 1u, 128u, 1u};
+    const CUresult cr = get_encode_tiled()(
+        &m_part, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, direct ? static_cast<void*>(dw) : workspace,
+        dim, str, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "backward filter: tensor map of dW failed (%d)", (int)cr);
+  }
+  static std::once_flag once;
+  static cudaError_t attr_err = cudaSuccess;
+  std::call_once(once, [] {
+    attr_err = cudaFuncSetAttribute(bwd_filter_tma_kernel,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, kTmaSmem);
+  });
+  if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(bwd_filter_tma_kernel)");
+  const dim3 grid(static_cast<unsigned>((p.K + 127) / 128),
+                  static_cast<unsigned>((t.units + t.per_cta - 1) / t.per_cta),
+                  static_cast<unsigned>(t.slices));
+  if (grid.y > 65535) return fail(TBN_ERR_UNSUPPORTED, "backward filter: R S C too large");
+  bwd_filter_tma_kernel<<<grid, kTmaThreads, kTmaSmem, s>>>(m_dy, m_x, m_part, a);
+  const tbn_status st = check_launch("bwd_filter_tma_kernel");
+  if (st != TBN_OK || direct) return st;
+  const float* part = static_cast<const float*>(workspace);
+  if (is_aligned(dw, 16)) {   // K % 8 == 0: count is a multiple of 4
+    const int groups = t.slices > 32 ? 8 : t.slices > 16 ? 4 : t.slices > 8 ? 2 : 1;
+    const int64_t per = 128 / groups;
+    bwd_filter_reduce4_kernel<<<static_cast<unsigned>((count / 4 + per - 1) / per), 128, 0, s>>>(
+        reinterpret_cast<const float4*>(part), t.slices, groups, count / 4,
+        reinterpret_cast<float4*>(dw));
+    return check_launch("bwd_filter_reduce4_kernel");
+  }
+  bwd_filter_reduce_kernel<<<static_cast<unsigned>((count + kBwdThreads - 1) / kBwdThreads),
+                             kBwdThreads, 0, s>>>(part, t.slices, 1, count, dw);
+  return check_launch("bwd_filter_reduce_kernel");
+}
+
 }  // namespace
 
 const char* bwd_shape_reason(const BwdConvShape& p) {
@@ -608,29 +1052,43 @@ tbn_status launch_bwd_data(const BwdConvShape& p, const void* dy, const uint32_t
   uint32_t* codes_t = reinterpret_cast<uint32_t*>(ws);
   float* ones = reinterpret_cast<float*>(ws + b.off_ones);
   __nv_bfloat16* dyd = reinterpret_cast<__nv_bfloat16*>(ws + b.off_dyd);
-  const int64_t wpf_in = (p.R * p.S * p.C + 15) / 16;
   {
-    const int64_t total = p.C * b.wpf_t;
-    const int64_t blocks = std::min<int64_t>((total + 255) / 256, 65536);
-    transpose_codes_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
-        codes, wpf_in, codes_t, b.wpf_t, static_cast<int>(p.K), static_cast<int>(p.C),
-        static_cast<int>(p.R), static_cast<int>(p.S));
-    const tbn_status st = check_launch("transpose_codes_kernel");
-    if (st != TBN_OK) return st;
-  }
-  {
-    const int64_t total = p.N * b.Hd * b.Wd * (p.K % 8 == 0 ? p.K / 8 : 1);
-    const int64_t blocks =
-        std::max<int64_t>(1, std::min<int64_t>((std::max<int64_t>(total, p.C) + 255) / 256,
-                                               static_cast<int64_t>(device_sm_count()) * 16));
+    PrepArgs a{};
+    a.codes = codes;
+    a.codes_t = codes_t;
+    a.wpf_in = (p.R * p.S * p.C + 15) / 16;
+    a.wpf_out = b.wpf_t;
+    a.K = static_cast<int>(p.K); a.C = static_cast<int>(p.C);
+    a.R = static_cast<int>(p.R); a.S = static_cast<int>(p.S);
+    a.dy = static_cast<const __nv_bfloat16*>(dy);
+    a.alpha = alpha;
+    a.dyd = dyd;
+    a.ones = ones;
+    a.N = static_cast<int>(p.N); a.P = static_cast<int>(p.P); a.Q = static_cast<int>(p.Q);
+    a.Hd = static_cast<int>(b.Hd); a.Wd = static_cast<int>(b.Wd);
+    a.sh = static_cast<int>(p.sh); a.sw = static_cast<int>(p.sw);
     // dyd is 256-aligned; alpha is read as float4 pairs
-    const int vec = (p.K % 8 == 0 && is_aligned(dy, 16) && is_aligned(alpha, 16)) ? 1 : 0;
-    dilate_scale_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(dy), alpha, static_cast<int>(p.N),
-        static_cast<int>(p.P), static_cast<int>(p.Q), static_cast<int>(p.K),
-        static_cast<int>(b.Hd), static_cast<int>(b.Wd), static_cast<int>(p.sh),
-        static_cast<int>(p.sw), dyd, ones, static_cast<int>(p.C), vec);
-    const tbn_status st = check_launch("dilate_scale_kernel");
+    a.vec = (p.K % 8 == 0 && is_aligned(dy, 16) && is_aligned(alpha, 16)) ? 1 : 0;
+    const int64_t per_pix = a.vec ? p.K / 8 : 1;
+    const int64_t items = p.N * b.Hd * b.Wd * per_pix;
+    a.small = items < (int64_t(1) << 31) ? 1 : 0;
+    a.by_pix = fast_div(static_cast<int>(per_pix));
+    a.by_w = fast_div(a.Wd);
+    a.by_h = fast_div(a.Hd);
+    a.by_sh = fast_div(a.sh);
+    a.by_sw = fast_div(a.sw);
+    a.code_blocks = static_cast<int>(std::min<int64_t>((p.C * b.wpf_t + 255) / 256, 65536));
+    // a thread of the unit-stride path takes four items at least
+    const bool unit = p.sh == 1 && p.sw == 1 && b.Hd == p.P && b.Wd == p.Q;
+    const int64_t threads = std::max<int64_t>(unit && a.vec && a.small ? (items + 3) / 4 : items, 1);
+    const int64_t blocks = std::min<int64_t>((threads + 255) / 256,
+                                             static_cast<int64_t>(device_sm_count()) * 16);
+    const unsigned grid = static_cast<unsigned>(a.code_blocks + blocks);
+    if (unit)
+      bwd_data_prep_kernel<true><<<grid, 256, 0, s>>>(a);
+    else
+      bwd_data_prep_kernel<false><<<grid, 256, 0, s>>>(a);
+    const tbn_status st = check_launch("bwd_data_prep_kernel");
     if (st != TBN_OK) return st;
   }
   // dx = the forward convolution of dyd with the transposed filters
@@ -653,12 +1111,17 @@ tbn_status launch_bwd_data(const BwdConvShape& p, const void* dy, const uint32_t
 }
 
 size_t bwd_filter_workspace_bytes(const BwdConvShape& p) {
-  const int slices = bwd_filter_slices(p);
+  // whichever kernel the pointers' alignment selects
+  int slices = bwd_filter_slices(p);
+  if (bwd_filter_tma_shape(p)) slices = std::max(slices, plan_bwd_tma(p).slices);
   return align256(static_cast<size_t>(slices) * p.K * p.R * p.S * p.C * 4);
 }
 
 tbn_status launch_bwd_filter(const BwdConvShape& p, const void* x, const void* dy, float* dw,
                              void* workspace, cudaStream_t s) {
+  if (bwd_filter_tma_shape(p) && is_aligned(x, 16) && is_aligned(dy, 16) &&
+      is_aligned(workspace, 16) && get_encode_tiled() != nullptr && get_encode_im2col() != nullptr)
+    return launch_bwd_filter_tma(p, x, dy, dw, workspace, s);
   BwdFilterArgs a{};
   a.x = static_cast<const __nv_bfloat16*>(x);
   a.dy = static_cast<const __nv_bfloat16*>(dy);

@@ -151,3 +151,37 @@ def test_bwd_vgg_small_batch128_sampled(i):
                                           (R, S), st, pd)
     got_dw = dw.cpu().reshape(K, R, S, C).permute(0, 3, 1, 2)[ks][:, cs].numpy()
     assert_within(got_dw, dw_orc, bw, out_bf16=False, what="vgg c%d b128 bwd filter" % (i + 1))
+
+
+TMA_CASES = [
+    # N, C, H, W, K, R, S, stride, pad: x and dy of at least 128 KiB, the
+    # filter gradient's TMA-fed tiles
+    (5, 64, 20, 21, 136, 3, 3, (1, 1), (1, 1)),    # two filter tiles, a last partial chunk
+    (6, 72, 23, 25, 128, 3, 3, (2, 2), (1, 1)),    # stride 2, a unit of 8 channels
+    (40, 40, 9, 11, 64, 1, 1, (1, 1), (0, 0)),     # one unit, partly channels
+    (3, 104, 20, 18, 72, 5, 5, (1, 1), (2, 2)),    # 50 units, the last tile short
+    (2, 128, 30, 27, 64, 2, 3, (1, 2), (1, 0)),    # R != S, stride and pad differ by axis
+    (700, 64, 2, 2, 64, 3, 3, (1, 1), (1, 1)),     # a chunk holds many images
+]
+
+
+@pytest.mark.parametrize("case", TMA_CASES)
+def test_bwd_tma_filter_and_prep(case):
+    """Both gradients at the edges of the TMA-fed filter tiles and of the
+    scaled (unit stride) and dilated copies of dy; run twice, bit for bit."""
+    N, C, H, W, K, R, S, st, pd = case
+    x, dy, codes, alpha, wt, al = make(case, 300 + sum(case[:7]))
+    xn = x.permute(0, 2, 3, 1).contiguous().cuda()
+    dyn = dy.permute(0, 2, 3, 1).contiguous().cuda()
+    dw = tbn.tbn_conv2d_bwd_filter(xn, dyn, R, S, st, pd)
+    assert torch.equal(dw, tbn.tbn_conv2d_bwd_filter(xn, dyn, R, S, st, pd))
+    dx = tbn.tbn_conv2d_bwd_data(dyn, codes, alpha, C, (H, W), R, S, st, pd)
+    torch.cuda.synchronize()
+    assert tbn.tbn_device_error() == 0
+    dw_orc, bound = oracle.conv2d_bwd_filter(x.float().numpy(), dy.float().numpy(), (R, S), st,
+                                             pd)
+    got = dw.cpu().reshape(K, R, S, C).permute(0, 3, 1, 2).numpy()
+    assert_within(got, dw_orc, bound, out_bf16=False, what="bwd filter %s" % (case,))
+    dx_orc, bx = oracle.conv2d_bwd_data(dy.float().numpy(), wt, al, (H, W), st, pd)
+    assert_within(dx.float().cpu().permute(0, 3, 1, 2).numpy(), dx_orc, bx, out_bf16=True,
+                  extra=BF16_TERM, what="bwd data %s" % (case,))
