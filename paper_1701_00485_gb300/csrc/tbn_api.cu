@@ -196,7 +196,10 @@ tbn_conv_algo pick_algo(const ConvProblem& p) {
 }
 
 tbn_status run_conv(const ConvProblem& p, tbn_conv_algo algo, cudaStream_t s) {
-  if (algo == TBN_CONV_AUTO) algo = pick_algo(p);
+  if (algo == TBN_CONV_AUTO) {
+    if (conv_igemm_pools_any_width(p)) return launch_conv_igemm(p, s);
+    algo = pick_algo(p);
+  }
   if (p.layout == TBN_S2D_NHWC && algo != TBN_CONV_IMPLICIT_GEMM) {
     if (algo != TBN_CONV_SMALL_TAPS && algo != TBN_CONV_DIRECT)
       return fail(TBN_ERR_INVALID_ARG, "conv: bad algorithm %d", (int)algo);

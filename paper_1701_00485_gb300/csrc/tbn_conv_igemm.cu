@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
 // tile is whole output rows of one image, the filter spans at most
 // kPatchMaxKBlocks K blocks and two patches fit beside the ring.
 int patch_cap_bytes(const ConvProblem& p, const TilePlan& t) {
-  if (use_tma(p) || t.tiles_q != 1 || t.bn != 1) return 0;
+  if (tma_fed(p) || t.tiles_q != 1 || t.bn != 1) return 0;
   const int64_t kblocks = (p.C * p.R * p.S + kBK - 1) / kBK;
   if (kblocks > kPatchMaxKBlocks) return 0;
   const int64_t rows = static_cast<int64_t>(t.bh - 1) * p.sh + p.R;
@@ -83,11 +83,11 @@ int conv_igemm_splitk(const ConvProblem& p, size_t* workspace_bytes) {
   // fully-connected shapes only (a 1x1 convolution over a 1x1 image): a
   // tile's pixel i is then image n0 + i, and the partial sums are stored
   // without the pixel walk of a general tile
-  if (!use_tma(p) || p.pool || p.P != 1 || p.Q != 1 || p.R != 1 || p.S != 1) return 1;
+  if (!tma_fed(p) || p.pool || p.P != 1 || p.Q != 1 || p.R != 1 || p.S != 1) return 1;
   const TilePlan t = plan_tiles(p);
   const int64_t base = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n *
                        ((p.K + kBM - 1) / kBM);
-  const int64_t kblocks = (p.C * p.R * p.S + kBK - 1) / kBK;
+  const int64_t kblocks = kblocks_of(p);
   const int sms = device_sm_count();
   if (2 * base > sms || kblocks < 8) return 1;
   int64_t S = std::min<int64_t>(sms / base, kblocks / 4);
@@ -144,16 +144,29 @@ const char* conv_igemm_unsupported_reason(const ConvProblem& p) {
   if (p.H * p.W * p.C >= (int64_t(1) << 31)) return "image too large";
   if (p.R >= (1 << 15) || p.S >= (1 << 15)) return "kernel too large";
   if (use_tma(p) && (p.ph > p.R || p.pw > p.S)) return "implicit GEMM needs pad <= kernel extent";
-  if (p.pool && pool_width(p, plan_tiles(p)) < 0)
+  const int pool_bw = pool_width(p, plan_tiles(p));
+  if (pool_bw < 0 || pool_bw == 1)
     return "fused pool needs whole output rows of width 8, 16 or 32 per tile";
   int dev = 0, major = 0, minor = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return "no CUDA device";
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
   if (major != 10 || minor != 3) return "implicit GEMM kernel is built for sm_103a only";
-  if ((use_tma(p) || use_tma_store(p)) && get_encode_tiled() == nullptr)
+  if ((tma_fed(p) || use_tma_store(p)) && get_encode_tiled() == nullptr)
     return "cuTensorMapEncodeTiled unavailable";
   return "";
+}
+
+// A fused pool over rows of a width that the explicit implicit-GEMM algorithm
+// refuses (not 8, 16 or 32) but its TMA-fed modes can pool: AUTO's choice
+// then, against the CUDA-core kernel (3x3, 64 -> 128 channels, 24 x 28, batch
+// 21, pooled: 454 us there).
+bool conv_igemm_pools_any_width(const ConvProblem& p) {
+  if (!p.pool || p.layout != TBN_NHWC || p.residual || !tma_fed(p)) return false;
+  ConvProblem q = p;
+  q.pool = 0;
+  if (conv_igemm_unsupported_reason(q)[0] != '\0') return false;
+  return pool_width(p, plan_tiles(p)) == 1;
 }
 
 tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
@@ -170,11 +183,11 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   a.tiles_k = ceil_div(p.K, kBM);
   const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n * a.tiles_k;
   a.ncodes = (int)(p.C * p.R * p.S);
-  a.kblocks = ceil_div(a.ncodes, kBK);
+  a.kblocks = static_cast<int>(kblocks_of(p));
   const bool split = p.ksplit > 1 && p.partial != nullptr;
   a.ksplit = split ? p.ksplit : 1;
   a.kb_per = ceil_div(a.kblocks, a.ksplit);
-  if (split && (!use_tma(p) || p.pool || p.P != 1 || p.Q != 1 || p.R != 1 || p.S != 1 ||
+  if (split && (!tma_fed(p) || p.pool || p.P != 1 || p.Q != 1 || p.R != 1 || p.S != 1 ||
                 (a.ksplit - 1) * a.kb_per >= a.kblocks))
     return fail(TBN_ERR_INVALID_ARG, "implicit GEMM: bad split-K request");
   if (tiles * a.ksplit > 0x7fffffffLL) return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: too many tiles");
@@ -222,8 +235,9 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const bool tst = use_tma_store(p) && !split;   // partial sums: direct fp32 stores
   if (split) {
     // the K ranges' partial sums, then their ordered sum with the epilogue
-    const tbn_status st = use_ch32(p) ? launch_igemm_tma32(p, t, a, pw, false, false, s)
-                                      : launch_igemm_tma64(p, t, a, pw, false, false, s);
+    const tbn_status st = use_tma_pad(p) ? launch_igemm_pad(p, t, a, pw, false, s)
+                          : use_ch32(p)  ? launch_igemm_tma32(p, t, a, pw, false, false, s)
+                                         : launch_igemm_tma64(p, t, a, pw, false, false, s);
     if (st != TBN_OK) return st;
     const int64_t mk = p.N * p.P * p.Q * p.K;
     const bool vec = p.K % 4 == 0 && is_aligned(p.partial, 16);
@@ -249,6 +263,7 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   if (use_tma(p)) {
     return launch_igemm_tma64(p, t, a, pw, tst, a.wq != nullptr, s);
   }
+  if (use_tma_pad(p)) return launch_igemm_pad(p, t, a, pw, tst, s);
   const int cap = patch_cap_bytes(p, t);
   if (cap > 0) {
     a.PR = (t.bh - 1) * a.sh + a.R;

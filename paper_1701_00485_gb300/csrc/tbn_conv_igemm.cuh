@@ -32,9 +32,13 @@
 //                   boxes of 32 channels, each from its own tap, into two
 //                   64-byte-row halves of the stage with the 64-byte swizzle
 //                   (a box past the filter's last code is loaded out of
-//                   range and arrives zero-filled).  Otherwise gather warps
-//                   assemble the rows from a per-K-block table of (tap,
-//                   channel) offsets.
+//                   range and arrives zero-filled).  When C % 8 == 0 (other
+//                   counts) every tap has ceil(C / 64) K blocks of its own:
+//                   the last box of a tap reaches past C and arrives
+//                   zero-filled there, so whatever codes stand in those
+//                   columns add zero, and whole steps of 16 past C are
+//                   skipped.  Otherwise gather warps assemble the rows from
+//                   a per-K-block table of (tap, channel) offsets.
 //   D               fp32 in tensor memory (256 columns).  Epilogue warps read
 //                   lane = filter, column = pixel, multiply by 2 * alpha (Eq. 1
 //                   applies alpha to the whole filter; the factor 2 undoes the
@@ -183,6 +187,7 @@ constexpr int kModePatch = 3;   // the tile's input rows are staged in shared me
                                 // copy, double-buffered) and threads build the rows from there
 constexpr int kModeS2d = 4;     // space-to-depth input: 64-channel TMA boxes, and the
                                 // filter's K blocks decoded once per CTA into tensor memory
+constexpr int kModeTmaPad = 5;  // 64-channel TMA boxes, each tap's last one padded (C % 8 == 0)
 constexpr int kMaxResidentKB = 15;   // resident K blocks: 32 columns each beside the accumulator
 
 __host__ __device__ constexpr bool mode_gathers(int mode) {
@@ -270,20 +275,21 @@ __device__ __forceinline__ TileCoord tile_coord(const IgArgs& a, int t) {
 
 // Direct global store of one output value (the path for fp32 output or
 // shapes the TMA store cannot take): fp32 math, residual, ReLU, rounding.
-__device__ __forceinline__ void store_out(const IgArgs& a, size_t o, float v) {
-  if (a.y_bf16) {
-    if (a.residual) v += __bfloat162float(static_cast<const __nv_bfloat16*>(a.residual)[o]);
-    if (a.relu) v = fmaxf(v, 0.0f);
+__device__ __forceinline__ float load_residual(const IgArgs& a, size_t o) {
+  return a.y_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(a.residual)[o])
+                  : static_cast<const float*>(a.residual)[o];
+}
+__device__ __forceinline__ void store_out(const IgArgs& a, size_t o, float v, float res = 0.0f) {
+  if (a.residual) v += res;
+  if (a.relu) v = fmaxf(v, 0.0f);
+  if (a.y_bf16)
     static_cast<__nv_bfloat16*>(a.y)[o] = __float2bfloat16_rn(v);
-  } else {
-    if (a.residual) v += static_cast<const float*>(a.residual)[o];
-    if (a.relu) v = fmaxf(v, 0.0f);
+  else
     static_cast<float*>(a.y)[o] = v;
-  }
 }
 
 // kPoolBW: 0 = no pool; 8, 16, 32 = fused 2x2/2 max pool for tiles of whole
-// output rows of that width.  kTmaStore: bf16 output through the staging
+// output rows of that width; 1 = of any width (a.bw).  kTmaStore: bf16 output through the staging
 // tile and TMA stores (else direct global stores).
 // Fused quantization prologue: CTA b quantizes filters [b K / G, (b + 1) K / G)
 // exactly as the quantize kernel does (the same per-word fields and sums,
@@ -408,6 +414,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
   constexpr bool kCh32 = kMode == kModeTma32;
   constexpr bool kPatch = kMode == kModePatch;
   constexpr bool kS2d = kMode == kModeS2d;
+  constexpr bool kPad = kMode == kModeTmaPad;
   constexpr int kSt = stages_for(kMode);   // ring stages
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte aligned by pointer arithmetic on the shared array, so that the
@@ -512,7 +519,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     constexpr int kBoxCh = kCh32 ? kBK / 2 : kBK;   // channels per box
     constexpr int kBoxes = kBK / kBoxCh;             // boxes per K block
     const uint32_t box_bytes = static_cast<uint32_t>(a.bw * a.bh * a.bn * kBoxCh * 2);
-    const int cblocks = a.C / kBoxCh;                // boxes per tap
+    const int cblocks = (a.C + kBoxCh - 1) / kBoxCh;   // boxes per tap
     int g = 0;  // global K-block counter of this CTA
     int st = 0;          // its ring stage
     uint32_t par = 0;    // and the parity of the stage's fill
@@ -897,6 +904,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     const uint32_t idesc = idesc_bf16_f32(kBM, static_cast<uint32_t>(a.tile_n));
     int issued = 0, st = 0;
     uint32_t tiles_done = 0, par = 0;
+    const int tap_blocks = (a.C + kBK - 1) / kBK;   // padded mode: K blocks per tap
     bool ok = true;
     for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++tiles_done) {
       const TileCoord tc = tile_coord(a, t);
@@ -906,6 +914,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const uint32_t acc_t = acc_tmem + ab * kAcc2Cols;
       ok = mbar_wait_warp(&ctl->acc_empty[ab], (use & 1u) ^ 1u, abort_flag, a.err, kWaitLimitNs);
       if (!ok) break;
+      int left = kPad ? a.C - kBK * (tc.kb0 % tap_blocks) : kBK;   // channels left in the tap
       for (int kb = tc.kb0; kb < tc.kb1; ++kb) {
         ok = mbar_wait_warp(&ctl->full[st], par, abort_flag, a.err, kWaitLimitNs);
         if (kS2d && tiles_done == 0 && ok)   // first use of a resident K block
@@ -921,8 +930,9 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         constexpr uint32_t kHalf = kCh32 ? (kStageBytes / 2) >> 4 : 4u;
         tc_mma_ts_block<2, kHalf, kHalf + 2>(
             acc_t, a_col, kCh32 ? smem_desc_sw64_kmajor(b_addr) : smem_desc_sw128_kmajor(b_addr),
-            idesc, kb != tc.kb0 ? 1u : 0u, 4, &ctl->empty[st],
+            idesc, kb != tc.kb0 ? 1u : 0u, kPad ? (left + 15) / 16 : 4, &ctl->empty[st],
             kb == tc.kb1 - 1 ? &ctl->acc_full[ab] : nullptr);
+        if (kPad) left = left > kBK ? left - kBK : a.C;
         ++issued;
         if (++st == kSt) {
           st = 0;
@@ -987,18 +997,57 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     int t_ld = blockIdx.x, kb_ld = 0, kb_end = 0, kb_lim = 0;
     const int kb_words = (a.wpf - 2 * half + 3) / 4;   // K blocks whose two words begin in the row
     const uint32_t* cp = a.codes;
+    // padded mode: this half block's first code, and channels left in its tap
+    const int tap_blocks = (a.C + kBK - 1) / kBK;
+    int code0 = 0, ch_left = 0;
     auto set_row = [&]() {
       const TileCoord tc = tile_coord(a, t_ld < a.tiles ? t_ld : 0);
       kb_ld = tc.kb0;
       kb_end = tc.kb1;
       const int k = tc.ktile * kBM + m;
       const bool in = t_ld < a.tiles && k < a.K;
+      if constexpr (kPad) {
+        const int tap = kb_ld / tap_blocks, cb = kb_ld - tap * tap_blocks;
+        ch_left = a.C - kBK * cb;
+        code0 = tap * a.C + kBK * cb + 32 * half;
+        kb_lim = in ? kb_end : 0;
+        cp = a.codes + static_cast<size_t>(in ? k : 0) * a.wpf;
+        return;
+      }
       kb_lim = in ? kb_words : 0;
       cp = a.codes + static_cast<size_t>(in ? k : 0) * a.wpf + 4 * kb_ld + 2 * half;
     };
     set_row();
     auto next_codes = [&]() -> uint2 {
       uint2 r = make_uint2(0u, 0u);
+      if constexpr (kPad) {
+        // 32 codes from code0 on (a multiple of 8: whole words, or the upper
+        // half of one and the lower half of the next); words past the row are
+        // zero, codes of the next tap multiply zero activations
+        if (kb_ld < kb_lim && ch_left > 32 * half) {
+          const int w = code0 >> 4;
+          const uint32_t w0 = __ldg(cp + w);
+          const uint32_t w1 = w + 1 < a.wpf ? __ldg(cp + w + 1) : 0u;
+          r = make_uint2(w0, w1);
+          if (code0 & 8) {
+            const uint32_t w2 = w + 2 < a.wpf ? __ldg(cp + w + 2) : 0u;
+            r.x = ((w0 >> 4) & 0x0F0F0F0Fu) | ((w1 & 0x0F0F0F0Fu) << 4);
+            r.y = ((w1 >> 4) & 0x0F0F0F0Fu) | ((w2 & 0x0F0F0F0Fu) << 4);
+          }
+        }
+        if (ch_left > kBK) {
+          ch_left -= kBK;
+          code0 += kBK;
+        } else {
+          code0 += ch_left;
+          ch_left = a.C;
+        }
+        if (++kb_ld == kb_end) {
+          t_ld += gridDim.x;
+          set_row();
+        }
+        return r;
+      }
       if (kb_ld < kb_lim) {
         // written by this launch's prologue when fused: ordinary (L1-cached,
         // coherent) loads after the grid barrier's acquire then, not the
@@ -1225,17 +1274,30 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
               if (kvalid && 32 * j + i < T && tc.n0 + 32 * j + i < a.N)
                 dst[static_cast<size_t>(i) * a.K] = __uint_as_float(v[i]);
           } else {
+            // eight pixels at a time: their residuals are all requested before
+            // the first output is stored (a load behind each store, which may
+            // alias it, cost a memory latency per pixel)
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const int px = 32 * j + i;
-              const int q = tc.q0 + wi, p = tc.p0 + hi, n = tc.n0 + ni;
-              if (kvalid && px < T && q < a.Q && p < a.P && n < a.N)
-                store_out(a, ((static_cast<size_t>(n) * a.P + p) * a.Q + q) * a.K + k,
-                          a2 * __uint_as_float(v[i]));
-              if (++wi == a.bw) {
-                wi = 0;
-                if (++hi == a.bh) { hi = 0; ++ni; }
+            for (int i0 = 0; i0 < 32; i0 += 8) {
+              size_t o[8];
+              bool in[8];
+              float res[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const int q = tc.q0 + wi, p = tc.p0 + hi, n = tc.n0 + ni;
+                in[i] = kvalid && 32 * j + i0 + i < T && q < a.Q && p < a.P && n < a.N;
+                o[i] = ((static_cast<size_t>(n) * a.P + p) * a.Q + q) * a.K + k;
+                if (++wi == a.bw) {
+                  wi = 0;
+                  if (++hi == a.bh) { hi = 0; ++ni; }
+                }
               }
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                res[i] = in[i] && a.residual ? load_residual(a, o[i]) : 0.0f;
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                if (in[i]) store_out(a, o[i], a2 * __uint_as_float(v[i0 + i]), res[i]);
             }
           }
         }
@@ -1243,6 +1305,37 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
           tc_fence_before_sync();
           mbar_arrive(&ctl->acc_empty[ab]);
         }
+      } else if constexpr (kPoolBW == 1) {
+        // fused 2x2 max pool of rows of any width a.bw: items of eight pooled
+        // outputs of one row pair, 16 columns of each row per load (columns
+        // past the row are read and not used; all 512 are allocated)
+        const int Qp = a.bw / 2, groups = (Qp + 7) / 8, bh2 = a.bh / 2;
+        const int items = a.bh * a.bn / 2 * groups;
+        for (int it = half; it < items; it += 2) {
+          const int pair = it / groups, g = it - pair * groups;
+          uint32_t v0[16], v1[16];
+          const uint32_t col = acc + static_cast<uint32_t>(pair * 2 * a.bw + 16 * g);
+          tmem_ld_32x32b_x16(col, v0);
+          tmem_ld_32x32b_x16(col + static_cast<uint32_t>(a.bw), v1);
+          tmem_wait_ld();
+          const int ni = pair / bh2, p2 = tc.p0 / 2 + pair - ni * bh2, n = tc.n0 + ni;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int q2 = 8 * g + j;
+            // alpha >= 0, so max commutes with the scaling (and with ReLU)
+            float mx = a2 * fmaxf(fmaxf(__uint_as_float(v0[2 * j]), __uint_as_float(v0[2 * j + 1])),
+                                  fmaxf(__uint_as_float(v1[2 * j]), __uint_as_float(v1[2 * j + 1])));
+            if (q2 >= Qp) continue;
+            if (kTmaStore) {
+              if (a.relu) mx = fmaxf(mx, 0.0f);
+              stage[(pair * Qp + q2) * kBM + m] = __float2bfloat16_rn(mx);
+            } else if (kvalid && p2 < Po && q2 < Qo && n < a.N) {
+              store_out(a, ((static_cast<size_t>(n) * Po + p2) * Qo + q2) * a.K + k, mx);
+            }
+          }
+        }
+        tc_fence_before_sync();
+        mbar_arrive(&ctl->acc_empty[ab]);
       } else {
         // fused 2x2 max pool: tiles hold whole rows of width kPoolBW (q0 = 0)
         // and an even number of rows per image; one TMEM load covers an even
@@ -1332,6 +1425,15 @@ inline int ceil_div(int64_t a, int64_t b) { return static_cast<int>((a + b - 1) 
 // TMA activations: whole 64-channel boxes, or 32-channel boxes in pairs.
 inline bool use_tma(const ConvProblem& p) { return p.C % (kBK / 2) == 0 && p.sh <= 2 && p.sw <= 2; }
 inline bool use_ch32(const ConvProblem& p) { return p.C % kBK != 0; }
+// Other multiples of 8 channels: 64-channel boxes, each tap's last one padded.
+inline bool use_tma_pad(const ConvProblem& p) {
+  return !use_tma(p) && p.C % 8 == 0 && p.sh <= 2 && p.sw <= 2 && p.ph <= p.R && p.pw <= p.S;
+}
+inline bool tma_fed(const ConvProblem& p) { return use_tma(p) || use_tma_pad(p); }
+inline int64_t kblocks_of(const ConvProblem& p) {
+  return use_tma_pad(p) ? p.R * p.S * ((p.C + kBK - 1) / kBK)
+                        : (p.C * p.R * p.S + kBK - 1) / kBK;
+}
 
 // Output pixels per tile: whole rows of the output (so one TMA box per tap
 // covers the tile), balanced so the last tile along each axis is not a
@@ -1339,8 +1441,8 @@ inline bool use_ch32(const ConvProblem& p) { return p.C % kBK != 0; }
 // output rows and an even number of them per image.
 inline TilePlan plan_tiles(const ConvProblem& p) {
   TilePlan t{};
-  const int stride_w = use_tma(p) ? static_cast<int>(p.sw) : 1;
-  const int stride_h = use_tma(p) ? static_cast<int>(p.sh) : 1;
+  const int stride_w = tma_fed(p) ? static_cast<int>(p.sw) : 1;
+  const int stride_h = tma_fed(p) ? static_cast<int>(p.sh) : 1;
   const int bw_max = static_cast<int>(std::min<int64_t>(p.Q, kMaxTileN / stride_w));
   t.tiles_q = ceil_div(p.Q, bw_max);
   t.bw = ceil_div(p.Q, t.tiles_q);
@@ -1373,11 +1475,15 @@ inline TilePlan plan_tiles(const ConvProblem& p) {
   return t;
 }
 
+// The kernel's kPoolBW for a plan: -1 where a tile cannot pool (whole rows,
+// an even number of them); 1 for rows of other widths than 8, 16 and 32,
+// which the TMA-fed modes alone take (the explicit algorithm refuses them:
+// conv_igemm_unsupported_reason).
 inline int pool_width(const ConvProblem& p, const TilePlan& t) {
   if (!p.pool) return 0;
   if (t.tiles_q != 1 || t.T > kMaxTileN || (t.bh & 1)) return -1;
   if (t.bw == 8 || t.bw == 16 || t.bw == 32) return t.bw;
-  return -1;
+  return tma_fed(p) ? 1 : -1;
 }
 
 // Estimated time (ns) of a TMA-mode plan.  A K block of a T-pixel tile takes
@@ -1390,7 +1496,7 @@ inline double plan_cost(const ConvProblem& p, const TilePlan& t, bool resident, 
   const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n *
                         ((p.K + kBM - 1) / kBM);
   const double waves = static_cast<double>((tiles + sms - 1) / sms);
-  const double kb = static_cast<double>((p.C * p.R * p.S + kBK - 1) / kBK);
+  const double kb = static_cast<double>(kblocks_of(p));
   const bool acc2 = !resident && t.tile_n <= kAcc2Cols;
   return waves * (kb * (215.0 + 0.25 * t.tile_n) + (acc2 ? 900.0 : 1700.0));
 }
@@ -1400,7 +1506,7 @@ inline double plan_cost(const ConvProblem& p, const TilePlan& t, bool resident, 
 // 32-bit pixel indices, and at least 128 KiB of input (smaller tensors are
 // left to tiled boxes, which is where the one-image layers are).
 inline bool im2col_ok(const ConvProblem& p) {
-  return use_tma(p) && p.R <= 128 && p.S <= 128 && p.ph <= 127 && p.pw <= 127 &&
+  return tma_fed(p) && p.R <= 128 && p.S <= 128 && p.ph <= 127 && p.pw <= 127 &&
          p.N * p.P * p.Q <= (int64_t(1) << 30) && p.N * p.H * p.W * p.C * 2 >= 131072 &&
          get_encode_im2col() != nullptr;
 }
@@ -1417,7 +1523,7 @@ inline bool im2col_ok(const ConvProblem& p) {
 // stay beside the accumulator.
 inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
   TilePlan best = plan_tiles(p);
-  if (!use_tma(p) || p.ksplit > 1) return best;
+  if (!tma_fed(p) || p.ksplit > 1) return best;
   const int sms = device_sm_count();
   double cost = plan_cost(p, best, resident, sms);
   const auto consider = [&](const TilePlan& t) {
@@ -1443,7 +1549,7 @@ inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
         t.tiles_q = ceil_div(t.oQ, T);
         consider(t);
       }
-    } else if (p.P % 2 == 0 && (p.Q == 8 || p.Q == 16 || p.Q == 32)) {
+    } else if (p.P % 2 == 0 && best.tiles_q == 1) {
       // row pairs of all images in sequence (P even: none crosses images)
       t.oP = p.N * p.P;
       t.oQ = p.Q;
@@ -1451,7 +1557,8 @@ inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
       t.tiles_q = 1;
       for (int rows = 2; rows * t.bw <= t_max; rows += 2) {
         t.bh = rows;
-        t.T = t.tile_n = rows * t.bw;
+        t.T = rows * t.bw;
+        t.tile_n = ((t.T + 15) / 16) * 16;
         t.tiles_p = ceil_div(t.oP, rows);
         consider(t);
       }
@@ -1589,6 +1696,10 @@ tbn_status launch_pool(const ConvProblem& p, const TilePlan& t, IgArgs& a, int p
     case 8: return launch_t<kMode, 8, kTmaStore, kFuse>(p, t, a, s);
     case 16: return launch_t<kMode, 16, kTmaStore, kFuse>(p, t, a, s);
     case 32: return launch_t<kMode, 32, kTmaStore, kFuse>(p, t, a, s);
+    case 1:
+      if constexpr (!mode_gathers(kMode) && !kFuse)
+        return launch_t<kMode, 1, kTmaStore, kFuse>(p, t, a, s);
+      return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: no pooled rows of this width");
     default: return launch_t<kMode, 0, kTmaStore, kFuse>(p, t, a, s);
   }
 }
@@ -1602,5 +1713,7 @@ tbn_status launch_igemm_tma64(const ConvProblem& p, const TilePlan& t, IgArgs& a
                               bool tma_store, bool fuse, cudaStream_t s);
 tbn_status launch_igemm_tma32(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
                               bool tma_store, bool fuse, cudaStream_t s);
+tbn_status launch_igemm_pad(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
+                            bool tma_store, cudaStream_t s);
 
 }  // namespace tbn

@@ -117,6 +117,8 @@ tbn_status launch_conv_direct(const ConvProblem& p, cudaStream_t s);
 // Empty string when the implicit-GEMM kernel can run `p`, else the reason.
 const char* conv_igemm_unsupported_reason(const ConvProblem& p);
 tbn_status launch_conv_igemm(const ConvProblem& p, cudaStream_t s);
+// True for a fused pool that only AUTO sends to the implicit GEMM.
+bool conv_igemm_pools_any_width(const ConvProblem& p);
 // Space-to-depth layout change of a bf16 NCHW or NHWC input for the
 // convolution geometry (C, H, W, R, S, stride, pad) (see S2dGeom).
 tbn_status launch_space_to_depth(const void* x, tbn_layout layout, int64_t N, int64_t C,

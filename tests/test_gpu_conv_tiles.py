@@ -77,3 +77,78 @@ def test_pixel_run_tiles_pooled(N, C, hw):
         y = y.float().cpu().permute(0, 3, 1, 2).numpy()
         assert_within(y, want, bound, out_bf16=dt == torch.bfloat16, epilogue=True,
                       what="pooled runs %d %d" % (N, hw))
+
+
+PADDED = [
+    # N, C, H, W, K, R, S, stride, pad: C % 8 == 0, no multiple of 32: each
+    # tap's last 64-channel box reaches past C
+    (3, 8, 12, 11, 40, 3, 3, (1, 1), (1, 1)),       # one step per K block, half-word taps
+    (9, 40, 27, 27, 136, 5, 5, (1, 1), (2, 2)),     # runs of pixels, two filter tiles
+    (2, 72, 9, 10, 72, 3, 3, (2, 2), (1, 1)),       # a block of 8 channels after one of 64
+    (5, 120, 14, 13, 64, 1, 1, (1, 1), (0, 0)),     # 1x1, half a word at the row's end
+    (1, 48, 3, 300, 24, 2, 3, (1, 2), (1, 0)),      # whole words, columns split
+    (130, 200, 1, 1, 300, 1, 1, (1, 1), (0, 0)),    # a linear layer's shape
+]
+
+
+@pytest.mark.parametrize("case", PADDED)
+def test_padded_channel_blocks(case):
+    c = _case(*case, seed=sum(case[:7]))
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.float32,
+                  algo=tbn.TBN_CONV_IMPLICIT_GEMM)
+    assert_within(y, y_orc, bound, out_bf16=False, what="padded %s" % (case,))
+    for dt in (torch.float32, torch.bfloat16):
+        res = torch.randn(*y_orc.shape, generator=inputs.generator(3)).to(dt)
+        want = oracle.epilogue(y_orc, res.float().numpy(), relu=True)
+        y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, dt, algo=tbn.TBN_CONV_IMPLICIT_GEMM, relu=True,
+                      residual=res)
+        assert_within(y, want, bound, out_bf16=dt == torch.bfloat16, epilogue=True,
+                      what="padded epi %s" % (case,))
+
+
+@pytest.mark.parametrize("B,K_in,K_out", [(9, 1000, 70), (64, 2008, 130), (2, 520, 33)])
+def test_padded_linear(B, K_in, K_out):
+    """Fully-connected layers whose K_in is a multiple of 8 only, with the
+    workspace that lets K be split."""
+    g = inputs.generator(K_in)
+    x = torch.randn(B, K_in, generator=g).to(torch.bfloat16)
+    W = torch.randn(K_out, K_in, generator=g)
+    codes, alpha = tbn.tbn_quantize_pack(W.cuda())
+    n = tbn.tbn_linear_workspace_bytes(B, K_in, K_out)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda") if n else None
+    wt, al = oracle.quantize(W.numpy())
+    want, bound = oracle.linear(x.float().numpy(), wt, al)
+    for w in {None, ws}:
+        y = tbn.tbn_linear_fwd_ws(x.cuda(), codes, alpha, K_out, w, out_dtype=torch.float32)
+        assert_within(y.cpu().numpy(), want, bound, out_bf16=False, what="padded linear")
+
+
+@pytest.mark.parametrize("case", [
+    (3, 64, 28, 28, 72, 3, 3, (1, 1), (1, 1)),      # even map: runs of row pairs
+    (2, 64, 13, 11, 136, 3, 3, (1, 1), (1, 1)),     # odd: the last row and column drop
+    (7, 64, 7, 9, 64, 3, 3, (1, 1), (1, 1)),        # several images per tile, odd rows
+    (2, 40, 20, 24, 64, 3, 3, (1, 1), (1, 1)),      # padded channels
+    (1, 96, 34, 128, 24, 3, 3, (1, 1), (1, 1)),     # the widest rows that pair up
+    (2, 64, 45, 44, 64, 3, 3, (2, 2), (1, 1)),      # strided
+])
+def test_pool_of_any_width(case):
+    """AUTO pools rows of other widths than 8, 16 and 32 in the implicit
+    GEMM; naming that algorithm is refused as before."""
+    c = _case(*case, seed=sum(case[:7]))
+    K = case[4]
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    P, Q = y_orc.shape[2] // 2, y_orc.shape[3] // 2
+    want = oracle.maxpool2d_nchw(oracle.epilogue(y_orc, None, relu=True), (2, 2), (2, 2))
+    bound = bound[:, :, :2 * P, :2 * Q].reshape(-1, K, P, 2, Q, 2).max(axis=(3, 5))
+    Wl, codes, alpha = c.quantize_gpu(tbn.TBN_NHWC)
+    x = c.x.to(torch.bfloat16).permute(0, 2, 3, 1).contiguous().cuda()
+    args = (x, codes, alpha, K, case[5], case[6], case[7], case[8])
+    for dt in (torch.float32, torch.bfloat16):
+        y = tbn.tbn_conv2d_fwd(*args, out_dtype=dt, relu=True, pool=2)
+        y = y.float().cpu().permute(0, 3, 1, 2).numpy()
+        assert_within(y, want, bound, out_bf16=dt == torch.bfloat16, epilogue=True,
+                      what="any width %s" % (case,))
+    assert tbn.tbn_device_error() == 0
+    with pytest.raises(tbn.TBNError):
+        tbn.tbn_conv2d_fwd(*args, relu=True, pool=2, algo=tbn.TBN_CONV_IMPLICIT_GEMM)
