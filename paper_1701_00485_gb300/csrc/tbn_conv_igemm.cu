@@ -178,12 +178,17 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   a.R = (int)p.R; a.S = (int)p.S; a.sh = (int)p.sh; a.sw = (int)p.sw;
   a.ph = (int)p.ph; a.pw = (int)p.pw; a.P = (int)t.oP; a.Q = (int)t.oQ;
   a.im2col = t.im2col ? 1 : 0; a.iP = (int)p.P; a.iQ = (int)p.Q;
+  if (t.rowpair) {   // the convolution of the row pairs
+    a.iP /= 2;
+    a.sh = 2;
+    a.R += 1;
+  }
   a.bw = t.bw; a.bh = t.bh; a.bn = t.bn; a.tile_n = t.tile_n;
   a.tiles_q = t.tiles_q; a.tiles_p = t.tiles_p;
   a.tiles_k = ceil_div(p.K, kBM);
   const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n * a.tiles_k;
   a.ncodes = (int)(p.C * p.R * p.S);
-  a.kblocks = static_cast<int>(kblocks_of(p));
+  a.kblocks = t.rowpair ? a.R * a.S * a.C / kBK : static_cast<int>(kblocks_of(p));
   const bool split = p.ksplit > 1 && p.partial != nullptr;
   a.ksplit = split ? p.ksplit : 1;
   a.kb_per = ceil_div(a.kblocks, a.ksplit);
@@ -257,6 +262,7 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
     return tst ? launch_t<kModeS2d, 0, true, false>(p, t, a, s)
                : launch_t<kModeS2d, 0, false, false>(p, t, a, s);
   }
+  if (t.rowpair) return launch_igemm_rowpair(p, t, a, s);
   if (use_tma(p) && use_ch32(p)) {
     return launch_igemm_tma32(p, t, a, pw, tst, a.wq != nullptr, s);
   }

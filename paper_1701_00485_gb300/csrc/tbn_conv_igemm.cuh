@@ -148,6 +148,7 @@ struct IgArgs {
 struct TilePlan {
   int bw, bh, bn, T, tile_n, tiles_q, tiles_p, tiles_n;
   bool im2col;             // tiles of consecutive pixels over the whole batch
+  bool rowpair;            // two output rows' filters in the MMA's 128 rows (kModeRowPair)
   int64_t oN, oP, oQ;      // output extents that the tiles walk
 };
 
@@ -188,6 +189,13 @@ constexpr int kModePatch = 3;   // the tile's input rows are staged in shared me
 constexpr int kModeS2d = 4;     // space-to-depth input: 64-channel TMA boxes, and the
                                 // filter's K blocks decoded once per CTA into tensor memory
 constexpr int kModeTmaPad = 5;  // 64-channel TMA boxes, each tap's last one padded (C % 8 == 0)
+// Row pairs (K <= 64 filters, stride 1): MMA rows 0-63 are the filters for the
+// even output rows, rows 64-127 the same filters, one tap row later, for the
+// odd ones.  Both read the same box of input rows 2 i + r', r' = 0 .. R, so
+// R + 1 tap rows serve two output rows where one at a time takes 2 R with
+// half the MMA's rows empty; the tap row that a half does not have is a
+// block of zero weights.
+constexpr int kModeRowPair = 6;
 constexpr int kMaxResidentKB = 15;   // resident K blocks: 32 columns each beside the accumulator
 
 __host__ __device__ constexpr bool mode_gathers(int mode) {
@@ -286,6 +294,27 @@ __device__ __forceinline__ void store_out(const IgArgs& a, size_t o, float v, fl
     static_cast<__nv_bfloat16*>(a.y)[o] = __float2bfloat16_rn(v);
   else
     static_cast<float*>(a.y)[o] = v;
+}
+
+// Row pairs: sum of x W~/2 over the taps of MMA row m (filter m & 63, row
+// parity m >> 6) at pixel f of the row pairs, in fp32.
+__device__ __noinline__ float rowpair_sum(const IgArgs& a, int m, int f) {
+  const int row = f / a.iQ, n = row / a.iP;
+  const int q = f - row * a.iQ, p = 2 * (row - n * a.iP) + (m >> 6);
+  const uint32_t* codes = a.codes + static_cast<size_t>(m & 63) * a.wpf;
+  float acc = 0.0f;
+  for (int r = 0; r < a.R - 1; ++r)
+    for (int s = 0; s < a.S; ++s) {
+      const int h = p - a.ph + r, w = q * a.sw - a.pw + s;
+      if (h < 0 || h >= a.H || w < 0 || w >= a.W) continue;
+      const __nv_bfloat16* x = a.x + ((static_cast<int64_t>(n) * a.H + h) * a.W + w) * a.C;
+      for (int c = 0; c < a.C; ++c) {
+        const int i = (r * a.S + s) * a.C + c;
+        acc = fmaf(__bfloat162float(x[c]), 0.5f * code_value(code_field(__ldg(codes + (i >> 4)), i & 15)),
+                   acc);
+      }
+    }
+  return acc;
 }
 
 // kPoolBW: 0 = no pool; 8, 16, 32 = fused 2x2/2 max pool for tiles of whole
@@ -415,6 +444,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
   constexpr bool kPatch = kMode == kModePatch;
   constexpr bool kS2d = kMode == kModeS2d;
   constexpr bool kPad = kMode == kModeTmaPad;
+  constexpr bool kRowPair = kMode == kModeRowPair;
   constexpr int kSt = stages_for(kMode);   // ring stages
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte aligned by pointer arithmetic on the shared array, so that the
@@ -996,6 +1026,11 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     // where the row has them (kb < kb_lim)
     int t_ld = blockIdx.x, kb_ld = 0, kb_end = 0, kb_lim = 0;
     const int kb_words = (a.wpf - 2 * half + 3) / 4;   // K blocks whose two words begin in the row
+    // row pairs: the upper 64 rows (two of the four sub-partitions) run one
+    // tap row behind; K blocks before and after a half's taps are zero
+    const int behind = kRowPair && sub >= 2 ? a.S * (a.C / kBK) : 0;
+    const int kb_taps = kRowPair ? (a.R - 1) * a.S * (a.C / kBK) : 0;
+    int kb_st = 0;   // row pairs: the K block (within its tile) next to be stored
     const uint32_t* cp = a.codes;
     // padded mode: this half block's first code, and channels left in its tap
     const int tap_blocks = (a.C + kBK - 1) / kBK;
@@ -1004,8 +1039,15 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const TileCoord tc = tile_coord(a, t_ld < a.tiles ? t_ld : 0);
       kb_ld = tc.kb0;
       kb_end = tc.kb1;
-      const int k = tc.ktile * kBM + m;
+      const int k = kRowPair ? (m & 63) : tc.ktile * kBM + m;
       const bool in = t_ld < a.tiles && k < a.K;
+      if constexpr (kRowPair) {
+        kb_lim = in ? kb_taps : 0;
+        kb_ld = -behind;
+        kb_end = KB - behind;
+        cp = a.codes + static_cast<int64_t>(in ? k : 0) * a.wpf + 4 * kb_ld + 2 * half;
+        return;
+      }
       if constexpr (kPad) {
         const int tap = kb_ld / tap_blocks, cb = kb_ld - tap * tap_blocks;
         ch_left = a.C - kBK * cb;
@@ -1048,7 +1090,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         }
         return r;
       }
-      if (kb_ld < kb_lim) {
+      if (kb_ld < kb_lim && (!kRowPair || kb_ld >= 0)) {
         // written by this launch's prologue when fused: ordinary (L1-cached,
         // coherent) loads after the grid barrier's acquire then, not the
         // read-only path, which assumes data constant for the whole launch
@@ -1082,6 +1124,19 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       word_to_bf16x2(q0.y, v0 + 8, pm);
       word_to_bf16x2(q1.x, v1 + 0, pm);
       word_to_bf16x2(q1.y, v1 + 8, pm);
+      if constexpr (kRowPair) {
+        // warp-uniform: a whole half's K block is taps or zeros
+        const auto zero = [&](uint32_t* v) {
+          const int kb = kb_st - behind;
+          if (kb < 0 || kb >= kb_taps) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = 0u;
+          }
+          if (++kb_st == KB) kb_st = 0;
+        };
+        zero(v0);
+        if (two) zero(v1);
+      }
       q0 = q2;
       q1 = q3;
       q2 = next_codes();
@@ -1134,7 +1189,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const uint32_t apar = (a.acc2 ? (tiles_done >> 1) : tiles_done) & 1u;
       const uint32_t acc_b = acc_tmem + ab * kAcc2Cols;
       const uint32_t acc = acc_b + lane_off;
-      const int k = tc.ktile * kBM + m;
+      const int k = kRowPair ? (m & 63) : tc.ktile * kBM + m;
       const bool kvalid = k < a.K;
       const float a2 = kvalid ? 2.0f * (kFuse ? __ldca(a.alpha + k) : __ldg(a.alpha + k)) : 0.0f;
       if (kTmaStore) {
@@ -1144,10 +1199,16 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         if (ok && a.residual && elected) {
           // the residual box, in the staging tile's own layout (two swizzled
           // halves of 64 filters), lands where the outputs will be staged
-          const bool both = tc.ktile * kBM + kBM / 2 < a.K;
+          const bool both = kRowPair || tc.ktile * kBM + kBM / 2 < a.K;
           mbar_arrive_expect_tx(&ctl->res_full, both ? 2 * res_half_bytes : res_half_bytes);
-          tma_load_4d(stage, &tmap_res, &ctl->res_full, tc.ktile * kBM, tc.q0, tc.p0, tc.n0);
-          if (both)
+          if constexpr (kRowPair) {   // (filter, column, row parity, row pair)
+            tma_load_4d(stage, &tmap_res, &ctl->res_full, 0, 0, 0, tc.p0);
+            tma_load_4d(reinterpret_cast<uint8_t*>(stage) + 32768, &tmap_res, &ctl->res_full, 0, 0,
+                        1, tc.p0);
+          } else {
+            tma_load_4d(stage, &tmap_res, &ctl->res_full, tc.ktile * kBM, tc.q0, tc.p0, tc.n0);
+          }
+          if (!kRowPair && both)
             tma_load_4d(reinterpret_cast<uint8_t*>(stage) + 32768, &tmap_res, &ctl->res_full,
                         tc.ktile * kBM + kBM / 2, tc.q0, tc.p0, tc.n0);
         }
@@ -1180,7 +1241,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         for (int lg = 0; lg < 2; ++lg) {
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            const int kk = tc.ktile * kBM + sub * 32 + lg * 16 + u * 8 + fr;
+            const int mm = sub * 32 + lg * 16 + u * 8 + fr;
+            const int kk = kRowPair ? (mm & 63) : tc.ktile * kBM + mm;
             a2f[lg][u] = kk < a.K ? 2.0f * (kFuse ? __ldca(a.alpha + kk) : __ldg(a.alpha + kk)) : 0.0f;
           }
         }
@@ -1198,6 +1260,26 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
           if (j == c_end - 1) {
             tc_fence_before_sync();
             mbar_arrive(&ctl->acc_empty[ab]);
+          }
+          if constexpr (kRowPair) {
+            // a zero weight times an infinite or NaN input of the other row's
+            // taps is NaN: such sums are recomputed from their own taps
+            float z = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              z = fmaf(__uint_as_float(v[0][i]), 0.0f, fmaf(__uint_as_float(v[1][i]), 0.0f, z));
+            if (z != 0.0f) {   // NaN
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                const int lg = i >> 4, e = i & 15;
+                const int mm = sub * 32 + lg * 16 + ((e >> 1) & 1) * 8 + fr;
+                const int px = 32 * j + 8 * (e >> 2) + 2 * (lane & 3) + (e & 1);
+                const int f = tc.p0 * a.Q + px;   // pixel of the row pairs
+                if ((mm & 63) < a.K && px < a.bw * a.bh && f < a.P * a.Q &&
+                    !(fabsf(__uint_as_float(v[lg][e])) <= 3.402823466e38f))
+                  v[lg][e] = __float_as_uint(rowpair_sum(a, mm, f));
+              }
+            }
           }
 #pragma unroll
           for (int lg = 0; lg < 2; ++lg) {
@@ -1396,6 +1478,9 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         if (elected && ok) {
           if (kPoolBW) {
             tma_store_4d(&tmap_y, stage, tc.ktile * kBM, 0, tc.p0 / 2, tc.n0);
+          } else if constexpr (kRowPair) {
+            tma_store_4d(&tmap_y, stage, 0, 0, 0, tc.p0);
+            tma_store_4d(&tmap_y, reinterpret_cast<uint8_t*>(stage) + 32768, 0, 0, 1, tc.p0);
           } else {
             tma_store_4d(&tmap_y, stage, tc.ktile * kBM, tc.q0, tc.p0, tc.n0);
             if (tc.ktile * kBM + kBM / 2 < a.K)
@@ -1468,7 +1553,7 @@ inline TilePlan plan_tiles(const ConvProblem& p) {
   t.tiles_n = ceil_div(p.N, t.bn);
   t.T = t.bw * t.bh * t.bn;
   t.tile_n = ((t.T + 15) / 16) * 16;
-  t.im2col = false;
+  t.im2col = t.rowpair = false;
   t.oN = p.N;
   t.oP = p.P;
   t.oQ = p.Q;
@@ -1496,7 +1581,8 @@ inline double plan_cost(const ConvProblem& p, const TilePlan& t, bool resident, 
   const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n *
                         ((p.K + kBM - 1) / kBM);
   const double waves = static_cast<double>((tiles + sms - 1) / sms);
-  const double kb = static_cast<double>(kblocks_of(p));
+  const double kb = t.rowpair ? static_cast<double>((p.R + 1) * p.S * p.C / kBK)
+                              : static_cast<double>(kblocks_of(p));
   const bool acc2 = !resident && t.tile_n <= kAcc2Cols;
   return waves * (kb * (215.0 + 0.25 * t.tile_n) + (acc2 ? 900.0 : 1700.0));
 }
@@ -1509,6 +1595,21 @@ inline bool im2col_ok(const ConvProblem& p) {
   return tma_fed(p) && p.R <= 128 && p.S <= 128 && p.ph <= 127 && p.pw <= 127 &&
          p.N * p.P * p.Q <= (int64_t(1) << 30) && p.N * p.H * p.W * p.C * 2 >= 131072 &&
          get_encode_im2col() != nullptr;
+}
+
+inline bool use_tma_store(const ConvProblem& p) {
+  return p.ydt == TBN_BF16 && p.K % 8 == 0 && is_aligned(p.y, 16) &&
+         (!p.residual || is_aligned(p.residual, 16));
+}
+
+// Whether the layer can run on row pairs (kModeRowPair): at most 64 filters,
+// stride 1 down the rows, an even number of output rows of at most a tile's
+// width, whole 64-channel boxes, and the staged bf16 epilogue.  It pays for
+// filters of several rows: 3 x 3 over 64 channels takes 12 K blocks for two
+// output rows instead of 18 (56 x 56, batch 64, with shortcut: see plan_conv).
+inline bool rowpair_ok(const ConvProblem& p) {
+  return p.C % kBK == 0 && p.K <= kBM / 2 && p.sh == 1 && p.sw <= 2 && p.P % 2 == 0 && p.R >= 2 &&
+         p.R < 128 && p.Q <= kMaxTileN && !p.pool && p.wq == nullptr && use_tma_store(p);
 }
 
 // The tile plan of a launch.  Gathering modes and split K: plan_tiles.  TMA
@@ -1549,6 +1650,21 @@ inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
         t.tiles_q = ceil_div(t.oQ, T);
         consider(t);
       }
+      if (rowpair_ok(p) && !resident) {
+        // runs of whole row pairs
+        t.rowpair = true;
+        t.oP = p.N * p.P / 2;
+        t.oQ = p.Q;
+        t.bw = static_cast<int>(p.Q);
+        t.tiles_q = 1;
+        for (int rows = 1; rows * t.bw <= kMaxTileN; ++rows) {
+          t.bh = rows;
+          t.T = rows * t.bw;
+          t.tile_n = ((t.T + 15) / 16) * 16;
+          t.tiles_p = ceil_div(t.oP, rows);
+          consider(t);
+        }
+      }
     } else if (p.P % 2 == 0 && best.tiles_q == 1) {
       // row pairs of all images in sequence (P even: none crosses images)
       t.oP = p.N * p.P;
@@ -1576,23 +1692,29 @@ inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
   return best;
 }
 
-inline bool use_tma_store(const ConvProblem& p) {
-  return p.ydt == TBN_BF16 && p.K % 8 == 0 && is_aligned(p.y, 16) &&
-         (!p.residual || is_aligned(p.residual, 16));
-}
-
 // Output map: box = 128 filters x the tile's pixels (no swizzle), or with
 // `halves`, 64 filters (128 bytes) per box with the 128-byte swizzle (the
 // staging layout of the fragment epilogue, two stores per tile).
 inline CUresult encode_out_map(CUtensorMap* m, const void* base, const ConvProblem& p, const TilePlan& t,
                         int pool, bool halves = false) {
+  const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
+  if (t.rowpair) {
+    // (filter, column, row parity, row pair)
+    const cuuint64_t gd[4] = {(cuuint64_t)p.K, (cuuint64_t)t.oQ, 2u, (cuuint64_t)t.oP};
+    const cuuint64_t gs[3] = {(cuuint64_t)(p.K * 2), (cuuint64_t)(t.oQ * p.K * 2),
+                              (cuuint64_t)(2 * t.oQ * p.K * 2)};
+    const cuuint32_t bx[4] = {(cuuint32_t)(kBM / 2), (cuuint32_t)t.bw, 1u, (cuuint32_t)t.bh};
+    return get_encode_tiled()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), gd,
+                              gs, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  }
   const int64_t Po = pool ? t.oP / 2 : t.oP, Qo = pool ? t.oQ / 2 : t.oQ;
   const cuuint64_t gdim[4] = {(cuuint64_t)p.K, (cuuint64_t)Qo, (cuuint64_t)Po, (cuuint64_t)t.oN};
   const cuuint64_t gstride[3] = {(cuuint64_t)(p.K * 2), (cuuint64_t)(Qo * p.K * 2),
                                  (cuuint64_t)(Po * Qo * p.K * 2)};
   const cuuint32_t box[4] = {(cuuint32_t)(halves ? kBM / 2 : kBM), (cuuint32_t)(pool ? t.bw / 2 : t.bw),
                              (cuuint32_t)(pool ? t.bh / 2 : t.bh), (cuuint32_t)t.bn};
-  const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
   return get_encode_tiled()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), gdim,
                             gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             halves ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1611,14 +1733,16 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
     const cuuint64_t gdim[4] = {(cuuint64_t)p.C, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.N};
     const cuuint64_t gstride[3] = {(cuuint64_t)(p.C * 2), (cuuint64_t)(p.W * p.C * 2),
                                    (cuuint64_t)(p.H * p.W * p.C * 2)};
-    const cuuint32_t estr[4] = {1u, (cuuint32_t)p.sw, (cuuint32_t)p.sh, 1u};
+    // row pairs: base rows two apart, R + 1 tap rows
+    const int rp = t.rowpair ? 1 : 0;
+    const cuuint32_t estr[4] = {1u, (cuuint32_t)p.sw, (cuuint32_t)(p.sh + rp), 1u};
     const cuuint32_t channels = kCh32 ? kBK / 2 : kBK;
     const CUtensorMapSwizzle swizzle = kCh32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
     CUresult cr;
     if (t.im2col) {
       // base positions [-pad, size - 1 + pad - (kernel - 1)] in steps of the stride
       const int lower[2] = {-(int)p.pw, -(int)p.ph};
-      const int upper[2] = {(int)(p.pw - (p.S - 1)), (int)(p.ph - (p.R - 1))};
+      const int upper[2] = {(int)(p.pw - (p.S - 1)), (int)(p.ph - (p.R - 1)) - rp};
       cr = get_encode_im2col()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
                                const_cast<void*>(p.x), gdim, gstride, lower, upper, channels,
                                (cuuint32_t)t.T, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
@@ -1715,5 +1839,7 @@ tbn_status launch_igemm_tma32(const ConvProblem& p, const TilePlan& t, IgArgs& a
                               bool tma_store, bool fuse, cudaStream_t s);
 tbn_status launch_igemm_pad(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
                             bool tma_store, cudaStream_t s);
+tbn_status launch_igemm_rowpair(const ConvProblem& p, const TilePlan& t, IgArgs& a,
+                                cudaStream_t s);
 
 }  // namespace tbn

@@ -152,3 +152,47 @@ def test_pool_of_any_width(case):
     assert tbn.tbn_device_error() == 0
     with pytest.raises(tbn.TBNError):
         tbn.tbn_conv2d_fwd(*args, relu=True, pool=2, algo=tbn.TBN_CONV_IMPLICIT_GEMM)
+
+
+ROW_PAIRS = [
+    # N, C, H, W, K, R, S, stride, pad: at most 64 filters, an even number of
+    # output rows, inputs of at least 128 KiB
+    (6, 64, 56, 56, 64, 3, 3, (1, 1), (1, 1)),      # 64 filters, several tiles per CTA
+    (9, 128, 14, 17, 40, 3, 3, (1, 1), (1, 1)),     # ragged filters, odd width
+    (5, 64, 21, 24, 8, 2, 3, (1, 2), (0, 1)),       # R = 2, column stride 2
+    (3, 64, 18, 60, 64, 5, 5, (1, 1), (2, 2)),
+]
+
+
+@pytest.mark.parametrize("case", ROW_PAIRS)
+def test_row_pairs(case):
+    c = _case(*case, seed=sum(case[:7]))
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    assert y_orc.shape[2] % 2 == 0
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16)
+    assert_within(y, y_orc, bound, out_bf16=True, what="row pairs %s" % (case,))
+    res = torch.randn(*y_orc.shape, generator=inputs.generator(3)).to(torch.bfloat16)
+    want = oracle.epilogue(y_orc, res.float().numpy(), relu=True)
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16, relu=True, residual=res)
+    assert_within(y, want, bound, out_bf16=True, epilogue=True, what="row pairs epi %s" % (case,))
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+def test_row_pairs_not_finite(value):
+    """An infinite or NaN input reaches the outputs whose taps read it and no
+    others, although both rows of a pair multiply it."""
+    g = inputs.generator(11)
+    x = torch.randn(6, 64, 20, 20, generator=g)
+    x[2, 5, 7, 9] = value
+    x[4, 60, 0, 0] = value
+    c = ConvCase(x, inputs.normal((48, 64, 3, 3), 1.2, g), (1, 1), (1, 1))
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16)
+    wt, al = oracle.quantize(c.W.reshape(48, -1).numpy())
+    w = torch.from_numpy((wt * al[:, None]).reshape(c.W.shape))
+    ref = torch.nn.functional.conv2d(x.to(torch.bfloat16).double(), w.double(), padding=1).numpy()
+    fin = torch.isfinite(torch.from_numpy(ref)).numpy()
+    assert 100 < (~fin).sum() < 2000
+    assert (torch.isnan(torch.from_numpy(y)).numpy() == torch.isnan(torch.from_numpy(ref)).numpy()).all()
+    inf = ~fin & ~torch.isnan(torch.from_numpy(ref)).numpy()
+    assert (y[inf] == ref[inf]).all()
+    assert (abs(y[fin] - ref[fin]) <= 2.0 ** -7 * abs(ref[fin]) + 1e-3).all()
