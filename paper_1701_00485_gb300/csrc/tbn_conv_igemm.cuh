@@ -209,6 +209,14 @@ __host__ __device__ constexpr int producer_warps(int mode) {
   return mode == kModePatch ? kPatchWarps : (mode == kModeGather ? kGatherWarps : 0);
 }
 
+// Epilogue warps of a mode: in space-to-depth mode the expanders, done with
+// the filter after the first tile, join them (the one accumulator is held for
+// half as long: AlexNet conv1 at batch 256, 9 K blocks per tile, spent 30% of
+// its time waiting for it).
+__host__ __device__ constexpr int epi_warps(int mode) {
+  return mode == kModeS2d ? kEpiWarps + kExpWarps : kEpiWarps;
+}
+
 template <int kMode>
 constexpr int threads_for() {
   return 32 * (kFirstGatherWarp +
@@ -472,7 +480,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     mbar_init(&ctl->patch_full[1], 1);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->acc_full[b], 1);
-      mbar_init(&ctl->acc_empty[b], 32 * kEpiWarps);
+      mbar_init(&ctl->acc_empty[b], 32 * epi_warps(kMode));
     }
     mbar_init(&ctl->res_full, 1);
     mbar_init(&ctl->mma_drain, 1);
@@ -1164,14 +1172,17 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       if (two) mbar_arrive(&ctl->full[s1]);
     }
     }
-  } else if (warp >= kFirstEpiWarp && warp < kFirstEpiWarp + kEpiWarps) {
+  }
+  if ((warp >= kFirstEpiWarp && warp < kFirstEpiWarp + kEpiWarps) ||
+      (kS2d && warp >= kFirstExpWarp && warp < kFirstExpWarp + kExpWarps)) {
     // ================= epilogue =================
-    // Two warps per TMEM sub-partition, each reading half of the columns.
+    // kParts warps per TMEM sub-partition, each reading a part of the columns.
+    constexpr int kParts = epi_warps(kMode) / 4;
     const int sub = warp & 3;
-    const int half = (warp - kFirstEpiWarp) >> 2;
+    const int half = warp >= kFirstEpiWarp ? (warp - kFirstEpiWarp) >> 2
+                                           : kEpiWarps / 4 + ((warp - kFirstExpWarp) >> 2);
     const int m = sub * 32 + lane;
-    const int et = threadIdx.x - 32 * kFirstEpiWarp;   // 0..255
-    const bool elected = et == 0;
+    const bool elected = threadIdx.x == 32 * kFirstEpiWarp;
     const uint32_t lane_off = static_cast<uint32_t>(sub * 32) << 16;
     const int Po = kPoolBW ? a.P / 2 : a.P;
     const int Qo = kPoolBW ? a.Q / 2 : a.Q;
@@ -1195,7 +1206,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       if (kTmaStore) {
         // the previous tile's store must have finished reading the staging tile
         if (elected) bulk_wait_group_read<0>();
-        named_barrier_sync(1, 32 * kEpiWarps);
+        named_barrier_sync(1, 32 * epi_warps(kMode));
         if (ok && a.residual && elected) {
           // the residual box, in the staging tile's own layout (two swizzled
           // halves of 64 filters), lands where the outputs will be staged
@@ -1233,17 +1244,19 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         // per value took a 64-filter 56x56 layer at batch 128 from 49 to
         // 103 us; this way the residual costs 51.4 MB more of reads, no more.)
         const int nchunks = (a.tile_n + 31) / 32;
-        const int c_begin = half ? (nchunks + 1) / 2 : 0;
-        const int c_end = half ? nchunks : (nchunks + 1) / 2;
+        const int c_begin = (nchunks * half + kParts - 1) / kParts;
+        const int c_end = (nchunks * (half + 1) + kParts - 1) / kParts;
         const int fr = lane >> 2;                       // fragment row within 8
-        float a2f[2][2];
+        uint64_t a2f[2][2];   // 2 alpha, twice
 #pragma unroll
         for (int lg = 0; lg < 2; ++lg) {
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             const int mm = sub * 32 + lg * 16 + u * 8 + fr;
             const int kk = kRowPair ? (mm & 63) : tc.ktile * kBM + mm;
-            a2f[lg][u] = kk < a.K ? 2.0f * (kFuse ? __ldca(a.alpha + kk) : __ldg(a.alpha + kk)) : 0.0f;
+            const float s2 =
+                kk < a.K ? 2.0f * (kFuse ? __ldca(a.alpha + kk) : __ldg(a.alpha + kk)) : 0.0f;
+            a2f[lg][u] = f32x2(__float_as_uint(s2), __float_as_uint(s2));
           }
         }
         // this lane's stmatrix row address pieces: matrix mi = lane / 8, row = lane % 8
@@ -1299,26 +1312,22 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
                 ldmatrix_x4_trans(addr[bp], pk[4 * bp + 0], pk[4 * bp + 1], pk[4 * bp + 2],
                                   pk[4 * bp + 3]);
             }
+            // pk[2b], pk[2b + 1]: pixels 2 (lane % 4) + 0/1 of block b, filters fr
+            // and fr + 8.  Two pixels per instruction: this loop is what holds
+            // the accumulator of a short filter's tile.
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-              float y0 = a2f[lg][0] * __uint_as_float(v[lg][4 * b + 0]);
-              float y1 = a2f[lg][0] * __uint_as_float(v[lg][4 * b + 1]);
-              float y2 = a2f[lg][1] * __uint_as_float(v[lg][4 * b + 2]);
-              float y3 = a2f[lg][1] * __uint_as_float(v[lg][4 * b + 3]);
-              if (a.residual) {   // bf16 pairs, low half first
-                y0 += __uint_as_float(pk[2 * b] << 16);
-                y1 += __uint_as_float(pk[2 * b] & 0xFFFF0000u);
-                y2 += __uint_as_float(pk[2 * b + 1] << 16);
-                y3 += __uint_as_float(pk[2 * b + 1] & 0xFFFF0000u);
-              }
-              if (a.relu) {
-                y0 = fmaxf(y0, 0.0f);
-                y1 = fmaxf(y1, 0.0f);
-                y2 = fmaxf(y2, 0.0f);
-                y3 = fmaxf(y3, 0.0f);
-              }
-              pk[2 * b] = pack_bf16x2(y0, y1);       // filters fr, pixels 2(i%4) + 0/1
-              pk[2 * b + 1] = pack_bf16x2(y2, y3);   // filters fr + 8
+            for (int e = 0; e < 8; ++e) {
+              const uint64_t acc2x = f32x2(v[lg][2 * e], v[lg][2 * e + 1]);
+              const uint64_t y =
+                  a.residual ? fma_f32x2(a2f[lg][e & 1], acc2x,
+                                         f32x2(pk[e] << 16, pk[e] & 0xFFFF0000u))
+                             : mul_f32x2(a2f[lg][e & 1], acc2x);
+              pk[e] = pack_bf16x2(__uint_as_float(static_cast<uint32_t>(y)),
+                                  __uint_as_float(static_cast<uint32_t>(y >> 32)));
+            }
+            if (a.relu) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) pk[e] = relu_bf16x2(pk[e]);
             }
 #pragma unroll
             for (int bp = 0; bp < 2; ++bp)
@@ -1333,8 +1342,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       } else if constexpr (kPoolBW == 0) {
         const int T = a.bw * a.bh * a.bn;
         const int nchunks = (a.tile_n + 31) / 32;
-        const int c_begin = half ? (nchunks + 1) / 2 : 0;
-        const int c_end = half ? nchunks : (nchunks + 1) / 2;
+        const int c_begin = (nchunks * half + kParts - 1) / kParts;
+        const int c_end = (nchunks * (half + 1) + kParts - 1) / kParts;
         // direct-store path: pixel of chunk c_begin walked in column order
         int px0 = 32 * c_begin;
         int wi = px0 % a.bw, hi = (px0 / a.bw) % a.bh, ni = px0 / (a.bw * a.bh);
@@ -1355,6 +1364,23 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
             for (int i = 0; i < 32; ++i)
               if (kvalid && 32 * j + i < T && tc.n0 + 32 * j + i < a.N)
                 dst[static_cast<size_t>(i) * a.K] = __uint_as_float(v[i]);
+          } else if (a.bh * a.bn == 1 && a.P * a.N == 1) {
+            // a run of pixels: outputs K apart from the tile's first pixel on
+            const int left = min(T, a.Q - tc.q0) - 32 * j;   // pixels of this chunk and after
+            const size_t o0 = static_cast<size_t>(tc.q0 + 32 * j) * a.K + k;
+#pragma unroll
+            for (int i0 = 0; i0 < 32; i0 += 8) {
+              float res[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                res[i] = a.residual && kvalid && i0 + i < left
+                             ? load_residual(a, o0 + static_cast<size_t>(i0 + i) * a.K) : 0.0f;
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                if (kvalid && i0 + i < left)
+                  store_out(a, o0 + static_cast<size_t>(i0 + i) * a.K,
+                            a2 * __uint_as_float(v[i0 + i]), res[i]);
+            }
           } else {
             // eight pixels at a time: their residuals are all requested before
             // the first output is stored (a load behind each store, which may
@@ -1474,7 +1500,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       }
       if (kTmaStore) {
         fence_proxy_async_smem();   // staged values -> visible to the TMA store
-        named_barrier_sync(1, 32 * kEpiWarps);
+        named_barrier_sync(1, 32 * epi_warps(kMode));
         if (elected && ok) {
           if (kPoolBW) {
             tma_store_4d(&tmap_y, stage, tc.ktile * kBM, 0, tc.p0 / 2, tc.n0);

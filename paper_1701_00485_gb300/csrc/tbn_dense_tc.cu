@@ -104,22 +104,6 @@ struct alignas(16) Ctl {
   int abort;
 };
 
-// Two fp32 additions / multiply-adds in one instruction, each rounded as by
-// itself.
-__device__ __forceinline__ uint64_t f32x2(uint32_t lo, uint32_t hi) {
-  return static_cast<uint64_t>(lo) | (static_cast<uint64_t>(hi) << 32);
-}
-__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // One output tap by tap, for results that are not finite.
 __device__ __noinline__ float dense_by_taps(const Args& a, int n, int k, int pix) {
   const int p = pix / a.Q, q = pix - p * a.Q;
