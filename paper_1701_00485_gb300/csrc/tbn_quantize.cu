@@ -229,11 +229,17 @@ __device__ bool task_stream(const StreamTask& t, const StreamTask* nxt, QShared&
       for (int u = 0; u < kChunkWords / kThreads; ++u) {
         const int w = threadIdx.x + u * kThreads;
         if (w >= wn) break;
+        // a word's four 16-byte quarters, starting with a different one in
+        // every other lane: words are 64 bytes apart, so the same quarter of
+        // eight lanes lies on two sets of four banks, four different ones on
+        // all of them (the reads took 4 x their cycles, half of the kernel's
+        // time at 8192 x 8192)
         float v[16];
         const float4* q4 = reinterpret_cast<const float4*>(chunk + 16 * w);
+        const int rot = (threadIdx.x >> 1) & 3;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const float4 t4 = q4[q];
+          const float4 t4 = q4[(q + rot) & 3];
           v[4 * q + 0] = t4.x;
           v[4 * q + 1] = t4.y;
           v[4 * q + 2] = t4.z;
@@ -242,7 +248,11 @@ __device__ bool task_stream(const StreamTask& t, const StreamTask* nxt, QShared&
         uint32_t word;
         float sum;
         int c2;
+        // the sum adds quarters 0 + 2 and 1 + 3 first, so it is the same for
+        // every rotation; each byte's four bit pairs turn back by `rot` pairs
         encode16(v, 16, word, sum, c2);
+        const uint32_t up = 0x01010101u * ((0xFFu << (2 * rot)) & 0xFFu);
+        word = ((word << (2 * rot)) & up) | ((word >> (8 - 2 * rot)) & ~up);
         out[w0 + w] = word;   // the task's words are contiguous in the codes array
         sh.sum[w0 + w] = sum;
         sh.cnt[w0 + w] = c2;
