@@ -2,7 +2,8 @@
 // every layout / dtype / stride / padding, plus the network glue kernels
 // (NHWC max pooling with optional padding, NCHW -> NHWC with channel padding).
 //
-// Direct convolution: a CTA computes 128 output pixels x 32 filters.  The
+// Direct convolution: a CTA computes 128 output pixels x 32 filters (8 where
+// that would leave SMs without a CTA).  The
 // filters' codes are decoded once per CTA into shared memory as fp32 W~ (a
 // chunk of taps at a time, tap-major so that all threads read the same
 // 32 weights -- a broadcast); each thread owns one pixel, walks the taps in
@@ -25,6 +26,7 @@ namespace {
 
 constexpr int kPix = 128;    // pixels (threads) per CTA
 constexpr int kFilt = 32;    // filters per CTA
+constexpr int kAhead = 8;    // taps whose activations are requested together
 constexpr int kTapChunk = 128;
 
 template <typename T>
@@ -57,13 +59,17 @@ struct DirectArgs {
   int relu;
 };
 
-// kWin = 1: one conv output per thread, 32 filters.  kWin = 4: one 2x2-pooled
+// kWin = 1: one conv output per thread, kF filters.  kWin = 4: one 2x2-pooled
 // output per thread (four conv outputs, max after ReLU), 8 filters.
 // kLayout (tbn_layout): x is NHWC only for TBN_NHWC; the codes are in
 // (r, s, c) order and y is NHWC for TBN_NHWC and TBN_NCHW_NHWC.
-template <typename TX, typename TY, int kLayout, int kWin>
+//
+// Bound: the tap chain.  A thread's activations come one per tap, so they are
+// requested kAhead taps at a time (one load behind each tap's FMAs cost a
+// cache latency per tap: 2 images of 20 x 26 x 24 through 15 filters of 5 x 5,
+// 500 taps, 87 us), and few pixels spread over more CTAs of fewer filters.
+template <typename TX, typename TY, int kLayout, int kWin, int kF>
 __global__ void __launch_bounds__(kPix) conv_direct_kernel(const DirectArgs a) {
-  constexpr int kF = kWin == 1 ? kFilt : 8;
   constexpr bool kXNhwc = kLayout == TBN_NHWC, kRsc = kLayout != TBN_NCHW;
   constexpr bool kYNhwc = kLayout != TBN_NCHW;
   __shared__ __align__(16) float s_w[kTapChunk][kF];
@@ -76,9 +82,18 @@ __global__ void __launch_bounds__(kPix) conv_direct_kernel(const DirectArgs a) {
   const int64_t k0 = static_cast<int64_t>(blockIdx.y) * kF;
   const bool active = pix < npix;
   const int64_t pc = active ? pix : 0;
-  const int64_t b = pc / (a.Po * a.Qo);
-  const int64_t po = (pc / a.Qo) % a.Po;
-  const int64_t qo = pc % a.Qo;
+  int64_t b, po, qo;
+  if (npix < (int64_t(1) << 31)) {   // 32-bit divisions
+    const uint32_t row = static_cast<uint32_t>(pc) / static_cast<uint32_t>(a.Qo);
+    const uint32_t im = row / static_cast<uint32_t>(a.Po);
+    b = im;
+    po = row - im * static_cast<uint32_t>(a.Po);
+    qo = static_cast<uint32_t>(pc) - row * static_cast<uint32_t>(a.Qo);
+  } else {
+    b = pc / (a.Po * a.Qo);
+    po = (pc / a.Qo) % a.Po;
+    qo = pc % a.Qo;
+  }
   int h0[kWin], w0[kWin];
   int64_t base[kWin];
 #pragma unroll
@@ -116,31 +131,56 @@ __global__ void __launch_bounds__(kPix) conv_direct_kernel(const DirectArgs a) {
       s_w[t][f] = v;
     }
     for (int t = threadIdx.x; t < tc; t += kPix) {
-      const int64_t ti = t0 + t;
-      int64_t c, r, s;
+      // C R S and C H W are below 2^31
+      const uint32_t ti = static_cast<uint32_t>(t0 + t), S = static_cast<uint32_t>(a.S);
+      uint32_t c, r, s;
       if (kRsc) {
-        r = ti / (a.S * a.C);
-        s = (ti / a.C) % a.S;
-        c = ti % a.C;
+        const uint32_t tap = ti / static_cast<uint32_t>(a.C);
+        c = ti - tap * static_cast<uint32_t>(a.C);
+        r = tap / S;
+        s = tap - r * S;
       } else {
-        c = ti / (a.R * a.S);
-        r = (ti / a.S) % a.R;
-        s = ti % a.S;
+        const uint32_t row = ti / S;
+        s = ti - row * S;
+        c = row / static_cast<uint32_t>(a.R);
+        r = row - c * static_cast<uint32_t>(a.R);
       }
-      s_off[t] = static_cast<int32_t>(kXNhwc ? (r * a.W + s) * a.C + c : (c * a.H + r) * a.W + s);
+      s_off[t] = static_cast<int32_t>(kXNhwc ? (int64_t(r) * a.W + s) * a.C + c
+                                             : (int64_t(c) * a.H + r) * a.W + s);
       s_rs[t] = static_cast<int32_t>((r << 16) | s);
     }
     __syncthreads();
     if (active) {
-      for (int t = 0; t < tc; ++t) {
+      const auto load = [&](int t, int wdx) {
         const int32_t rs = s_rs[t];
-        const int off = s_off[t];
+        const int h = h0[wdx] + (rs >> 16), w = w0[wdx] + (rs & 0xFFFF);
+        return h >= 0 && h < H && w >= 0 && w < W ? to_f32<TX>(x[base[wdx] + s_off[t]]) : 0.0f;
+      };
+      int t = 0;
+      if constexpr (kWin == 1) {
+        for (; t + kAhead <= tc; t += kAhead) {
+          float xv[kAhead];
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u) xv[u] = load(t + u, 0);
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u) {
+            const float4* wr = reinterpret_cast<const float4*>(&s_w[t + u][0]);
+#pragma unroll
+            for (int f4 = 0; f4 < kF / 4; ++f4) {
+              const float4 wv = wr[f4];
+              acc[0][4 * f4 + 0] = fmaf(xv[u], wv.x, acc[0][4 * f4 + 0]);
+              acc[0][4 * f4 + 1] = fmaf(xv[u], wv.y, acc[0][4 * f4 + 1]);
+              acc[0][4 * f4 + 2] = fmaf(xv[u], wv.z, acc[0][4 * f4 + 2]);
+              acc[0][4 * f4 + 3] = fmaf(xv[u], wv.w, acc[0][4 * f4 + 3]);
+            }
+          }
+        }
+      }
+      for (; t < tc; ++t) {
         const float4* wr = reinterpret_cast<const float4*>(&s_w[t][0]);
 #pragma unroll
         for (int wdx = 0; wdx < kWin; ++wdx) {
-          const int h = h0[wdx] + (rs >> 16), w = w0[wdx] + (rs & 0xFFFF);
-          float xv = 0.0f;
-          if (h >= 0 && h < H && w >= 0 && w < W) xv = to_f32<TX>(x[base[wdx] + off]);
+          const float xv = load(t, wdx);
 #pragma unroll
           for (int f4 = 0; f4 < kF / 4; ++f4) {
             const float4 wv = wr[f4];
@@ -175,9 +215,8 @@ __global__ void __launch_bounds__(kPix) conv_direct_kernel(const DirectArgs a) {
   }
 }
 
-template <typename TX, typename TY, int kLayout, int kWin>
+template <typename TX, typename TY, int kLayout, int kWin, int kF>
 tbn_status launch_direct_t(const DirectArgs& a, cudaStream_t s) {
-  constexpr int kF = kWin == 1 ? kFilt : 8;
   const int64_t npix = a.N * a.Po * a.Qo;
   const int64_t gx = (npix + kPix - 1) / kPix;
   const int64_t gy = (a.K + kF - 1) / kF;
@@ -186,13 +225,18 @@ tbn_status launch_direct_t(const DirectArgs& a, cudaStream_t s) {
                 (long long)gy);
   if (a.H >= (1 << 30) || a.W >= (1 << 30))
     return fail(TBN_ERR_UNSUPPORTED, "conv direct: image too large");
-  conv_direct_kernel<TX, TY, kLayout, kWin><<<dim3((unsigned)gx, (unsigned)gy), kPix, 0, s>>>(a);
+  conv_direct_kernel<TX, TY, kLayout, kWin, kF><<<dim3((unsigned)gx, (unsigned)gy), kPix, 0, s>>>(a);
   return check_launch("conv_direct_kernel");
 }
 
 template <typename TX, typename TY, int kLayout>
 tbn_status launch_direct_w(const DirectArgs& a, bool pool, cudaStream_t s) {
-  return pool ? launch_direct_t<TX, TY, kLayout, 4>(a, s) : launch_direct_t<TX, TY, kLayout, 1>(a, s);
+  if (pool) return launch_direct_t<TX, TY, kLayout, 4, 8>(a, s);
+  // 32 filters per CTA share each activation load; 8 where those CTAs would be
+  // fewer than the SMs
+  const int64_t ctas = (a.N * a.Po * a.Qo + kPix - 1) / kPix * ((a.K + kFilt - 1) / kFilt);
+  if (ctas < device_sm_count() && a.K > 8) return launch_direct_t<TX, TY, kLayout, 1, 8>(a, s);
+  return launch_direct_t<TX, TY, kLayout, 1, kFilt>(a, s);
 }
 
 template <int kLayout>

@@ -1277,11 +1277,12 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
           if constexpr (kRowPair) {
             // a zero weight times an infinite or NaN input of the other row's
             // taps is NaN: such sums are recomputed from their own taps
-            float z = 0.0f;
+            uint64_t z2 = 0;
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-              z = fmaf(__uint_as_float(v[0][i]), 0.0f, fmaf(__uint_as_float(v[1][i]), 0.0f, z));
-            if (z != 0.0f) {   // NaN
+              z2 = fma_f32x2(f32x2(v[i >> 3][(2 * i) & 15], v[i >> 3][(2 * i + 1) & 15]), 0ull, z2);
+            if (__uint_as_float(static_cast<uint32_t>(z2)) != 0.0f ||
+                __uint_as_float(static_cast<uint32_t>(z2 >> 32)) != 0.0f) {   // NaN
 #pragma unroll
               for (int i = 0; i < 32; ++i) {
                 const int lg = i >> 4, e = i & 15;
