@@ -126,6 +126,9 @@ __device__ __forceinline__ uint4 scale8(uint4 i4, const float* __restrict__ alph
 // channel.
 template <bool kUnit>
 __global__ void __launch_bounds__(256) bwd_data_prep_kernel(const __grid_constant__ PrepArgs a) {
+  // no grid_dependents_launch(): the convolution after this kernel reads the
+  // codes written here before its own wait
+  grid_dependency_wait();
   if (static_cast<int>(blockIdx.x) < a.code_blocks) {
     transpose_codes(a.codes, a.wpf_in, a.codes_t, a.wpf_out, a.K, a.C, a.R, a.S,
                     static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x,
@@ -681,6 +684,8 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
     if (warp == 1) tmem_dealloc(ctl->tmem_base, kTmaTmem);
     return;
   }
+  grid_dependency_wait();   // x, dy and the partial tiles' buffer
+  grid_dependents_launch();
   bool ok = true;
   if (warp == 0) {
     // ---------------- producer
@@ -809,6 +814,8 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
 __global__ void __launch_bounds__(128) bwd_filter_reduce4_kernel(
     const float4* __restrict__ part, int slices, int groups, int64_t count4,
     float4* __restrict__ dw) {
+  grid_dependency_wait();
+  grid_dependents_launch();
   __shared__ float4 sums[128];
   const int per = 128 / groups;
   const int li = threadIdx.x % per, g = threadIdx.x / per;
@@ -1007,16 +1014,20 @@ tbn_status launch_bwd_filter_tma(const BwdConvShape& p, const void* x, const voi
                   static_cast<unsigned>((t.units + t.per_cta - 1) / t.per_cta),
                   static_cast<unsigned>(t.slices));
   if (grid.y > 65535) return fail(TBN_ERR_UNSUPPORTED, "backward filter: R S C too large");
-  bwd_filter_tma_kernel<<<grid, kTmaThreads, kTmaSmem, s>>>(m_dy, m_x, m_part, a);
+  const cudaError_t le = launch_dependent(bwd_filter_tma_kernel, grid, dim3(kTmaThreads), kTmaSmem,
+                                          s, m_dy, m_x, m_part, a);
+  if (le != cudaSuccess) return cuda_fail(le, "bwd_filter_tma_kernel");
   const tbn_status st = check_launch("bwd_filter_tma_kernel");
   if (st != TBN_OK || direct) return st;
   const float* part = static_cast<const float*>(workspace);
   if (is_aligned(dw, 16)) {   // K % 8 == 0: count is a multiple of 4
     const int groups = t.slices > 32 ? 8 : t.slices > 16 ? 4 : t.slices > 8 ? 2 : 1;
     const int64_t per = 128 / groups;
-    bwd_filter_reduce4_kernel<<<static_cast<unsigned>((count / 4 + per - 1) / per), 128, 0, s>>>(
-        reinterpret_cast<const float4*>(part), t.slices, groups, count / 4,
+    const cudaError_t e = launch_dependent(
+        bwd_filter_reduce4_kernel, dim3(static_cast<unsigned>((count / 4 + per - 1) / per)),
+        dim3(128), 0, s, reinterpret_cast<const float4*>(part), t.slices, groups, count / 4,
         reinterpret_cast<float4*>(dw));
+    if (e != cudaSuccess) return cuda_fail(e, "bwd_filter_reduce4_kernel");
     return check_launch("bwd_filter_reduce4_kernel");
   }
   bwd_filter_reduce_kernel<<<static_cast<unsigned>((count + kBwdThreads - 1) / kBwdThreads),
@@ -1084,10 +1095,10 @@ tbn_status launch_bwd_data(const BwdConvShape& p, const void* dy, const uint32_t
     const int64_t blocks = std::min<int64_t>((threads + 255) / 256,
                                              static_cast<int64_t>(device_sm_count()) * 16);
     const unsigned grid = static_cast<unsigned>(a.code_blocks + blocks);
-    if (unit)
-      bwd_data_prep_kernel<true><<<grid, 256, 0, s>>>(a);
-    else
-      bwd_data_prep_kernel<false><<<grid, 256, 0, s>>>(a);
+    const cudaError_t e = launch_dependent(
+        unit ? bwd_data_prep_kernel<true> : bwd_data_prep_kernel<false>, dim3(grid), dim3(256), 0,
+        s, a);
+    if (e != cudaSuccess) return cuda_fail(e, "bwd_data_prep_kernel");
     const tbn_status st = check_launch("bwd_data_prep_kernel");
     if (st != TBN_OK) return st;
   }

@@ -53,6 +53,28 @@ inline cudaStream_t as_stream(tbn_stream s) { return reinterpret_cast<cudaStream
 
 inline size_t dtype_size(tbn_dtype d) { return d == TBN_BF16 ? 2 : 4; }
 
+// Launch as a programmatic dependent of the previous kernel on the stream: its
+// blocks may be placed while that kernel still runs.  The kernel begins with
+// grid_dependency_wait(), so it reads and writes nothing before that kernel
+// has completed; what is saved is the launch itself between two short kernels.
+// A kernel that then calls grid_dependents_launch() does so after that wait,
+// so everything older than it is complete when its own dependents start.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // One convolution problem after validation.
 struct ConvProblem {
   int64_t N, C, H, W, K, R, S, sh, sw, ph, pw, P, Q;
