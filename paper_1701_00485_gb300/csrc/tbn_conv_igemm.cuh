@@ -1203,6 +1203,23 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const int k = kRowPair ? (m & 63) : tc.ktile * kBM + m;
       const bool kvalid = k < a.K;
       const float a2 = kvalid ? 2.0f * (kFuse ? __ldca(a.alpha + k) : __ldg(a.alpha + k)) : 0.0f;
+      // fragment epilogue: 2 alpha, twice, of this lane's filters (requested
+      // before the accumulator is waited for)
+      const int fr = lane >> 2;   // fragment row within 8
+      uint64_t a2f[2][2];
+      if constexpr (kPoolBW == 0 && kTmaStore) {
+#pragma unroll
+        for (int lg = 0; lg < 2; ++lg) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int mm = sub * 32 + lg * 16 + u * 8 + fr;
+            const int kk = kRowPair ? (mm & 63) : tc.ktile * kBM + mm;
+            const float s2 =
+                kk < a.K ? 2.0f * (kFuse ? __ldca(a.alpha + kk) : __ldg(a.alpha + kk)) : 0.0f;
+            a2f[lg][u] = f32x2(__float_as_uint(s2), __float_as_uint(s2));
+          }
+        }
+      }
       if (kTmaStore) {
         // the previous tile's store must have finished reading the staging tile
         if (elected) bulk_wait_group_read<0>();
@@ -1246,57 +1263,52 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         const int nchunks = (a.tile_n + 31) / 32;
         const int c_begin = (nchunks * half + kParts - 1) / kParts;
         const int c_end = (nchunks * (half + 1) + kParts - 1) / kParts;
-        const int fr = lane >> 2;                       // fragment row within 8
-        uint64_t a2f[2][2];   // 2 alpha, twice
-#pragma unroll
-        for (int lg = 0; lg < 2; ++lg) {
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int mm = sub * 32 + lg * 16 + u * 8 + fr;
-            const int kk = kRowPair ? (mm & 63) : tc.ktile * kBM + mm;
-            const float s2 =
-                kk < a.K ? 2.0f * (kFuse ? __ldca(a.alpha + kk) : __ldg(a.alpha + kk)) : 0.0f;
-            a2f[lg][u] = f32x2(__float_as_uint(s2), __float_as_uint(s2));
-          }
-        }
         // this lane's stmatrix row address pieces: matrix mi = lane / 8, row = lane % 8
         const int mi = lane >> 3, mrow = lane & 7;
         const uint32_t stage_s = smem_addr(stage);
+        // 16 lanes (filters) at a time: the other 16 lanes' columns are on
+        // their way while these are processed.  The accumulator is released
+        // once the last have arrived.
+        uint32_t v[2][16];
+        const auto load = [&](int j, int lg) {
+          tmem_ld_16x256b_x4(acc_b + (static_cast<uint32_t>(sub * 32 + lg * 16) << 16) +
+                                 static_cast<uint32_t>(32 * j),
+                             v[lg]);
+        };
+        if (c_begin < c_end) load(c_begin, 0);
         for (int j = c_begin; j < c_end; ++j) {
-          uint32_t v[2][16];
-#pragma unroll
-          for (int lg = 0; lg < 2; ++lg)
-            tmem_ld_16x256b_x4(acc_b + (static_cast<uint32_t>(sub * 32 + lg * 16) << 16) +
-                                   static_cast<uint32_t>(32 * j),
-                               v[lg]);
-          tmem_wait_ld();
-          if (j == c_end - 1) {
-            tc_fence_before_sync();
-            mbar_arrive(&ctl->acc_empty[ab]);
-          }
-          if constexpr (kRowPair) {
-            // a zero weight times an infinite or NaN input of the other row's
-            // taps is NaN: such sums are recomputed from their own taps
-            uint64_t z2 = 0;
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-              z2 = fma_f32x2(f32x2(v[i >> 3][(2 * i) & 15], v[i >> 3][(2 * i + 1) & 15]), 0ull, z2);
-            if (__uint_as_float(static_cast<uint32_t>(z2)) != 0.0f ||
-                __uint_as_float(static_cast<uint32_t>(z2 >> 32)) != 0.0f) {   // NaN
-#pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                const int lg = i >> 4, e = i & 15;
-                const int mm = sub * 32 + lg * 16 + ((e >> 1) & 1) * 8 + fr;
-                const int px = 32 * j + 8 * (e >> 2) + 2 * (lane & 3) + (e & 1);
-                const int f = tc.p0 * a.Q + px;   // pixel of the row pairs
-                if ((mm & 63) < a.K && px < a.bw * a.bh && f < a.P * a.Q &&
-                    !(fabsf(__uint_as_float(v[lg][e])) <= 3.402823466e38f))
-                  v[lg][e] = __float_as_uint(rowpair_sum(a, mm, f));
-              }
-            }
-          }
 #pragma unroll
           for (int lg = 0; lg < 2; ++lg) {
+            tmem_wait_ld();
+            if (lg == 0) {
+              load(j, 1);
+            } else if (j + 1 < c_end) {
+              load(j + 1, 0);
+            } else {
+              tc_fence_before_sync();
+              mbar_arrive(&ctl->acc_empty[ab]);
+            }
+            if constexpr (kRowPair) {
+              // a zero weight times an infinite or NaN input of the other row's
+              // taps is NaN: such sums are recomputed from their own taps
+              uint64_t z2[2] = {0, 0};
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                z2[i & 1] = fma_f32x2(f32x2(v[lg][2 * i], v[lg][2 * i + 1]), 0ull, z2[i & 1]);
+              z2[0] = add_f32x2(z2[0], z2[1]);
+              if (__uint_as_float(static_cast<uint32_t>(z2[0])) != 0.0f ||
+                  __uint_as_float(static_cast<uint32_t>(z2[0] >> 32)) != 0.0f) {   // NaN
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                  const int mm = sub * 32 + lg * 16 + ((e >> 1) & 1) * 8 + fr;
+                  const int px = 32 * j + 8 * (e >> 2) + 2 * (lane & 3) + (e & 1);
+                  const int f = tc.p0 * a.Q + px;   // pixel of the row pairs
+                  if ((mm & 63) < a.K && px < a.bw * a.bh && f < a.P * a.Q &&
+                      !(fabsf(__uint_as_float(v[lg][e])) <= 3.402823466e38f))
+                    v[lg][e] = __float_as_uint(rowpair_sum(a, mm, f));
+                }
+              }
+            }
             uint32_t pk[8];
             uint32_t addr[2];
 #pragma unroll
@@ -1314,8 +1326,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
                                   pk[4 * bp + 3]);
             }
             // pk[2b], pk[2b + 1]: pixels 2 (lane % 4) + 0/1 of block b, filters fr
-            // and fr + 8.  Two pixels per instruction: this loop is what holds
-            // the accumulator of a short filter's tile.
+            // and fr + 8
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
               const uint64_t acc2x = f32x2(v[lg][2 * e], v[lg][2 * e + 1]);
