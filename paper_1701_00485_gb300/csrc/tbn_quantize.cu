@@ -16,7 +16,8 @@
 // rows are 16-byte aligned with n % 16 == 0 streams its weights (contiguous
 // in W, at most 2048 words = 128 KB) through a ring of three 32 KB shared-
 // memory stages filled by 1-D TMA bulk copies (thread 0 keeps three in
-// flight, every wait bounded); other tasks load through registers, and a
+// flight, every wait bounded); other tasks are staged there 4 bytes at a time
+// (at most 1024 words), and a
 // filter longer than 2048 words is a task of its own with its words strided
 // over the threads.
 //
@@ -40,7 +41,9 @@ namespace tbn {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kGroupWords = 1024;                        // words of a register-loaded task
+constexpr int kGroupWords = 1024;                        // words of a staged task, at most
+constexpr int kStagedPitch = 17;                         // floats per word of a staged task
+constexpr int kStagedBytes = kGroupWords * kStagedPitch * 4;
 constexpr int kItemWords = 2048;                         // words of a streamed item, at most
 constexpr int kChunkBytes = 32768;                       // one ring stage: 512 words
 constexpr int kChunkWords = kChunkBytes / 64;
@@ -59,10 +62,10 @@ struct QJob {
   int32_t wpf;   // words per filter
   int32_t vec;   // 16-byte loads allowed
   int32_t rows;  // filters per task (0: one long filter per task, strided words)
-  int32_t mode;  // kModeStream, kModeRegs or kModeLong
+  int32_t mode;  // one of the modes below
 };
 
-enum : int32_t { kModeStream = 0, kModeRegs = 1, kModeLong = 2 };
+enum : int32_t { kModeStream = 0, kModeStaged = 1, kModeLong = 2, kModeRegs = 3 };
 
 struct QParams {
   QJob job[TBN_MAX_QUANT_JOBS];
@@ -275,8 +278,58 @@ __device__ bool task_stream(const StreamTask& t, const StreamTask* nxt, QShared&
   return true;
 }
 
-// Register-loaded task (rows not 16-byte aligned or n % 16 != 0; small
-// layers such as a network's first): one word per thread per round.
+// Staged task (rows not 16-byte aligned or n % 16 != 0): the task's weights, one
+// contiguous range of W, are copied 4 bytes at a time by consecutive threads
+// into shared memory, all in flight at once, each word's 16 at a pitch of 17
+// so that the threads then read their words without bank conflicts.  (Each
+// thread loading its own word from global memory touched 32 words' lines per
+// instruction: 6388 filters of 1351 weights 22 us, a quarter of the copy rate.)
+__device__ void task_staged(const QJob& jb, int64_t k0, int nrows, QShared& sh, float* buf) {
+  const int n = jb.n, wpf = jb.wpf, nwords = nrows * wpf, total = nrows * n;
+  const float* base = jb.W + k0 * static_cast<int64_t>(n);
+  uint32_t* out = jb.codes + k0 * static_cast<int64_t>(wpf);
+  {
+    int r = threadIdx.x / n, j = threadIdx.x - r * n;
+    const int dr = kThreads / n, dj = kThreads - dr * n;
+    for (int i = threadIdx.x; i < total; i += kThreads) {
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                       smem_addr(buf + (r * wpf + (j >> 4)) * kStagedPitch + (j & 15))),
+                   "l"(base + i)
+                   : "memory");
+      r += dr;
+      j += dj;
+      if (j >= n) {
+        j -= n;
+        ++r;
+      }
+    }
+  }
+  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  int c = threadIdx.x % wpf;
+  const int dc = kThreads % wpf;
+  for (int w = threadIdx.x; w < nwords; w += kThreads) {
+    const int nv = min(16, n - 16 * c);
+    float v[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = e < nv ? buf[w * kStagedPitch + e] : 0.0f;
+    uint32_t word;
+    float sum;
+    int c2;
+    encode16(v, nv, word, sum, c2);
+    out[w] = word;
+    sh.sum[w] = sum;
+    sh.cnt[w] = c2;
+    c += dc;
+    if (c >= wpf) c -= wpf;
+  }
+  fence_proxy_async_smem();   // a streamed task's bulk copies may reuse the buffer
+  __syncthreads();
+  reduce_rows(jb, k0, nrows, base, sh);
+  __syncthreads();
+}
+
+// Register-loaded task (a small layer of such rows, e.g. a network's first): one word per thread per round.
 __device__ void task_regs(const QJob& jb, int64_t k0, int nrows, QShared& sh) {
   const int nwords = nrows * jb.wpf;
   const float* base = jb.W + k0 * static_cast<int64_t>(jb.n);
@@ -343,7 +396,8 @@ __device__ __forceinline__ int job_of(const QParams& prm, int64_t task) {
 // filters of one job (sized so that tasks carry about equal bytes).
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_pack_kernel(const __grid_constant__ QParams prm,
                                                                     int64_t ntasks) {
-  extern __shared__ __align__(128) uint8_t q_ring[];   // kRingBytes when any job streams
+  extern __shared__ __align__(128) uint8_t q_ring[];   // kRingBytes when any job streams,
+                                                       // kStagedBytes when one is staged
   __shared__ QShared sh;
   __shared__ uint64_t full[kStages];
   if (threadIdx.x == 0) {
@@ -376,7 +430,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_pack_kernel(con
         if (!task_stream(stream_task(jb, k0, nrows), nxt, sh, q_ring, full, seq, issued, prm.err))
           return;
       } else {
-        task_regs(jb, k0, nrows, sh);
+        if (jb.mode == kModeStaged)
+          task_staged(jb, k0, nrows, sh, reinterpret_cast<float*>(q_ring));
+        else
+          task_regs(jb, k0, nrows, sh);
       }
     }
   }
@@ -467,7 +524,7 @@ tbn_status launch_quantize_group(const tbn_quant_job* jobs, int njobs, cudaStrea
   for (int i = 0; i < njobs; ++i) total_words += jobs[i].K * ((jobs[i].n + 15) / 16);
   const int64_t target = std::max<int64_t>(1, (total_words + slots - 1) / std::max(1, slots));
   int64_t tasks = 0;
-  bool any_stream = false;
+  bool any_stream = false, any_staged = false;
   for (int i = 0; i < njobs; ++i) {
     const tbn_quant_job& j = jobs[i];
     QJob& q = prm.job[i];
@@ -484,8 +541,17 @@ tbn_status launch_quantize_group(const tbn_quant_job* jobs, int njobs, cudaStrea
       q.rows = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>({want, j.K, kItemWords / q.wpf})));
       any_stream = true;
     } else if (q.wpf <= kGroupWords) {
-      q.mode = kModeRegs;
+      // a task's worth or less: straight through registers (20 filters of 25
+      // weights 2.4 us, staged 2.8)
+      const bool small = j.K * q.wpf <= kGroupWords;
+      q.mode = small ? kModeRegs : kModeStaged;
+      any_staged |= !small;
       q.rows = static_cast<int32_t>(std::min<int64_t>(j.K, kGroupWords / q.wpf));
+      // like a streamed task's share, but never so few words that a task's
+      // phases are all latency
+      const int64_t want =
+          (std::min<int64_t>(std::max<int64_t>(target, 128), kGroupWords) + q.wpf - 1) / q.wpf;
+      if (!small) q.rows = static_cast<int32_t>(std::min<int64_t>(want, q.rows));
     } else {
       q.mode = kModeLong;
       q.rows = 0;
@@ -506,7 +572,9 @@ tbn_status launch_quantize_group(const tbn_quant_job* jobs, int njobs, cudaStrea
   });
   if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(quantize)");
   const unsigned grid = static_cast<unsigned>(std::min<int64_t>(tasks, slots));
-  quantize_pack_kernel<<<grid, kThreads, any_stream ? kRingBytes : 0, s>>>(prm, tasks);
+  static_assert(kStagedBytes <= kRingBytes, "the staged words share the ring");
+  const size_t smem = any_stream ? kRingBytes : any_staged ? kStagedBytes : 0;
+  quantize_pack_kernel<<<grid, kThreads, smem, s>>>(prm, tasks);
   return check_launch("quantize_pack_kernel");
 }
 

@@ -118,3 +118,19 @@ def test_unpack_formats(K, n):
 
 def test_no_device_error_recorded():
     assert tbn.tbn_device_error() == 0
+
+
+@pytest.mark.parametrize("K,n", [(700, 1), (300, 15), (257, 17), (40, 255), (33, 257), (12, 1351),
+                                 (3, 16381), (2, 16400), (5000, 33)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_quantize_staged_tasks(K, n, offset):
+    """Filters that are staged 4 bytes at a time: counts around a word, a
+    thread row of 256 and a task of 1024 words, one filter more than staged
+    tasks take, and weights that start off a 16-byte boundary."""
+    W = _weights(K, n, "wide", seed=K * 31 + n)
+    buf = torch.empty(K * n + offset, device="cuda")
+    Wd = buf[offset:].view(K, n)
+    Wd.copy_(W)
+    codes, alpha = tbn.tbn_quantize_pack(Wd)
+    torch.cuda.synchronize()
+    check_quantize(W, codes, alpha)
