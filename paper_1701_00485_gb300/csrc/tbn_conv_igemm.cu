@@ -51,6 +51,43 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
   }
 }
 
+// Split K within clusters: the K ranges (2 .. 8) that a cluster's CTAs take of
+// each tile, with `t` set to its tiles, or 1 where the two launches of
+// splitk_reduce_kernel's form are estimated to be quicker.  At most the
+// p.ksplit ranges that the caller's workspace holds, and clusters in whole
+// waves of those that the device runs at once (GB300: 36 of four CTAs, 15 of
+// eight).  Costs in ns: a K block as in plan_cost; start, exchange and end,
+// fitted, 3.5 us + 12 ns a pixel in a cluster; two launches 4.5 us + 12 ns a
+// pixel + 80 ns a range, whose sums one thread adds in turn.  Measured, two
+// launches and clusters: 256 x 9216 -> 4096 21.0 and 19.2 us, 256 x 4096 ->
+// 4096 15.6 and 13.8, 256 x 4096 -> 1000 11.4 and 9.3 (two tiles of 128
+// images, six ranges), 64 x 2048 -> 300 7.9 and 5.4; even at 64 x 25088 -> 128
+// (98 ranges of four K blocks), beyond which two launches win.
+int cluster_split(const ConvProblem& p, TilePlan& t) {
+  const int64_t kb = kblocks_of(p), tk = ceil_div(p.K, kBM);
+  const auto block = [](int64_t bn) { return 215.0 + 0.25 * bn; };
+  double cost = ceil_div(kb, p.ksplit) * block(t.bn) + 4500.0 + 12.0 * t.bn + 80.0 * p.ksplit;
+  const int parts0 = t.tiles_n;
+  int best = 1;
+  for (int parts = parts0; parts <= 4 * parts0; ++parts) {
+    const int bn = ceil_div(p.N, parts);
+    if (ceil_div(p.N, bn) != parts) continue;
+    for (int S = 2; S <= std::min(kMaxCluster, p.ksplit); ++S) {
+      const int per = ceil_div(kb, S), fit = igemm_max_clusters(S);
+      if ((S - 1) * per >= kb || fit < 1) continue;
+      const double c = ceil_div(parts * tk, fit) * (per * block(bn) + 3500.0 + 12.0 * bn);
+      // narrower tiles only for a clear gain
+      if (c >= (parts > t.tiles_n && best > 1 ? 0.95 : 1.0) * cost) continue;
+      cost = c;
+      best = S;
+      t.bn = t.T = bn;
+      t.tiles_n = parts;
+      t.tile_n = (bn + 15) / 16 * 16;
+    }
+  }
+  return best;
+}
+
 // Patch mode (gathered activations staged per tile in shared memory) when a
 // tile is whole output rows of one image, the filter spans at most
 // kPatchMaxKBlocks K blocks and two patches fit beside the ring.
@@ -172,7 +209,9 @@ bool conv_igemm_pools_any_width(const ConvProblem& p) {
 tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const bool s2d = p0.layout == TBN_S2D_NHWC;
   const ConvProblem p = s2d ? s2d_problem(p0) : p0;
-  const TilePlan t = plan_conv(p, s2d);
+  TilePlan t = plan_conv(p, s2d);
+  const bool split = p.ksplit > 1 && p.partial != nullptr;
+  const int cluster = split && is_aligned(p.partial, 16) ? cluster_split(p, t) : 1;
   IgArgs a{};
   a.N = (int)t.oN; a.C = (int)p.C; a.H = (int)p.H; a.W = (int)p.W; a.K = (int)p.K;
   a.R = (int)p.R; a.S = (int)p.S; a.sh = (int)p.sh; a.sw = (int)p.sw;
@@ -189,8 +228,8 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n * a.tiles_k;
   a.ncodes = (int)(p.C * p.R * p.S);
   a.kblocks = t.rowpair ? a.R * a.S * a.C / kBK : static_cast<int>(kblocks_of(p));
-  const bool split = p.ksplit > 1 && p.partial != nullptr;
-  a.ksplit = split ? p.ksplit : 1;
+  a.cluster = cluster > 1 ? 1 : 0;
+  a.ksplit = a.cluster ? cluster : split ? p.ksplit : 1;
   a.kb_per = ceil_div(a.kblocks, a.ksplit);
   if (split && (!tma_fed(p) || p.pool || p.P != 1 || p.Q != 1 || p.R != 1 || p.S != 1 ||
                 (a.ksplit - 1) * a.kb_per >= a.kblocks))
@@ -199,7 +238,7 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   a.base_tiles = static_cast<int>(tiles);
   a.tiles = static_cast<int>(tiles * a.ksplit);
   a.partial = split ? p.partial : nullptr;
-  a.by_base = fast_div(a.base_tiles);
+  a.by_base = fast_div(a.cluster ? a.ksplit : a.base_tiles);
   a.by_k = fast_div(a.tiles_k);
   a.by_tq = fast_div(a.tiles_q);
   a.by_tp = fast_div(a.tiles_p);
@@ -239,11 +278,12 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const int pw = pool_width(p, t);
   const bool tst = use_tma_store(p) && !split;   // partial sums: direct fp32 stores
   if (split) {
-    // the K ranges' partial sums, then their ordered sum with the epilogue
+    // the K ranges' partial sums, then (unless each cluster adds its own)
+    // their ordered sum with the epilogue
     const tbn_status st = use_tma_pad(p) ? launch_igemm_pad(p, t, a, pw, false, s)
                           : use_ch32(p)  ? launch_igemm_tma32(p, t, a, pw, false, false, s)
                                          : launch_igemm_tma64(p, t, a, pw, false, false, s);
-    if (st != TBN_OK) return st;
+    if (st != TBN_OK || a.cluster) return st;
     const int64_t mk = p.N * p.P * p.Q * p.K;
     const bool vec = p.K % 4 == 0 && is_aligned(p.partial, 16);
     const int64_t items = vec ? mk / 4 : mk;

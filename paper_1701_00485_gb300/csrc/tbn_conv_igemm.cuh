@@ -116,7 +116,7 @@ struct IgArgs {
   // pooling); an image's output is iP x iQ
   int im2col, iP, iQ;
   // divisors of the tile and pixel coordinates
-  FastDiv by_base, by_k, by_tq, by_tp, by_iq, by_ip;
+  FastDiv by_base /* by ksplit with clusters */, by_k, by_tq, by_tp, by_iq, by_ip;
   // patch mode: the patch is rows [p0 sh - ph, + PR) x columns [-pw, W + pw)
   int PR, PW;              // patch rows, patch columns (W + 2 pw)
   int patch_cap;           // bytes per patch buffer (multiple of 16)
@@ -126,6 +126,9 @@ struct IgArgs {
   // tile t % base_tiles; the fp32 partial sums go to `partial`
   // [ksplit][N][P][Q][K] and a second kernel adds them in split order
   int ksplit, kb_per, base_tiles;
+  // or, in clusters of ksplit CTAs (CTA i: K-block range i % ksplit of output
+  // tile i / ksplit), the cluster adds them itself (add_cluster_sums)
+  int cluster;
   // two accumulators (tile_n <= 176): tile i accumulates into columns
   // [176 (i % 2), + 176), so its MMAs need not wait for the epilogue of
   // tile i - 1; the weight ring then starts at column 352
@@ -176,6 +179,7 @@ constexpr int kFirstGatherWarp = kFirstEpiWarp + kEpiWarps;
 constexpr int kStageBytes = kMaxTileN * kBK * 2;     // 32 KiB
 constexpr int kOutStageBytes = kMaxTileN * kBM * 2;  // 64 KiB bf16 output box
 constexpr uint64_t kWaitLimitNs = 1000000000ull;    // 1 s
+constexpr int kMaxCluster = 8;      // K ranges of a cluster (the portable cluster size)
 
 static_assert(kAccCols + kStages * kAColsPerStage <= kTmemCols, "TMEM budget");
 static_assert(2 * kAcc2Cols + kStages * kAColsPerStage <= kTmemCols, "TMEM budget");
@@ -273,8 +277,9 @@ struct TileCoord {
 
 __device__ __forceinline__ TileCoord tile_coord(const IgArgs& a, int t) {
   TileCoord c;
-  c.split = a.by_base(t);
-  t -= c.split * a.base_tiles;
+  const int d = a.by_base(t);
+  c.split = a.cluster ? t - d * a.ksplit : d;
+  t = a.cluster ? d : t - d * a.base_tiles;
   c.kb0 = c.split * a.kb_per;
   c.kb1 = min(a.kblocks, c.kb0 + a.kb_per);
   const int pt_lin = a.by_k(t);
@@ -323,6 +328,78 @@ __device__ __noinline__ float rowpair_sum(const IgArgs& a, int m, int f) {
       }
     }
   return acc;
+}
+
+// Split K in a cluster: its CTAs have stored the sums of one K range each for
+// the same tile to a.partial.  Once all have, CTA r adds the ranges of the
+// r-th share of the tile's pixels in range order (as splitk_reduce_kernel
+// does: the same bits) and applies the epilogue: a warp takes a pixel at a
+// time, a lane four filters, all ranges requested at once.  Called by all
+// threads; the barrier is reached by every CTA, since every other wait is
+// bounded.
+__device__ __forceinline__ void add_cluster_sums(const IgArgs& a) {
+  cluster_sync();
+  const TileCoord tc = tile_coord(a, blockIdx.x);
+  const int T = min(a.bn, a.N - tc.n0);   // pixels of the tile: images of a 1 x 1 map
+  const int share = (T + a.ksplit - 1) / a.ksplit;
+  const int px_end = min(T, share * (tc.split + 1));
+  const int k0 = tc.ktile * kBM + 4 * (threadIdx.x & 31);
+  if (k0 >= a.K) return;
+  const bool vec = (a.K & 3) == 0;   // partial is 16-byte aligned
+  const size_t mk = static_cast<size_t>(a.N) * a.K;
+  float a2[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) a2[e] = k0 + e < a.K ? 2.0f * __ldg(a.alpha + k0 + e) : 0.0f;
+  for (int px = share * tc.split + static_cast<int>(threadIdx.x >> 5); px < px_end;
+       px += static_cast<int>(blockDim.x >> 5)) {
+    const size_t o = static_cast<size_t>(tc.n0 + px) * a.K + k0;
+    float4 v[kMaxCluster];
+#pragma unroll
+    for (int i = 0; i < kMaxCluster; ++i)
+      if (i < a.ksplit) {
+        const float* src = a.partial + i * mk + o;
+        if (vec) {
+          v[i] = __ldcg(reinterpret_cast<const float4*>(src));
+        } else {
+          v[i].x = __ldcg(src);
+          v[i].y = k0 + 1 < a.K ? __ldcg(src + 1) : 0.0f;
+          v[i].z = k0 + 2 < a.K ? __ldcg(src + 2) : 0.0f;
+          v[i].w = k0 + 3 < a.K ? __ldcg(src + 3) : 0.0f;
+        }
+      }
+    float res[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (a.residual) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (k0 + e < a.K) res[e] = load_residual(a, o + e);
+    }
+#pragma unroll
+    for (int i = 1; i < kMaxCluster; ++i)
+      if (i < a.ksplit) {
+        v[0].x += v[i].x; v[0].y += v[i].y; v[0].z += v[i].z; v[0].w += v[i].w;
+      }
+    float y[4] = {a2[0] * v[0].x, a2[1] * v[0].y, a2[2] * v[0].z, a2[3] * v[0].w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (a.residual) y[e] += res[e];
+      if (a.relu) y[e] = fmaxf(y[e], 0.0f);
+    }
+    if (vec && a.y_bf16 && (reinterpret_cast<uintptr_t>(a.y) & 7) == 0) {
+      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(a.y) + o) =
+          make_uint2(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]));
+    } else if (vec && !a.y_bf16 && (reinterpret_cast<uintptr_t>(a.y) & 15) == 0) {
+      *reinterpret_cast<float4*>(static_cast<float*>(a.y) + o) = make_float4(y[0], y[1], y[2], y[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (k0 + e >= a.K) break;
+        if (a.y_bf16)
+          static_cast<__nv_bfloat16*>(a.y)[o + e] = __float2bfloat16_rn(y[e]);
+        else
+          static_cast<float*>(a.y)[o + e] = y[e];
+      }
+    }
+  }
 }
 
 // kPoolBW: 0 = no pool; 8, 16, 32 = fused 2x2/2 max pool for tiles of whole
@@ -453,6 +530,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
   constexpr bool kS2d = kMode == kModeS2d;
   constexpr bool kPad = kMode == kModeTmaPad;
   constexpr bool kRowPair = kMode == kModeRowPair;
+  constexpr bool kCanCluster = kPoolBW == 0 && !kTmaStore && !kFuse &&
+                               (kMode == kModeTma64 || kMode == kModeTma32 || kPad);
   constexpr int kSt = stages_for(kMode);   // ring stages
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte aligned by pointer arithmetic on the shared array, so that the
@@ -539,7 +618,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
   }
   if (*abort_flag) {
     if (warp == 1) tmem_dealloc(ctl->tmem_base, kTmemCols);
-    return;
+    return;   // (the others of a cluster count an exited CTA as arrived)
   }
   const uint32_t acc_tmem = tmem;               // columns [0, 256), or two of 176
   const uint32_t a_tmem0 = tmem + (a.acc2 ? 2u * kAcc2Cols : static_cast<uint32_t>(kAccCols));   // weight ring
@@ -1538,6 +1617,12 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }
+  if constexpr (kCanCluster) {
+    if (a.cluster) {
+      grid_dependency_wait();   // for every thread: the residual is read, y written
+      add_cluster_sums(a);
+    }
+  }
 }
 
 
@@ -1831,7 +1916,7 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
   cfg.blockDim = dim3(threads_for<kMode>());
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   if (kFuse) {
     // fused quantization: the CTAs meet at a grid-wide barrier, so they must
     // all be resident at once
@@ -1843,6 +1928,13 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
   }
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (a.cluster) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(a.ksplit);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+    cfg.gridDim = dim3(static_cast<unsigned>(a.tiles));   // whole clusters, a tile each
+  }
   if (kFuse) {
     const cudaError_t me = cudaMemsetAsync(a.gbar, 0, sizeof(unsigned), s);
     if (me != cudaSuccess) return cuda_fail(me, "cudaMemsetAsync(barrier word)");
@@ -1873,6 +1965,9 @@ tbn_status launch_pool(const ConvProblem& p, const TilePlan& t, IgArgs& a, int p
 // a.wq in the same (cooperative) launch.
 tbn_status launch_igemm_tma64(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
                               bool tma_store, bool fuse, cudaStream_t s);
+// Clusters of `size` (2 .. kMaxCluster) CTAs of the TMA modes that the device
+// runs at once (0: none).
+int igemm_max_clusters(int size);
 tbn_status launch_igemm_tma32(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
                               bool tma_store, bool fuse, cudaStream_t s);
 tbn_status launch_igemm_pad(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,

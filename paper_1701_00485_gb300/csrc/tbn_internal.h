@@ -88,8 +88,9 @@ struct ConvProblem {
   const void* residual;
   int pool;  // 0 or 2 (2x2 max pool, stride 2, after ReLU)
   // split K (implicit GEMM only; set by tbn_linear_fwd_ws): ksplit > 1 K
-  // ranges accumulate into fp32 `partial` [ksplit][N][P][Q][K], then a
-  // second kernel adds them in order and applies the epilogue
+  // ranges (fewer, in clusters, where those are quicker) accumulate into fp32
+  // `partial` [ksplit][N][P][Q][K]; the clusters, or else a second kernel, add
+  // them in order and apply the epilogue
   float* partial;
   int ksplit;
   // fused quantization (implicit GEMM only; set by tbn_conv2d_fwd_quant):

@@ -124,6 +124,39 @@ def test_padded_linear(B, K_in, K_out):
         assert_within(y.cpu().numpy(), want, bound, out_bf16=False, what="padded linear")
 
 
+@pytest.mark.parametrize("B,K_in,K_out,dtype,res", [
+    (256, 4096, 1000, torch.bfloat16, False),   # tiles of 128 images
+    (300, 4096, 512, torch.float32, True),      # a last tile of fewer images
+    (33, 2016, 131, torch.bfloat16, True),      # K_out odd, 32-channel boxes, a ragged last range
+    (9, 520, 128, torch.float32, False),        # two ranges, padded channels
+    (17, 8192, 129, torch.bfloat16, False),     # eight ranges, one filter in the last tile
+    (64, 100352, 64, torch.float32, False),     # a filter so long that it takes two launches
+])
+def test_linear_split_in_clusters(B, K_in, K_out, dtype, res):
+    """Split K whose ranges are added by the clusters that computed them, y at
+    an odd element offset and aligned."""
+    g = inputs.generator(B + K_in)
+    x = torch.randn(B, K_in, generator=g).to(torch.bfloat16)
+    W = torch.randn(K_out, K_in, generator=g)
+    r = torch.randn(B, K_out, generator=g).to(dtype) if res else None
+    codes, alpha = tbn.tbn_quantize_pack(W.cuda())
+    n = tbn.tbn_linear_workspace_bytes(B, K_in, K_out)
+    assert n >= 2 * 4 * B * K_out
+    ws = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda")
+    wt, al = oracle.quantize(W.numpy())
+    y_orc, bound = oracle.linear(x.float().numpy(), wt, al)
+    want = oracle.epilogue(y_orc, r.float().numpy() if res else None, relu=True)
+    for off in (0, 1):
+        buf = torch.full((B * K_out + 2,), float("nan"), dtype=dtype, device="cuda")
+        y = buf[off:off + B * K_out].view(B, K_out)
+        tbn.tbn_linear_fwd_ws(x.cuda(), codes, alpha, K_out, ws, relu=True,
+                              residual=r.cuda() if res else None, out=y, out_dtype=dtype)
+        assert_within(y.float().cpu().numpy(), want, bound, out_bf16=dtype == torch.bfloat16,
+                      epilogue=True, what="clusters %s" % ((B, K_in, K_out, off),))
+        assert torch.isnan(buf[:off]).all() and torch.isnan(buf[off + B * K_out:]).all()
+    assert tbn.tbn_device_error() == 0
+
+
 @pytest.mark.parametrize("case", [
     (3, 64, 28, 28, 72, 3, 3, (1, 1), (1, 1)),      # even map: runs of row pairs
     (2, 64, 13, 11, 136, 3, 3, (1, 1), (1, 1)),     # odd: the last row and column drop
