@@ -118,7 +118,10 @@ typedef enum {
   TBN_CONV_AUTO = 0,
   TBN_CONV_DIRECT = 1,        /* CUDA-core direct convolution, any layout/dtype   */
   TBN_CONV_IMPLICIT_GEMM = 2, /* tcgen05 implicit GEMM, NHWC bf16 x; activations
-                                 by TMA when C % 64 == 0, else gathered by threads */
+                                 by TMA when C % 8 == 0 and the strides are 1 or
+                                 2, else gathered by threads; a fused pool over
+                                 rows of 8, 16 or 32 (AUTO also sends TMA-fed
+                                 layers with other rows of up to 128 here) */
   TBN_CONV_SMALL_TAPS = 3     /* tensor-core convolution for short filters,
                                  C*R*S <= 64, bf16 x in any layout, no fused
                                  pool: the input patch and its im2col
@@ -285,7 +288,7 @@ tbn_status tbn_repack(const uint32_t *in, int64_t K, int64_t n, uint32_t *out,
  *   epi    optional fused epilogue (NULL = none).
  * Accumulation is fp32; x * W~ products are exact.  y must not alias x.
  * The tensor-core implicit-GEMM path needs NHWC and bf16 x (16-byte aligned
- * x, y and residual; stride 1 or 2 when C % 64 == 0, any stride otherwise);
+ * x, y and residual; fastest with C % 8 == 0 and strides of 1 or 2);
  * the small-tap path takes bf16 x with C*R*S <= 64 in any layout; AUTO falls
  * back to the CUDA-core direct kernel for every other case. */
 tbn_status tbn_conv2d_fwd(const void *x, tbn_dtype xdt, tbn_layout layout, int64_t N,
