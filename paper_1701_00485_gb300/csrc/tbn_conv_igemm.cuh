@@ -1147,22 +1147,37 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       cp = a.codes + static_cast<size_t>(in ? k : 0) * a.wpf + 4 * kb_ld + 2 * half;
     };
     set_row();
-    auto next_codes = [&]() -> uint2 {
-      uint2 r = make_uint2(0u, 0u);
+    // the two words of a half K block; in padded mode the three words that hold
+    // its codes and whether they begin in the middle of the first, put together
+    // when they are decoded: put together here, every K block would wait for
+    // its own loads (27 x 27, 56 channels, 5 x 5, 128 filters, batch 32: 13.5 us
+    // so, 12.1 now)
+    struct Codes {
+      uint32_t x, y, z;
+      bool mid;
+    };
+    const auto decode = [&](const Codes& q, uint32_t* v, const PairMultipliers& pm) {
+      uint32_t x = q.x, y = q.y;
+      if (kPad && q.mid) {
+        x = ((x >> 4) & 0x0F0F0F0Fu) | ((y & 0x0F0F0F0Fu) << 4);
+        y = ((y >> 4) & 0x0F0F0F0Fu) | ((q.z & 0x0F0F0F0Fu) << 4);
+      }
+      word_to_bf16x2(x, v, pm);
+      word_to_bf16x2(y, v + 8, pm);
+    };
+    auto next_codes = [&]() -> Codes {
+      Codes r{0u, 0u, 0u, false};
       if constexpr (kPad) {
         // 32 codes from code0 on (a multiple of 8: whole words, or the upper
-        // half of one and the lower half of the next); words past the row are
-        // zero, codes of the next tap multiply zero activations
-        if (kb_ld < kb_lim && ch_left > 32 * half) {
-          const int w = code0 >> 4;
-          const uint32_t w0 = __ldg(cp + w);
-          const uint32_t w1 = w + 1 < a.wpf ? __ldg(cp + w + 1) : 0u;
-          r = make_uint2(w0, w1);
-          if (code0 & 8) {
-            const uint32_t w2 = w + 2 < a.wpf ? __ldg(cp + w + 2) : 0u;
-            r.x = ((w0 >> 4) & 0x0F0F0F0Fu) | ((w1 & 0x0F0F0F0Fu) << 4);
-            r.y = ((w1 >> 4) & 0x0F0F0F0Fu) | ((w2 & 0x0F0F0F0Fu) << 4);
-          }
+        // half of one and the lower half of the next), fewer where the tap
+        // ends: other columns multiply zero activations
+        const int n = min(32, ch_left - 32 * half);
+        if (kb_ld < kb_lim && n > 0) {
+          const int w = code0 >> 4, end = (code0 & 8) + n;
+          r.mid = (code0 & 8) != 0;
+          r.x = __ldg(cp + w);
+          if (end > 16) r.y = __ldg(cp + w + 1);
+          if (end > 32) r.z = __ldg(cp + w + 2);
         }
         if (ch_left > kBK) {
           ch_left -= kBK;
@@ -1182,13 +1197,16 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         // coherent) loads after the grid barrier's acquire then, not the
         // read-only path, which assumes data constant for the whole launch
         const bool two = 4 * kb_ld + 2 * half + 1 < a.wpf;
+        uint2 t;
         if constexpr (kFuse) {
-          if (pair_ok) r = __ldca(reinterpret_cast<const uint2*>(cp));
-          else r = make_uint2(__ldca(cp), two ? __ldca(cp + 1) : 0u);
+          if (pair_ok) t = __ldca(reinterpret_cast<const uint2*>(cp));
+          else t = make_uint2(__ldca(cp), two ? __ldca(cp + 1) : 0u);
         } else {
-          if (pair_ok) r = __ldg(reinterpret_cast<const uint2*>(cp));
-          else r = make_uint2(__ldg(cp), two ? __ldg(cp + 1) : 0u);
+          if (pair_ok) t = __ldg(reinterpret_cast<const uint2*>(cp));
+          else t = make_uint2(__ldg(cp), two ? __ldg(cp + 1) : 0u);
         }
+        r.x = t.x;
+        r.y = t.y;
       }
       cp += 4;
       if (++kb_ld == kb_end) {
@@ -1198,7 +1216,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       return r;
     };
     const PairMultipliers pm;
-    uint2 q0 = next_codes(), q1 = next_codes(), q2 = next_codes(), q3 = next_codes();
+    Codes q0 = next_codes(), q1 = next_codes(), q2 = next_codes(), q3 = next_codes();
     const uint32_t col = a_tmem0 + lane_off + static_cast<uint32_t>(16 * half);
     // two K blocks per iteration: their tensor-memory stores share one
     // tcgen05.wait::st
@@ -1207,10 +1225,8 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     for (int g = 0; g < total; g += 2) {
       const bool two = g + 1 < total;   // warp-uniform
       uint32_t v0[16], v1[16];
-      word_to_bf16x2(q0.x, v0 + 0, pm);
-      word_to_bf16x2(q0.y, v0 + 8, pm);
-      word_to_bf16x2(q1.x, v1 + 0, pm);
-      word_to_bf16x2(q1.y, v1 + 8, pm);
+      decode(q0, v0, pm);
+      decode(q1, v1, pm);
       if constexpr (kRowPair) {
         // warp-uniform: a whole half's K block is taps or zeros
         const auto zero = [&](uint32_t* v) {
@@ -1861,6 +1877,14 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
     const cuuint32_t estr[4] = {1u, (cuuint32_t)p.sw, (cuuint32_t)(p.sh + rp), 1u};
     const cuuint32_t channels = kCh32 ? kBK / 2 : kBK;
     const CUtensorMapSwizzle swizzle = kCh32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+    // Boxes narrower than a pixel's channels, or than the 64 of a box, read
+    // rows that do not fill 256-byte lines: promoting their requests to whole
+    // ones reads beside what is wanted (27 x 27, batch 256, 96 -> 256 channels,
+    // 5 x 5: 142 us so, 138 without; 40 -> 128 channels, batch 32, fp32 y: 26.3
+    // and 22.2; layers of 64-channel boxes are within 1% either way).
+    const CUtensorMapL2promotion promotion = kCh32 || kMode == kModeTmaPad
+                                                 ? CU_TENSOR_MAP_L2_PROMOTION_NONE
+                                                 : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
     CUresult cr;
     if (t.im2col) {
       // base positions [-pad, size - 1 + pad - (kernel - 1)] in steps of the stride
@@ -1869,7 +1893,7 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
       cr = get_encode_im2col()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
                                const_cast<void*>(p.x), gdim, gstride, lower, upper, channels,
                                (cuuint32_t)t.T, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               promotion,
                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     } else {
       const cuuint32_t box[4] = {channels, (cuuint32_t)(t.bw * p.sw), (cuuint32_t)(t.bh * p.sh),
@@ -1879,7 +1903,7 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
       cr = get_encode_tiled()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
                               const_cast<void*>(p.x), gdim, gstride, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              promotion,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "tensor map of x failed (%d)", (int)cr);
