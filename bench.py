@@ -87,7 +87,7 @@ WORKLOADS = {
 CONV_TRAFFIC = {"sources": ["paper_1701_00485_gb300/csrc/tbn_conv_igemm.cuh",
                             "paper_1701_00485_gb300/csrc/tbn_conv_igemm.cu",
                             "paper_1701_00485_gb300/csrc/tbn_device.cuh"],
-                "sha256_16": "2edd57ba5c2ffeed", "bytes_per_launch": 48.08e6}
+                "sha256_16": "aa3fc36135142804", "bytes_per_launch": 48.04e6}
 
 
 def measured_traffic(rec):
@@ -316,7 +316,7 @@ def net_spec(name, dev, batch=None):
             kernel_desc = "conv_igemm_kernel (tcgen05 implicit GEMM): conv1 (space-to-depth " \
                           "input, filter resident in tensor memory), " \
                           "conv2 (32-channel TMA), conv3-5, fc6-8 (1x1, split K; their " \
-                          "ordered split sums included in the chain time)"
+                          "ranges added within clusters)"
         else:
             flops = net.flops
             cfg = {"workload": "vgg_small_b128_cifar", "global_batch": N, "image": [3, 32, 32],
@@ -734,7 +734,8 @@ def run_fused_quant_conv(args, local_rank, reps=5):
 # ------------------------------------------------------------------ backward
 def run_backward(args, rank, world, local_rank):
     """TwoBitBackward for every VGG-small layer: dx (tensor-core forward
-    kernels on the transposed filters) and dW^ (CUDA-core fp32 kernel)."""
+    kernels on the transposed filters) and dW^ (tensor cores, fp32
+    accumulation)."""
     import paper_1701_00485_gb300 as tbn
     from paper_1701_00485_gb300 import inputs
     torch.cuda.set_device(local_rank)
@@ -829,8 +830,8 @@ def run_backward(args, rank, world, local_rank):
             "per_layer_us": per_layer,
             "roofline": {"bound": "tensor", "achieved": round(filt_tf, 3), "peak": bf16_peak,
                          "unit": "TFLOP/s", "frac": round(filt_tf / bf16_peak, 4), "traffic": None,
-                         "kernel": "bwd_filter_tc_kernel (tcgen05 M128 N128 bf16, accumulator "
-                                   "in tensor memory, cp.async ring; c1: bwd_filter_kernel on "
+                         "kernel": "bwd_filter_tma_kernel (tcgen05 bf16, two accumulators in "
+                                   "tensor memory, TMA ring; c1: bwd_filter_kernel on "
                                    "mma.sync), 6 launches + slice reductions",
                          "peak_kind": "%s bf16 dense, %s" % (peak_kind, which),
                          "input_grad_vs_bf16_peak": round(gflop_data / ms_data / bf16_peak, 4)},

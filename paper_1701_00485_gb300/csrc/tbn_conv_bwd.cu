@@ -13,11 +13,11 @@
 // * Filter gradient dW^[k, r, s, c] = sum over (n, p, q) of dy[n, p, q, k]
 //   x[n, p sigma - pad + r, q sigma - pad + s, c]: a product of dy^T
 //   (K x pixels) and the im2col view of x (pixels x R S C).  Each CTA
-//   computes a tile over a slice of the pixels: 128 x 128 on tcgen05 with
-//   the accumulator in tensor memory when K and C are multiples of 8, else
-//   64 x 64 on mma.sync (bf16 products exact, fp32 accumulation); a second
-//   kernel adds the slices in a fixed order, so results are bitwise
-//   reproducible.
+//   computes a tile over a slice of the pixels on tcgen05 with the accumulator
+//   in tensor memory when K and C are multiples of 8 (operands by TMA where
+//   im2col boxes can fetch x, else by cp.async), and 64 x 64 on mma.sync
+//   otherwise (bf16 products exact, fp32 accumulation); a second kernel adds
+//   the slices in a fixed order, so results are bitwise reproducible.
 #include <cuda_bf16.h>
 
 #include <algorithm>

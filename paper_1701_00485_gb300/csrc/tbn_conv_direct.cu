@@ -3,11 +3,11 @@
 // (NHWC max pooling with optional padding, NCHW -> NHWC with channel padding).
 //
 // Direct convolution: a CTA computes 128 output pixels x 32 filters (8 where
-// that would leave SMs without a CTA).  The
-// filters' codes are decoded once per CTA into shared memory as fp32 W~ (a
-// chunk of taps at a time, tap-major so that all threads read the same
-// 32 weights -- a broadcast); each thread owns one pixel, walks the taps in
-// the codes' order, loads one activation per tap and does 32 FMAs.  This is
+// that would leave SMs without a CTA).  The filters' codes are decoded once
+// per CTA into shared memory as fp32 W~ (a chunk of taps at a time, tap-major
+// so that all threads read the same weights -- a broadcast); each thread owns
+// one pixel, walks the taps in the codes' order, loads eight taps'
+// activations ahead and does one FMA per tap and filter.  This is
 // the path for small-channel layers (the first layer of a network, where
 // the implicit GEMM would pad C up to its tile) and the fallback for shapes
 // the tensor-core kernel does not take.  x * W~ is exact in fp32; the sum is

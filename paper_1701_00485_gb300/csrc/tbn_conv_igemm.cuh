@@ -1,8 +1,9 @@
 // tbn_conv_igemm.cuh -- the tcgen05 implicit-GEMM kernel of the two-bit
 // convolution (Eq. 1, Section 2) and its launch, shared by the translation
-// units that instantiate it (tbn_conv_igemm.cu: host dispatch and the
-// gathering modes; tbn_conv_igemm_tma64.cu / _tma32.cu: the TMA modes with
-// and without fused quantization), so that its variants compile in parallel.
+// units that instantiate it (tbn_conv_igemm.cu: host dispatch, the gathering
+// and space-to-depth modes; tbn_conv_igemm_tma64.cu / _tma32.cu: the TMA modes
+// with and without fused quantization; tbn_conv_igemm_pad.cu: padded channels
+// and row pairs), so that its variants compile in parallel.
 //
 //
 // GEMM view of one tile:  D[128 filters x T pixels] = A[128 x n] * B[n x T]
@@ -43,10 +44,11 @@
 //                   lane = filter, column = pixel, multiply by 2 * alpha (Eq. 1
 //                   applies alpha to the whole filter; the factor 2 undoes the
 //                   W~/2 encoding -- exact scalings), add the optional
-//                   residual, apply ReLU and the optional 2x2 max pool, round
-//                   to bf16 into a shared-memory staging tile laid out as the
-//                   NHWC output box, and one TMA bulk tensor store writes the
-//                   box (clipped at the tensor's edges).  The accumulator is
+//                   residual (loaded by TMA to where its outputs are staged),
+//                   apply ReLU and the optional 2x2 max pool, round to bf16
+//                   into a shared-memory staging tile laid out as the NHWC
+//                   output box, and TMA tensor stores write the box (clipped
+//                   at the tensor's edges).  The accumulator is
 //                   released as soon as it has been read, before the staging
 //                   writes and the store complete.
 //
@@ -62,7 +64,8 @@
 //                 issuing thread delivers tiled boxes at a limited rate, so
 //                 several keep the activation ring fuller
 //   warp 1        TMEM allocator + MMA issuer
-//   warps 2-9     expanders
+//   warps 2-9     expanders (in space-to-depth mode, done with the filter
+//                 after the first tile, they join the epilogue)
 //   warps 10-17   epilogue
 //   warps 18-21   gather producers (gather mode only)
 // Every wait is bounded (tbn_device.cuh); on a timeout the CTA records the
@@ -403,8 +406,8 @@ __device__ __forceinline__ void add_cluster_sums(const IgArgs& a) {
 }
 
 // kPoolBW: 0 = no pool; 8, 16, 32 = fused 2x2/2 max pool for tiles of whole
-// output rows of that width; 1 = of any width (a.bw).  kTmaStore: bf16 output through the staging
-// tile and TMA stores (else direct global stores).
+// output rows of that width; 1 = of any width (a.bw).  kTmaStore: bf16 output
+// through the staging tile and TMA stores (else direct global stores).
 // Fused quantization prologue: CTA b quantizes filters [b K / G, (b + 1) K / G)
 // exactly as the quantize kernel does (the same per-word fields and sums,
 // reduced per filter in the same order: bitwise the same codes and alpha),
@@ -1745,7 +1748,9 @@ inline bool use_tma_store(const ConvProblem& p) {
 // stride 1 down the rows, an even number of output rows of at most a tile's
 // width, whole 64-channel boxes, and the staged bf16 epilogue.  It pays for
 // filters of several rows: 3 x 3 over 64 channels takes 12 K blocks for two
-// output rows instead of 18 (56 x 56, batch 64, with shortcut: see plan_conv).
+// output rows instead of 18 (56 x 56 with shortcut, 64 filters, batch 64: 27.5 ->
+// 24.5 us; the ResNet-18 step at batch 128: 602 -> 574); plan_cost decides by
+// the K blocks.
 inline bool rowpair_ok(const ConvProblem& p) {
   return p.C % kBK == 0 && p.K <= kBM / 2 && p.sh == 1 && p.sw <= 2 && p.P % 2 == 0 && p.R >= 2 &&
          p.R < 128 && p.Q <= kMaxTileN && !p.pool && p.wq == nullptr && use_tma_store(p);
@@ -1758,9 +1763,10 @@ inline bool rowpair_ok(const ConvProblem& p) {
 // tile.  Whole-image tiles leave the last wave nearly empty (13 x 13 images,
 // 384 filters, batch 256: 768 tiles on 152 SMs, six waves for 5.05) or their
 // columns short of 256; runs of pixels are cut to the machine instead:
-// four waves of 224 (that layer at 1152 codes per filter: 63.9 -> 50.6 us,
-// at 3456: 91.4 -> 69.7; the AlexNet step at batch 256: 680 -> 627 us).  `resident`: the space-to-depth mode, whose K blocks
-// stay beside the accumulator.
+// four waves of 224 (that layer at 2304 codes per filter: 63.9 -> 50.6 us,
+// at 3456: 91.4 -> 69.7; the AlexNet step at batch 256: 680 -> 627 us).
+// `resident`: the space-to-depth mode, whose K blocks stay beside the
+// accumulator.
 inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
   TilePlan best = plan_tiles(p);
   if (!tma_fed(p) || p.ksplit > 1) return best;

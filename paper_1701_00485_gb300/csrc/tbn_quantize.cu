@@ -17,9 +17,8 @@
 // in W, at most 2048 words = 128 KB) through a ring of three 32 KB shared-
 // memory stages filled by 1-D TMA bulk copies (thread 0 keeps three in
 // flight, every wait bounded); other tasks are staged there 4 bytes at a time
-// (at most 1024 words), and a
-// filter longer than 2048 words is a task of its own with its words strided
-// over the threads.
+// (at most 1024 words), and a filter longer than 2048 words is a task of its
+// own with its words strided over the threads.
 //
 // The word sums are accumulated exactly as a two-float (hi, lo) pair
 // (TwoSum, fp32 adds only: GB300's fp64 rate is a small fraction of its fp32

@@ -175,7 +175,10 @@ class FCStack:
             y = torch.empty((batch, kout), dtype=torch.bfloat16, device=self.device)
             self.layers.append((W, codes, alpha, relu, y))
             need = tbn_linear_workspace_bytes(batch, kin, kout)
-            self.launches += 2 if need > 0 else 1     # split K adds the ordered sum
+            # one launch: with split K the clusters add their ranges themselves
+            # (filters of very many ranges, which these networks do not have,
+            # add the sums in a second launch)
+            self.launches += 1
             ws = max(ws, need)
         self.workspace = (torch.empty(ws, dtype=torch.uint8, device=self.device)
                           if ws > 0 else None)
