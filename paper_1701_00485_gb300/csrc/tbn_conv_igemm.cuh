@@ -1025,6 +1025,9 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     int issued = 0, st = 0;
     uint32_t tiles_done = 0, par = 0;
     const int tap_blocks = (a.C + kBK - 1) / kBK;   // padded mode: K blocks per tap
+    // space-to-depth mode: K steps that hold channels (the others are zero in
+    // both operands; AlexNet conv1, batch 256, three of four: 83.8 -> 79.4 us)
+    const int s2d_steps = (a.s2d_s * a.s2d_s * a.s2d_C + 15) / 16;
     bool ok = true;
     for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++tiles_done) {
       const TileCoord tc = tile_coord(a, t);
@@ -1050,7 +1053,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         constexpr uint32_t kHalf = kCh32 ? (kStageBytes / 2) >> 4 : 4u;
         tc_mma_ts_block<2, kHalf, kHalf + 2>(
             acc_t, a_col, kCh32 ? smem_desc_sw64_kmajor(b_addr) : smem_desc_sw128_kmajor(b_addr),
-            idesc, kb != tc.kb0 ? 1u : 0u, kPad ? (left + 15) / 16 : 4, &ctl->empty[st],
+            idesc, kb != tc.kb0 ? 1u : 0u, kPad ? (left + 15) / 16 : kS2d ? s2d_steps : 4, &ctl->empty[st],
             kb == tc.kb1 - 1 ? &ctl->acc_full[ab] : nullptr);
         if (kPad) left = left > kBK ? left - kBK : a.C;
         ++issued;
