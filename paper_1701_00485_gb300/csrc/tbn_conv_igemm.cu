@@ -209,7 +209,8 @@ bool conv_igemm_pools_any_width(const ConvProblem& p) {
 tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const bool s2d = p0.layout == TBN_S2D_NHWC;
   const ConvProblem p = s2d ? s2d_problem(p0) : p0;
-  TilePlan t = plan_conv(p, s2d);
+  const int resident = s2d ? 8 * ceil_div(p0.sh * p0.sh * p0.C, 16) : 0;
+  TilePlan t = plan_conv(p, resident);
   const bool split = p.ksplit > 1 && p.partial != nullptr;
   const int cluster = split && is_aligned(p.partial, 16) ? cluster_split(p, t) : 1;
   IgArgs a{};
@@ -253,7 +254,7 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
     a.s2d_R = static_cast<int>(p0.R);
     a.s2d_S = static_cast<int>(p0.S);
     if (split || a.tiles_k != 1 || a.kblocks > kMaxResidentKB ||
-        t.tile_n + 32 * a.kblocks > kTmemCols || p.pool || p.residual)
+        t.tile_n + resident * a.kblocks > kTmemCols || p.pool || p.residual)
       return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: space-to-depth problem out of range");
   }
   // tiles of at most 176 pixels: two accumulators, so each tile's MMAs

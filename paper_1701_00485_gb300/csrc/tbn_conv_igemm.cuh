@@ -203,7 +203,7 @@ constexpr int kModeTmaPad = 5;  // 64-channel TMA boxes, each tap's last one pad
 // half the MMA's rows empty; the tap row that a half does not have is a
 // block of zero weights.
 constexpr int kModeRowPair = 6;
-constexpr int kMaxResidentKB = 15;   // resident K blocks: 32 columns each beside the accumulator
+constexpr int kMaxResidentKB = 15;   // resident K blocks: up to 32 columns each beside the accumulator
 
 __host__ __device__ constexpr bool mode_gathers(int mode) {
   return mode == kModeGather || mode == kModePatch;
@@ -1045,7 +1045,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         if (!ok) break;
         tc_fence_after_sync();
         const uint32_t a_col =
-            kS2d ? static_cast<uint32_t>(kTmemCols - 32 * KB + 32 * kb)
+            kS2d ? static_cast<uint32_t>(kTmemCols - 8 * s2d_steps * (KB - kb))
                  : a_tmem0 + static_cast<uint32_t>(st * kAColsPerStage);
         // K step kk: 16 codes = 8 TMEM columns of A, 32 bytes of B rows (two
         // halves of 32 codes, 64-byte rows, with 32-channel boxes)
@@ -1076,12 +1076,14 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     const int m = sub * 32 + lane;                    // filter row within the tile
     const uint32_t lane_off = static_cast<uint32_t>(sub * 32) << 16;
     if constexpr (kS2d) {
-      // Decode every K block of the filter once into its resident columns
-      // [512 - 32 KB + 32 kb, + 32) (this warp: codes [32 half, + 32) of
-      // each, i.e. 16 columns).  Filter rows past K hold zeros.
+      // Decode every K block of the filter once into its resident columns,
+      // the last of which end at 512: eight for each K step that holds
+      // channels (this warp: those of codes [32 half, + 32)).  Filter rows
+      // past K hold zeros.
       const uint32_t* tab = reinterpret_cast<const uint32_t*>(out_stage);
       const uint32_t* crow = m < a.K ? a.codes + static_cast<size_t>(m) * a.wpf : nullptr;
-      const uint32_t res0 = static_cast<uint32_t>(kTmemCols - 32 * KB);
+      const int cols = 8 * ((a.s2d_s * a.s2d_s * a.s2d_C + 15) / 16);
+      const int part = min(16, cols - 16 * half);   // 16, 8 or none
       for (int kb = 0; kb < KB; ++kb) {
         uint32_t v[16];
 #pragma unroll
@@ -1096,7 +1098,10 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
             hi = ((__ldg(crow + (e1 & 0xFFFFu)) >> (e1 >> 16)) & 0x101u) * 128u + 0x3F00u;
           v[i] = lo | (hi << 16);
         }
-        tmem_st_32x32b_x16(tmem + lane_off + res0 + static_cast<uint32_t>(32 * kb + 16 * half), v);
+        const uint32_t col =
+            tmem + lane_off + static_cast<uint32_t>(kTmemCols - cols * (KB - kb) + 16 * half);
+        if (part == 16) tmem_st_32x32b_x16(col, v);
+        else if (part == 8) tmem_st_32x32b_x8(col, v);
         tmem_wait_st();
         tc_fence_before_sync();
         mbar_arrive(&ctl->wready[kb]);
@@ -1768,9 +1773,12 @@ inline bool rowpair_ok(const ConvProblem& p) {
 // columns short of 256; runs of pixels are cut to the machine instead:
 // four waves of 224 (that layer at 2304 codes per filter: 63.9 -> 50.6 us,
 // at 3456: 91.4 -> 69.7; the AlexNet step at batch 256: 680 -> 627 us).
-// `resident`: the space-to-depth mode, whose K blocks stay beside the
-// accumulator.
-inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
+// `resident`: columns of tensor memory that each K block takes in the
+// space-to-depth mode, where they all stay beside the accumulator (else 0).
+// 24 instead of 32 columns for 48 channels leave room for tiles of 256 pixels
+// instead of 224 (AlexNet conv1, batch 256: 79.4 -> 76.8 us; two accumulators
+// beside them, of 144 pixels each, take 82 even with eight ring stages).
+inline TilePlan plan_conv(const ConvProblem& p, int resident) {
   TilePlan best = plan_tiles(p);
   if (!tma_fed(p) || p.ksplit > 1) return best;
   const int sms = device_sm_count();
@@ -1783,7 +1791,7 @@ inline TilePlan plan_conv(const ConvProblem& p, bool resident) {
     }
   };
   const int kb = ceil_div(p.C * p.R * p.S, kBK);
-  const int t_max = resident ? std::min(kMaxTileN, kTmemCols - 32 * kb) : kMaxTileN;
+  const int t_max = resident ? std::min(kMaxTileN, kTmemCols - resident * kb) : kMaxTileN;
   if (im2col_ok(p)) {
     TilePlan t = best;
     t.im2col = true;

@@ -139,3 +139,16 @@ def test_space_to_depth_conv_refuses_unsupported(bad):
     with pytest.raises((tbn.TBNError, ValueError)):
         tbn.tbn_conv2d_fwd(xs, codes, alpha, K, R, S, stride, (0, 0), layout=tbn.TBN_S2D_NHWC,
                            in_chw=(C, H, W))
+
+
+@pytest.mark.parametrize("C,s", [(1, 2), (4, 2), (5, 2), (8, 2), (3, 4), (13, 2), (7, 3)])
+def test_space_to_depth_conv_channel_steps(C, s):
+    """One to four K steps of 16 channels per resident K block, enough pixels
+    for tiles of consecutive pixels over several images."""
+    g = inputs.generator(100 * C + s)
+    x = torch.randn(6, C, 37 * s // 2, 41 * s // 2, generator=g)
+    c = ConvCase(x, inputs.normal((72, C, 2 * s + 1, 2 * s + 1), 1.3, g), (s, s), (1, 0))
+    y = _run_s2d(c, torch.bfloat16)
+    sites = random_sites(y.shape, 3000, seed=C)
+    y_orc, bound = c.oracle_sites(torch.bfloat16, sites)
+    assert_within(y[tuple(sites.T)], y_orc, bound, out_bf16=True, what="s2d steps %s" % ((C, s),))
