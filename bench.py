@@ -87,7 +87,7 @@ WORKLOADS = {
 CONV_TRAFFIC = {"sources": ["paper_1701_00485_gb300/csrc/tbn_conv_igemm.cuh",
                             "paper_1701_00485_gb300/csrc/tbn_conv_igemm.cu",
                             "paper_1701_00485_gb300/csrc/tbn_device.cuh"],
-                "sha256_16": "aa3fc36135142804", "bytes_per_launch": 48.04e6}
+                "sha256_16": "2bedd746d0760c87", "bytes_per_launch": 47.88e6}
 
 
 def measured_traffic(rec):
