@@ -88,6 +88,18 @@ int cluster_split(const ConvProblem& p, TilePlan& t) {
   return best;
 }
 
+// Whether a layer of 64 m + 32 channels runs on tap pairs instead of pairs of
+// 32-channel boxes: on the widest tiles the boxes' rows set the pace of a K
+// block (256 pixels: 96 -> 256 channels, 27 x 27, 5 x 5, batch 256, 137 -> 128
+// us; 160 -> 256, 3 x 3, 92.0 -> 87.7; 416 -> 384, 14 x 14, 3 x 3, 83.6 ->
+// 78.5).  Narrower ones are paced by the warps' own instructions, of which the
+// pairs take more (224 pixels: 224 -> 512 channels, 14 x 14, 65.5 and 65.2; 160
+// -> 384, 13 x 13, 5 x 5, 77.2 and 80.8; 160 pixels: 96 -> 128, 27 x 27, 5 x
+// 5, batch 32, 13.9 and 15.4).
+bool tap_pairs_pay(const ConvProblem& p, const TilePlan& t) {
+  return p.C > kBK && t.tile_n > 224 && p.R * p.S > 1;
+}
+
 // Patch mode (gathered activations staged per tile in shared memory) when a
 // tile is whole output rows of one image, the filter spans at most
 // kPatchMaxKBlocks K blocks and two patches fit beside the ring.
@@ -304,6 +316,8 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
                : launch_t<kModeS2d, 0, false, false>(p, t, a, s);
   }
   if (t.rowpair) return launch_igemm_rowpair(p, t, a, s);
+  if (use_tma(p) && use_ch32(p) && tap_pairs_pay(p, t))
+    return launch_igemm_tappair(p, t, a, pw, tst, a.wq != nullptr, s);
   if (use_tma(p) && use_ch32(p)) {
     return launch_igemm_tma32(p, t, a, pw, tst, a.wq != nullptr, s);
   }

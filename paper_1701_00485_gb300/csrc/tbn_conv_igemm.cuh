@@ -203,6 +203,11 @@ constexpr int kModeTmaPad = 5;  // 64-channel TMA boxes, each tap's last one pad
 // half the MMA's rows empty; the tap row that a half does not have is a
 // block of zero weights.
 constexpr int kModeRowPair = 6;
+// Tap pairs (C = 64 m + 32, m >= 1): the K blocks of two taps are each tap's m
+// whole 64-channel boxes, then one block of both taps' last 32 channels, so
+// that 4 m + 2 boxes of 64-byte rows become 2 m boxes of 128-byte rows and two
+// of 64: the boxes' rows are what paces wide tiles (see tap_pairs_pay).
+constexpr int kModeTapPair = 7;
 constexpr int kMaxResidentKB = 15;   // resident K blocks: up to 32 columns each beside the accumulator
 
 __host__ __device__ constexpr bool mode_gathers(int mode) {
@@ -519,6 +524,24 @@ __device__ void quantize_prologue(const IgArgs& a, uint8_t* scratch, int scratch
   __syncthreads();
 }
 
+// Place in the K blocks of the tap pairs (kModeTapPair); the last tap of an odd
+// number has no partner.
+struct TapPairs {
+  int m, taps;
+  int g, j, na;   // pair, K block within it, 64-channel blocks of the pair
+  __device__ __forceinline__ explicit TapPairs(const IgArgs& a)
+      : m(a.C / kBK), taps(a.R * a.S), g(0), j(0), na(taps > 1 ? 2 * m : m) {}
+  __device__ __forceinline__ bool whole() const { return j < na; }   // a 64-channel block
+  __device__ __forceinline__ int second() const { return j >= m ? 1 : 0; }   // of the second tap
+  __device__ __forceinline__ void next() {
+    if (++j > na) {
+      j = 0;
+      ++g;
+      na = 2 * g + 1 < taps ? 2 * m : m;
+    }
+  }
+};
+
 // kMode: how activations reach the ring (kModeTma64 / kModeTma32 /
 // kModeGather / kModePatch).
 template <int kMode, int kPoolBW, bool kTmaStore, bool kFuse>
@@ -526,6 +549,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     conv_igemm_kernel(const __grid_constant__ CUtensorMap tmap_x,
                       const __grid_constant__ CUtensorMap tmap_y,
                       const __grid_constant__ CUtensorMap tmap_res,
+                      const __grid_constant__ CUtensorMap tmap_x32,
                       const __grid_constant__ IgArgs a) {
   constexpr bool kGather = mode_gathers(kMode);
   constexpr bool kCh32 = kMode == kModeTma32;
@@ -533,6 +557,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
   constexpr bool kS2d = kMode == kModeS2d;
   constexpr bool kPad = kMode == kModeTmaPad;
   constexpr bool kRowPair = kMode == kModeRowPair;
+  constexpr bool kTapPair = kMode == kModeTapPair;
   constexpr bool kCanCluster = kPoolBW == 0 && !kTmaStore && !kFuse &&
                                (kMode == kModeTma64 || kMode == kModeTma32 || kPad);
   constexpr int kSt = stages_for(kMode);   // ring stages
@@ -571,6 +596,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     ctl->abort = 0;
     fence_mbar_init();
     if (!kGather) prefetch_tmap(&tmap_x);
+    if (kTapPair) prefetch_tmap(&tmap_x32);
     if (kTmaStore) prefetch_tmap(&tmap_y);
   }
   if (warp == 1) {
@@ -667,6 +693,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
           }
         }
       };
+      TapPairs tp(a);   // (r, q): the pair's first tap
       for (int kb = tc.kb0; kb < tc.kb1; ++kb, ++g) {
         const int sb = st;
         const uint32_t ph = par;
@@ -679,7 +706,31 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         if (mine) {
           ok = mbar_wait_warp(&ctl->empty[sb], ph ^ 1u, abort_flag, a.err, kWaitLimitNs);
           if (!ok) break;
-          if (elect_one()) {
+          if (kTapPair && elect_one()) {
+            mbar_arrive_expect_tx(&ctl->full[sb], box_bytes * kBoxes);
+            const bool wrap = q + 1 == a.S;
+            const int q1 = wrap ? 0 : q + 1, r1 = wrap ? r + 1 : r;
+            const auto box = [&](uint8_t* dst, const CUtensorMap* map, int c0, int dr, int dq) {
+              // past the last tap: entirely out of range, it arrives zero-filled
+              if (dr >= a.R) {
+                c0 = a.C;
+                dr = dq = 0;
+              }
+              if (a.im2col)
+                tma_load_im2col_4d(dst, map, &ctl->full[sb], c0, w0, h0, n0, dq, dr);
+              else
+                tma_load_4d(dst, map, &ctl->full[sb], c0, w0 + dq, h0 + dr, n0);
+            };
+            uint8_t* dst = ring + sb * kStageBytes;
+            if (tp.whole()) {
+              const bool s = tp.second();
+              box(dst, &tmap_x, kBK * (tp.j - (s ? tp.m : 0)), s ? r1 : r, s ? q1 : q);
+            } else {
+              box(dst, &tmap_x32, kBK * tp.m, r, q);
+              box(dst + kStageBytes / 2, &tmap_x32, kBK * tp.m, r1, q1);
+            }
+          }
+          if (!kTapPair && elect_one()) {
             mbar_arrive_expect_tx(&ctl->full[sb], box_bytes * kBoxes);
             int cb_ = cb, r_ = r, q_ = q;
 #pragma unroll
@@ -705,8 +756,19 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
           }
           __syncwarp();
         }
+        if constexpr (kTapPair) {
+          tp.next();
+          if (tp.j == 0) {
+            q += 2;
+            while (q >= a.S) {
+              q -= a.S;
+              ++r;
+            }
+          }
+        } else {
 #pragma unroll
-        for (int bx = 0; bx < kBoxes; ++bx) next_box();
+          for (int bx = 0; bx < kBoxes; ++bx) next_box();
+        }
       }
     }
     // drain: every copy this warp issued must land before the CTA may exit
@@ -1037,6 +1099,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const uint32_t acc_t = acc_tmem + ab * kAcc2Cols;
       ok = mbar_wait_warp(&ctl->acc_empty[ab], (use & 1u) ^ 1u, abort_flag, a.err, kWaitLimitNs);
       if (!ok) break;
+      TapPairs tp(a);
       int left = kPad ? a.C - kBK * (tc.kb0 % tap_blocks) : kBK;   // channels left in the tap
       for (int kb = tc.kb0; kb < tc.kb1; ++kb) {
         ok = mbar_wait_warp(&ctl->full[st], par, abort_flag, a.err, kWaitLimitNs);
@@ -1051,11 +1114,16 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         // halves of 32 codes, 64-byte rows, with 32-channel boxes)
         const uint32_t b_addr = smem_addr(ring) + static_cast<uint32_t>(st * kStageBytes);
         constexpr uint32_t kHalf = kCh32 ? (kStageBytes / 2) >> 4 : 4u;
-        tc_mma_ts_block<2, kHalf, kHalf + 2>(
+        if (kTapPair && !tp.whole())
+          tc_mma_ts_block<2, (kStageBytes / 2 >> 4), (kStageBytes / 2 >> 4) + 2>(
+              acc_t, a_col, smem_desc_sw64_kmajor(b_addr), idesc, kb != tc.kb0 ? 1u : 0u, 4,
+              &ctl->empty[st], kb == tc.kb1 - 1 ? &ctl->acc_full[ab] : nullptr);
+        else tc_mma_ts_block<2, kHalf, kHalf + 2>(
             acc_t, a_col, kCh32 ? smem_desc_sw64_kmajor(b_addr) : smem_desc_sw128_kmajor(b_addr),
             idesc, kb != tc.kb0 ? 1u : 0u, kPad ? (left + 15) / 16 : kS2d ? s2d_steps : 4, &ctl->empty[st],
             kb == tc.kb1 - 1 ? &ctl->acc_full[ab] : nullptr);
         if (kPad) left = left > kBK ? left - kBK : a.C;
+        if (kTapPair) tp.next();
         ++issued;
         if (++st == kSt) {
           st = 0;
@@ -1133,6 +1201,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     // padded mode: this half block's first code, and channels left in its tap
     const int tap_blocks = (a.C + kBK - 1) / kBK;
     int code0 = 0, ch_left = 0;
+    TapPairs tp(a);
     auto set_row = [&]() {
       const TileCoord tc = tile_coord(a, t_ld < a.tiles ? t_ld : 0);
       kb_ld = tc.kb0;
@@ -1150,6 +1219,12 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         const int tap = kb_ld / tap_blocks, cb = kb_ld - tap * tap_blocks;
         ch_left = a.C - kBK * cb;
         code0 = tap * a.C + kBK * cb + 32 * half;
+        kb_lim = in ? kb_end : 0;
+        cp = a.codes + static_cast<size_t>(in ? k : 0) * a.wpf;
+        return;
+      }
+      if constexpr (kTapPair) {
+        tp = TapPairs(a);
         kb_lim = in ? kb_end : 0;
         cp = a.codes + static_cast<size_t>(in ? k : 0) * a.wpf;
         return;
@@ -1203,23 +1278,34 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         }
         return r;
       }
-      if (kb_ld < kb_lim && (!kRowPair || kb_ld >= 0)) {
+      // tap pairs: the words of the block's tap (4 m + 2 each)
+      const uint32_t* wp = cp;
+      bool there = true;
+      if constexpr (kTapPair) {
+        const bool w = tp.whole();
+        const int s = w ? tp.second() : half;
+        wp += (2 * tp.g + s) * (4 * tp.m + 2) + 4 * (w ? tp.j - (s ? tp.m : 0) : tp.m) +
+              (w ? 2 * half : 0);
+        there = 2 * tp.g + s < tp.taps;
+        tp.next();
+      }
+      if (there && kb_ld < kb_lim && (!kRowPair || kb_ld >= 0)) {
         // written by this launch's prologue when fused: ordinary (L1-cached,
         // coherent) loads after the grid barrier's acquire then, not the
         // read-only path, which assumes data constant for the whole launch
-        const bool two = 4 * kb_ld + 2 * half + 1 < a.wpf;
+        const bool two = kTapPair || 4 * kb_ld + 2 * half + 1 < a.wpf;
         uint2 t;
         if constexpr (kFuse) {
-          if (pair_ok) t = __ldca(reinterpret_cast<const uint2*>(cp));
-          else t = make_uint2(__ldca(cp), two ? __ldca(cp + 1) : 0u);
+          if (pair_ok) t = __ldca(reinterpret_cast<const uint2*>(wp));
+          else t = make_uint2(__ldca(wp), two ? __ldca(wp + 1) : 0u);
         } else {
-          if (pair_ok) t = __ldg(reinterpret_cast<const uint2*>(cp));
-          else t = make_uint2(__ldg(cp), two ? __ldg(cp + 1) : 0u);
+          if (pair_ok) t = __ldg(reinterpret_cast<const uint2*>(wp));
+          else t = make_uint2(__ldg(wp), two ? __ldg(wp + 1) : 0u);
         }
         r.x = t.x;
         r.y = t.y;
       }
-      cp += 4;
+      if constexpr (!kTapPair) cp += 4;
       if (++kb_ld == kb_end) {
         t_ld += gridDim.x;
         set_row();
@@ -1881,10 +1967,11 @@ template <int kMode, int kPoolBW, bool kTmaStore, bool kFuse>
 tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStream_t s) {
   constexpr bool kGather = mode_gathers(kMode);
   constexpr bool kCh32 = kMode == kModeTma32;
-  alignas(64) CUtensorMap tmap_x, tmap_y, tmap_res;
+  alignas(64) CUtensorMap tmap_x, tmap_y, tmap_res, tmap_x32;
   std::memset(&tmap_x, 0, sizeof(tmap_x));
   std::memset(&tmap_y, 0, sizeof(tmap_y));
   std::memset(&tmap_res, 0, sizeof(tmap_res));
+  std::memset(&tmap_x32, 0, sizeof(tmap_x32));
   if (!kGather) {
     const cuuint64_t gdim[4] = {(cuuint64_t)p.C, (cuuint64_t)p.W, (cuuint64_t)p.H, (cuuint64_t)p.N};
     const cuuint64_t gstride[3] = {(cuuint64_t)(p.C * 2), (cuuint64_t)(p.W * p.C * 2),
@@ -1892,37 +1979,37 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
     // row pairs: base rows two apart, R + 1 tap rows
     const int rp = t.rowpair ? 1 : 0;
     const cuuint32_t estr[4] = {1u, (cuuint32_t)p.sw, (cuuint32_t)(p.sh + rp), 1u};
-    const cuuint32_t channels = kCh32 ? kBK / 2 : kBK;
-    const CUtensorMapSwizzle swizzle = kCh32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
     // Boxes narrower than a pixel's channels, or than the 64 of a box, read
     // rows that do not fill 256-byte lines: promoting their requests to whole
     // ones reads beside what is wanted (27 x 27, batch 256, 96 -> 256 channels,
     // 5 x 5: 142 us so, 138 without; 40 -> 128 channels, batch 32, fp32 y: 26.3
     // and 22.2; layers of 64-channel boxes are within 1% either way).
-    const CUtensorMapL2promotion promotion = kCh32 || kMode == kModeTmaPad
+    const CUtensorMapL2promotion promotion = kCh32 || kMode == kModeTapPair || kMode == kModeTmaPad
                                                  ? CU_TENSOR_MAP_L2_PROMOTION_NONE
                                                  : CU_TENSOR_MAP_L2_PROMOTION_L2_256B;
-    CUresult cr;
-    if (t.im2col) {
-      // base positions [-pad, size - 1 + pad - (kernel - 1)] in steps of the stride
-      const int lower[2] = {-(int)p.pw, -(int)p.ph};
-      const int upper[2] = {(int)(p.pw - (p.S - 1)), (int)(p.ph - (p.R - 1)) - rp};
-      cr = get_encode_im2col()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
-                               const_cast<void*>(p.x), gdim, gstride, lower, upper, channels,
-                               (cuuint32_t)t.T, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-                               promotion,
-                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    } else {
-      const cuuint32_t box[4] = {channels, (cuuint32_t)(t.bw * p.sw), (cuuint32_t)(t.bh * p.sh),
-                                 (cuuint32_t)t.bn};
-      if (box[1] > 256 || box[2] > 256 || box[3] > 256)
-        return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: TMA box too large");
-      cr = get_encode_tiled()(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
-                              const_cast<void*>(p.x), gdim, gstride, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
-                              promotion,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
+    const cuuint32_t box[4] = {0u, (cuuint32_t)(t.bw * p.sw), (cuuint32_t)(t.bh * p.sh),
+                               (cuuint32_t)t.bn};
+    if (!t.im2col && (box[1] > 256 || box[2] > 256 || box[3] > 256))
+      return fail(TBN_ERR_UNSUPPORTED, "implicit GEMM: TMA box too large");
+    const auto encode = [&](CUtensorMap* m, cuuint32_t channels) {
+      const CUtensorMapSwizzle swizzle =
+          channels == kBK ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+      if (t.im2col) {
+        // base positions [-pad, size - 1 + pad - (kernel - 1)] in steps of the stride
+        const int lower[2] = {-(int)p.pw, -(int)p.ph};
+        const int upper[2] = {(int)(p.pw - (p.S - 1)), (int)(p.ph - (p.R - 1)) - rp};
+        return get_encode_im2col()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
+                                   const_cast<void*>(p.x), gdim, gstride, lower, upper, channels,
+                                   (cuuint32_t)t.T, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                                   promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      }
+      const cuuint32_t b[4] = {channels, box[1], box[2], box[3]};
+      return get_encode_tiled()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(p.x),
+                                gdim, gstride, b, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                                promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult cr = encode(&tmap_x, kCh32 ? kBK / 2 : kBK);
+    if (cr == CUDA_SUCCESS && kMode == kModeTapPair) cr = encode(&tmap_x32, kBK / 2);
     if (cr != CUDA_SUCCESS) return fail(TBN_ERR_CUDA, "tensor map of x failed (%d)", (int)cr);
   }
   if (kTmaStore) {
@@ -1980,7 +2067,7 @@ tbn_status launch_t(const ConvProblem& p, const TilePlan& t, IgArgs& a, cudaStre
     const cudaError_t me = cudaMemsetAsync(a.gbar, 0, sizeof(unsigned), s);
     if (me != cudaSuccess) return cuda_fail(me, "cudaMemsetAsync(barrier word)");
   }
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, tmap_x, tmap_y, tmap_res, a);
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, tmap_x, tmap_y, tmap_res, tmap_x32, a);
   if (le != cudaSuccess) return cuda_fail(le, "cudaLaunchKernelEx(conv_igemm_kernel)");
   return check_launch("conv_igemm_kernel");
 }
@@ -2013,6 +2100,8 @@ tbn_status launch_igemm_tma32(const ConvProblem& p, const TilePlan& t, IgArgs& a
                               bool tma_store, bool fuse, cudaStream_t s);
 tbn_status launch_igemm_pad(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
                             bool tma_store, cudaStream_t s);
+tbn_status launch_igemm_tappair(const ConvProblem& p, const TilePlan& t, IgArgs& a, int pw,
+                                bool tma_store, bool fuse, cudaStream_t s);
 tbn_status launch_igemm_rowpair(const ConvProblem& p, const TilePlan& t, IgArgs& a,
                                 cudaStream_t s);
 

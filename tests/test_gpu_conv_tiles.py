@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_1701_00485_gb300 as tbn
 from paper_1701_00485_gb300 import inputs
-from parity_util import ConvCase, assert_within
+from parity_util import ConvCase, assert_within, random_sites
 
 pytestmark = pytest.mark.gpu
 
@@ -122,6 +122,40 @@ def test_padded_linear(B, K_in, K_out):
     for w in {None, ws}:
         y = tbn.tbn_linear_fwd_ws(x.cuda(), codes, alpha, K_out, w, out_dtype=torch.float32)
         assert_within(y.cpu().numpy(), want, bound, out_bf16=False, what="padded linear")
+
+
+@pytest.mark.parametrize("case,pool", [
+    ((8, 96, 8, 8, 130, 3, 3, (1, 1), (1, 1)), 0),    # nine taps: the last has no partner
+    ((8, 96, 8, 8, 64, 3, 3, (1, 1), (1, 1)), 2),
+    ((4, 160, 8, 7, 72, 1, 2, (1, 1), (0, 1)), 0),    # one pair, two whole blocks a tap
+    ((8, 160, 7, 7, 40, 2, 4, (1, 1), (1, 2)), 0),    # pairs that end in the next row
+    ((4, 96, 15, 8, 24, 5, 5, (2, 1), (2, 2)), 0),   # strided
+    ((2, 224, 8, 16, 24, 3, 1, (1, 1), (1, 0)), 0),
+    ((256, 96, 27, 27, 256, 5, 5, (1, 1), (2, 2)), 0),   # runs of pixels
+])
+def test_tap_pairs(case, pool):
+    """64 m + 32 channels on tiles of 256 pixels: K blocks of tap pairs."""
+    c = _case(*case, seed=sum(case[:7]))
+    N, C, H, W, K, R, S, st, pad = case
+    Wl, codes, alpha = c.quantize_gpu(tbn.TBN_NHWC)
+    x = c.x.to(torch.bfloat16).permute(0, 2, 3, 1).contiguous().cuda()
+    for dt in (torch.float32, torch.bfloat16):
+        y = tbn.tbn_conv2d_fwd(x, codes, alpha, K, R, S, st, pad, out_dtype=dt, relu=bool(pool),
+                               pool=pool)
+        assert tbn.tbn_device_error() == 0
+        got = y.float().cpu().permute(0, 3, 1, 2).contiguous().numpy()
+        if N > 64:
+            sites = random_sites(got.shape, 2000, seed=5)
+            want, bound = c.oracle_sites(torch.bfloat16, sites)
+            got = got[tuple(sites.T)]
+        else:
+            want, bound = c.oracle_full(torch.bfloat16)
+            if pool:
+                P, Q = want.shape[2] // 2, want.shape[3] // 2
+                want = oracle.maxpool2d_nchw(oracle.epilogue(want, None, relu=True), (2, 2), (2, 2))
+                bound = bound[:, :, :2 * P, :2 * Q].reshape(N, K, P, 2, Q, 2).max(axis=(3, 5))
+        assert_within(got, want, bound, out_bf16=dt == torch.bfloat16, epilogue=bool(pool),
+                      what="tap pairs %s" % (case,))
 
 
 @pytest.mark.parametrize("B,K_in,K_out,dtype,res", [
