@@ -87,7 +87,7 @@ WORKLOADS = {
 CONV_TRAFFIC = {"sources": ["paper_1701_00485_gb300/csrc/tbn_conv_igemm.cuh",
                             "paper_1701_00485_gb300/csrc/tbn_conv_igemm.cu",
                             "paper_1701_00485_gb300/csrc/tbn_device.cuh"],
-                "sha256_16": "2bedd746d0760c87", "bytes_per_launch": 47.88e6}
+                "sha256_16": "903afa2b252578e8", "bytes_per_launch": 47.82e6}
 
 
 def measured_traffic(rec):
@@ -315,7 +315,7 @@ def net_spec(name, dev, batch=None):
                    "requantize_per_step": True}
             kernel_desc = "conv_igemm_kernel (tcgen05 implicit GEMM): conv1 (space-to-depth " \
                           "input, filter resident in tensor memory), " \
-                          "conv2 (32-channel TMA), conv3-5, fc6-8 (1x1, split K; their " \
+                          "conv2 (tap pairs), conv3-5, fc6-8 (1x1, split K; their " \
                           "ranges added within clusters)"
         else:
             flops = net.flops

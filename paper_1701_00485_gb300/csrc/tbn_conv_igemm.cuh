@@ -2,8 +2,8 @@
 // convolution (Eq. 1, Section 2) and its launch, shared by the translation
 // units that instantiate it (tbn_conv_igemm.cu: host dispatch, the gathering
 // and space-to-depth modes; tbn_conv_igemm_tma64.cu / _tma32.cu: the TMA modes
-// with and without fused quantization; tbn_conv_igemm_pad.cu: padded channels
-// and row pairs), so that its variants compile in parallel.
+// with and without fused quantization; tbn_conv_igemm_pair.cu: tap pairs;
+// tbn_conv_igemm_pad.cu: padded channels and row pairs), so that its variants compile in parallel.
 //
 //
 // GEMM view of one tile:  D[128 filters x T pixels] = A[128 x n] * B[n x T]
@@ -33,7 +33,10 @@
 //                   boxes of 32 channels, each from its own tap, into two
 //                   64-byte-row halves of the stage with the 64-byte swizzle
 //                   (a box past the filter's last code is loaded out of
-//                   range and arrives zero-filled).  When C % 8 == 0 (other
+//                   range and arrives zero-filled); on the widest tiles two
+//                   taps share such a block for their last 32 channels and
+//                   have 64-channel boxes before it (kModeTapPair).  When
+//                   C % 8 == 0 (other
 //                   counts) every tap has ceil(C / 64) K blocks of its own:
 //                   the last box of a tap reaches past C and arrives
 //                   zero-filled there, so whatever codes stand in those
