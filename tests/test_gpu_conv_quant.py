@@ -46,6 +46,17 @@ def test_fused_quant_conv_equals_separate(case):
     check_quantize(Wl.cpu(), codes, alpha)
 
 
+@pytest.mark.parametrize("case", [
+    (8, 96, 8, 8, 64, 3, 3, 1, 1, 1.3),        # tap pairs, nine taps
+    (2, 160, 8, 16, 130, 1, 3, 1, 0, 1.3),     # three taps of two whole blocks
+    (64, 64, 28, 28, 64, 3, 3, 1, 1, 1.3),     # row pairs without the fusion
+])
+def test_fused_quant_conv_equals_separate_on_paired_blocks(case):
+    N, C, H, W, K, R, S, st, pd, wscale = case
+    W = W + S - 1 if pd == 0 else W
+    test_fused_quant_conv_equals_separate((N, C, H, W, K, R, S, st, pd, wscale))
+
+
 def test_fused_quant_conv_matches_oracle():
     N, C, H, W, K = 2, 64, 10, 10, 96
     g = inputs.generator(77)
