@@ -126,8 +126,6 @@ __device__ __forceinline__ uint4 scale8(uint4 i4, const float* __restrict__ alph
 // channel.
 template <bool kUnit>
 __global__ void __launch_bounds__(256) bwd_data_prep_kernel(const __grid_constant__ PrepArgs a) {
-  // no grid_dependents_launch(): the convolution after this kernel reads the
-  // codes written here before its own wait
   grid_dependency_wait();
   if (static_cast<int>(blockIdx.x) < a.code_blocks) {
     transpose_codes(a.codes, a.wpf_in, a.codes_t, a.wpf_out, a.K, a.C, a.R, a.S,

@@ -75,15 +75,13 @@
 // error, drains its own in-flight copies and MMAs, frees TMEM and returns.
 //
 // The kernel is launched as a programmatic dependent of the previous kernel
-// on the stream: its start-up (TMEM allocation, barrier set-up, loading and
-// decoding the first blocks of codes) may overlap the previous kernel's last
-// wave, and only the reads of activations and of the residual wait for that
-// kernel to complete (grid_dependency_wait).  Codes and alpha are read
-// before that wait, so they must not be written by the immediately
-// preceding kernel when that kernel is one of this library's convolutions
-// (which let their dependents start early); no convolution writes anything
-// but its output.  Each CTA lets its own dependents start once it has passed
-// its wait, so everything older than the previous kernel is complete by then.
+// on the stream: its start-up (TMEM allocation, barrier set-up, tables) may
+// overlap the previous kernel's last wave.  Every role passes
+// grid_dependency_wait() before its first global read or write: only behind
+// that wait are the previous kernel's writes visible, and the codes may be
+// among them (a quantizer, or the transposition of the backward pass).  Each
+// CTA lets its own dependents start once it has passed its wait, so
+// everything older than the previous kernel is complete by then.
 #pragma once
 
 #include <cuda.h>
@@ -1155,6 +1153,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       const uint32_t* crow = m < a.K ? a.codes + static_cast<size_t>(m) * a.wpf : nullptr;
       const int cols = 8 * ((a.s2d_s * a.s2d_s * a.s2d_C + 15) / 16);
       const int part = min(16, cols - 16 * half);   // 16, 8 or none
+      grid_dependency_wait();   // the codes may come from the previous kernel
       for (int kb = 0; kb < KB; ++kb) {
         uint32_t v[16];
 #pragma unroll
@@ -1316,6 +1315,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       return r;
     };
     const PairMultipliers pm;
+    grid_dependency_wait();   // the codes may come from the previous kernel
     Codes q0 = next_codes(), q1 = next_codes(), q2 = next_codes(), q3 = next_codes();
     const uint32_t col = a_tmem0 + lane_off + static_cast<uint32_t>(16 * half);
     // two K blocks per iteration: their tensor-memory stores share one
