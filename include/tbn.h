@@ -43,7 +43,7 @@
  *   tbn_device_error() after synchronizing.
  * - tbn_last_error() returns a human-readable detail string for the most
  *   recent failing call on the calling host thread.
- * - The convolutions are launched as programmatic dependents of the previous
+ * - Most kernels are launched as programmatic dependents of the previous
  *   kernel on `stream`: their start-up may overlap that kernel's end, and
  *   they read activations, residuals, codes and alpha only after it has
  *   completed, so any of them may be the output of the preceding call.

@@ -236,6 +236,18 @@ __device__ __forceinline__ void tma_load_im2col_4d(void* dst, const void* tmap, 
       : "memory");
 }
 
+// A box of a 2-D tensor map, or a 16-byte aligned run, asked for in L2 only: a
+// hint that reads nothing, so it may stand before grid_dependency_wait().
+__device__ __forceinline__ void tma_prefetch_2d(const void* tmap, int c0, int c1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];" ::"l"(tmap), "r"(c0),
+               "r"(c1)
+               : "memory");
+}
+
+__device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // 4-D tiled bulk tensor store shared -> global (out-of-range box elements
 // are clipped), tracked by this thread's bulk async-group.
 __device__ __forceinline__ void tma_store_4d(const void* tmap, const void* src, int c0, int c1,

@@ -33,12 +33,12 @@
 // returns.
 //
 // The kernel is launched as a programmatic dependent of the previous kernel
-// on the stream: the first ring's worth of code boxes is requested before
-// griddepcontrol.wait, the inputs (and the residual) only after it, so in a
-// chain of layers the weight stream of one starts while the previous one
-// finishes.  Codes and alpha must therefore not be the output of the
-// immediately preceding call when that call is one of this library's
-// kernels that let their dependents start early.
+// on the stream.  Codes, inputs and residual may be that kernel's output, so
+// all are read behind griddepcontrol.wait; before it the first ring of code
+// boxes is asked for in L2, so in a chain of layers the weight stream of one
+// starts while the previous one finishes (batch 1, weights not in L2: 4096
+// square 5.1 us a call, 5.4 without; 8192 square 9.0; batch 8, 1024 square 3.3
+// and 3.6).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -253,6 +253,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     int it = 0;                      // stages issued so far
     int slot = 0;                    // it % stages
     uint32_t empty_parity = 1;       // parity of the release before use it / stages
+    // Codes and inputs may come from the previous kernel, so nothing is read
+    // before the wait.  The first ring of code boxes is only asked for in L2
+    // until then (a hint).
+    if (elected && static_cast<int>(blockIdx.x) * a.n_t < a.T)
+      for (int i = 0, kc = k_start; i < min(a.stages, a.nks); ++i) {
+        tma_prefetch_2d(&tmap_w, kc * kWordsPerStage, static_cast<int>(blockIdx.x) * a.n_t * 16);
+        if (++kc == a.nks) kc = 0;
+      }
+    __syncwarp();
+    grid_dependency_wait();
+    grid_dependents_launch();
     auto load_x = [&](int sl, int kc) {
       uint8_t* st = ring_ptr + static_cast<size_t>(sl) * a.stage_bytes;
       if (kB == 1) {
@@ -263,23 +274,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         tma_load_3d(st + a.w_bytes, &tmap_x, &full_bar[sl], 0, 0, kc * (kCodesPerStage / 8));
       }
     };
-    // The first band's first stages: codes now, inputs after the wait.
-    int deferred = 0;
-    bool waited = false;
-    auto finish_wait = [&]() {
-      grid_dependency_wait();   // the inputs may come from the previous kernel
-      grid_dependents_launch();
-      if (elected)
-        for (int i = 0; i < deferred; ++i) load_x(i, (k_start + i) % a.nks);
-      __syncwarp();
-      waited = true;
-    };
     for (int r = 0; r < a.rounds; ++r) {
       const int band = blockIdx.x + r * gridDim.x;
       if (band * a.n_t >= a.T) break;
       int kc = k_start;
       for (int ks = 0; ks < a.nks; ++ks) {
-        if (!waited && (r > 0 || it >= a.stages)) finish_wait();
         bool ok = true;
         if (it >= a.stages)
           ok = mbar_wait_sleep(&empty_bar[slot], empty_parity, &abort_flag, a.err, kWaitLimitNs);
@@ -289,9 +288,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           uint8_t* st = ring_ptr + static_cast<size_t>(slot) * a.stage_bytes;
           mbar_arrive_expect_tx(&full_bar[slot], a.stage_bytes);
           tma_load_2d(st, &tmap_w, &full_bar[slot], kc * kWordsPerStage, band * a.n_t * 16);
-          if (waited) load_x(slot, kc);
+          load_x(slot, kc);
         }
-        if (!waited) ++deferred;
         __syncwarp();
         ++it;
         if (++kc == a.nks) kc = 0;
@@ -302,7 +300,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (__shfl_sync(0xffffffffu, abort_flag, 0)) break;
     }
-    if (!waited) finish_wait();
     // On abort, wait (bounded) for the last copy issued into each slot so
     // no TMA write lands after the CTA has exited.
     if (elected && abort_flag) {

@@ -262,6 +262,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_f8_kernel(const __grid_const
 
   if (warp == 0) {
     // ================= producer: code boxes =================
+    // they may come from the previous kernel: until the wait, the first ring
+    // of them is only asked for in L2 (a hint)
+    if (elect_one())
+      for (int u = ur.u0; u < min(ur.u1, ur.u0 + CS); ++u)
+        bulk_prefetch(a.prepared + static_cast<size_t>(u) * (kRows * kStageWords), kCodeStageBytes);
+    __syncwarp();
+    grid_dependency_wait();
     int g = 0;
     bool ok = true;
     for (int u = ur.u0; u < ur.u1 && ok; ++u, ++g) {

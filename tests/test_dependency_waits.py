@@ -21,6 +21,9 @@ ROLES = [
     ("tbn_conv_igemm.cuh", "= expanders =", "= epilogue ="),
     ("tbn_conv_igemm.cuh", "= epilogue =", "- host side"),
     ("tbn_conv_smalltap.cu", "conv_smalltap_kernel(SmallTapArgs", "struct TcTile"),
+    ("tbn_gemv.cu", "- producer", "- consumers"),
+    ("tbn_gemv_f8.cu", "= producer: code boxes =", "} else {"),
+    ("tbn_gemv_f8.cu", "// The exact three-term split of x (which", "named_barrier_sync(1, nt);"),
     ("tbn_conv_bwd.cu", "bwd_data_prep_kernel(", "struct BwdFilterArgs"),
     ("tbn_conv_bwd.cu", "bwd_filter_tma_kernel(const", "add4("),
     ("tbn_conv_bwd.cu", "bwd_filter_reduce4_kernel(\n", "bwd_filter_reduce_kernel("),

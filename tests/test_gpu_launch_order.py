@@ -69,3 +69,34 @@ def test_input_gradients_share_a_workspace(case):
     assert tbn.tbn_device_error() == 0
     for i, dx in enumerate(got):
         assert torch.equal(dx, want[i % 2]), "round %d" % i
+
+
+@pytest.mark.parametrize("B,K", [(1, 1024), (8, 1024), (1, 4096)])
+@pytest.mark.parametrize("fp8", [False, True])
+def test_linear_after_its_quantizer(B, K, fp8):
+    """The GEMVs, from codes just quantized and from codes just prepared."""
+    if fp8 and B > 1:
+        pytest.skip("the fp8 layer takes batch 1")
+    x = torch.randn(B, K, generator=inputs.generator(B)).to(torch.bfloat16).cuda()
+    Ws = _filters(K, K, K)
+    codes, alpha = tbn.tbn_quantize_pack(Ws[0])
+    if fp8:
+        prep = torch.empty(tbn.tbn_linear_f8_prepared_words(K, K), dtype=torch.int32, device="cuda")
+        ws = torch.empty(tbn.tbn_linear_f8_workspace_bytes(1, K, K), dtype=torch.uint8,
+                         device="cuda")
+
+    def layer(w, wait):
+        tbn.tbn_quantize_pack(w, codes=codes, alpha=alpha)
+        if fp8:
+            tbn.tbn_linear_prepare_f8(codes, K, out=prep)
+        if wait:
+            torch.cuda.synchronize()
+        return (tbn.tbn_linear_fwd_f8(x, prep, alpha, K, ws) if fp8
+                else tbn.tbn_linear_fwd(x, codes, alpha, K))
+
+    want = [layer(w, True) for w in Ws]
+    got = [layer(Ws[i % 2], False) for i in range(ROUNDS)]
+    torch.cuda.synchronize()
+    assert tbn.tbn_device_error() == 0
+    for i, y in enumerate(got):
+        assert torch.equal(y, want[i % 2]), "round %d" % i
