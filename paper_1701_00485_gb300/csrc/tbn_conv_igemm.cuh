@@ -201,8 +201,10 @@ constexpr int kModeTmaPad = 5;  // 64-channel TMA boxes, each tap's last one pad
 // even output rows, rows 64-127 the same filters, one tap row later, for the
 // odd ones.  Both read the same box of input rows 2 i + r', r' = 0 .. R, so
 // R + 1 tap rows serve two output rows where one at a time takes 2 R with
-// half the MMA's rows empty; the tap row that a half does not have is a
-// block of zero weights.
+// half the MMA's rows empty.  The first tap row is the even rows' alone and
+// the last the odd rows': their MMAs leave the other half's accumulators as
+// they are (disabled output lanes), so an infinite or NaN input reaches the
+// outputs whose taps read it and no others, at no cost.
 constexpr int kModeRowPair = 6;
 // Tap pairs (C = 64 m + 32, m >= 1): the K blocks of two taps are each tap's m
 // whole 64-channel boxes, then one block of both taps' last 32 channels, so
@@ -316,27 +318,6 @@ __device__ __forceinline__ void store_out(const IgArgs& a, size_t o, float v, fl
     static_cast<__nv_bfloat16*>(a.y)[o] = __float2bfloat16_rn(v);
   else
     static_cast<float*>(a.y)[o] = v;
-}
-
-// Row pairs: sum of x W~/2 over the taps of MMA row m (filter m & 63, row
-// parity m >> 6) at pixel f of the row pairs, in fp32.
-__device__ __noinline__ float rowpair_sum(const IgArgs& a, int m, int f) {
-  const int row = f / a.iQ, n = row / a.iP;
-  const int q = f - row * a.iQ, p = 2 * (row - n * a.iP) + (m >> 6);
-  const uint32_t* codes = a.codes + static_cast<size_t>(m & 63) * a.wpf;
-  float acc = 0.0f;
-  for (int r = 0; r < a.R - 1; ++r)
-    for (int s = 0; s < a.S; ++s) {
-      const int h = p - a.ph + r, w = q * a.sw - a.pw + s;
-      if (h < 0 || h >= a.H || w < 0 || w >= a.W) continue;
-      const __nv_bfloat16* x = a.x + ((static_cast<int64_t>(n) * a.H + h) * a.W + w) * a.C;
-      for (int c = 0; c < a.C; ++c) {
-        const int i = (r * a.S + s) * a.C + c;
-        acc = fmaf(__bfloat162float(x[c]), 0.5f * code_value(code_field(__ldg(codes + (i >> 4)), i & 15)),
-                   acc);
-      }
-    }
-  return acc;
 }
 
 // Split K in a cluster: its CTAs have stored the sums of one K range each for
@@ -1088,6 +1069,7 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     int issued = 0, st = 0;
     uint32_t tiles_done = 0, par = 0;
     const int tap_blocks = (a.C + kBK - 1) / kBK;   // padded mode: K blocks per tap
+    const int tap_row = a.S * (a.C / kBK);          // row pairs: K blocks per tap row
     // space-to-depth mode: K steps that hold channels (the others are zero in
     // both operands; AlexNet conv1, batch 256, three of four: 83.8 -> 79.4 us)
     const int s2d_steps = (a.s2d_s * a.s2d_s * a.s2d_C + 15) / 16;
@@ -1115,7 +1097,14 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
         // halves of 32 codes, 64-byte rows, with 32-channel boxes)
         const uint32_t b_addr = smem_addr(ring) + static_cast<uint32_t>(st * kStageBytes);
         constexpr uint32_t kHalf = kCh32 ? (kStageBytes / 2) >> 4 : 4u;
-        if (kTapPair && !tp.whole())
+        // row pairs: the first tap row's blocks are the lower half's alone, the
+        // last one's the upper half's
+        if (kRowPair && (kb <= tap_row || kb >= KB - tap_row))
+          tc_mma_ts_block_halves(acc_t, a_col, smem_desc_sw128_kmajor(b_addr), idesc,
+                                 kb != 0 ? 1u : 0u, kb >= KB - tap_row ? ~0u : 0u,
+                                 kb <= tap_row ? ~0u : 0u, kb < tap_row ? ~0u : 0u,
+                                 &ctl->empty[st], kb == KB - 1 ? &ctl->acc_full[ab] : nullptr);
+        else if (kTapPair && !tp.whole())
           tc_mma_ts_block<2, (kStageBytes / 2 >> 4), (kStageBytes / 2 >> 4) + 2>(
               acc_t, a_col, smem_desc_sw64_kmajor(b_addr), idesc, kb != tc.kb0 ? 1u : 0u, 4,
               &ctl->empty[st], kb == tc.kb1 - 1 ? &ctl->acc_full[ab] : nullptr);
@@ -1195,10 +1184,10 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     int t_ld = blockIdx.x, kb_ld = 0, kb_end = 0, kb_lim = 0;
     const int kb_words = (a.wpf - 2 * half + 3) / 4;   // K blocks whose two words begin in the row
     // row pairs: the upper 64 rows (two of the four sub-partitions) run one
-    // tap row behind; K blocks before and after a half's taps are zero
+    // tap row behind; what is stored in the K blocks before and after a half's
+    // taps is of no account (the MMA leaves that half's accumulators alone)
     const int behind = kRowPair && sub >= 2 ? a.S * (a.C / kBK) : 0;
     const int kb_taps = kRowPair ? (a.R - 1) * a.S * (a.C / kBK) : 0;
-    int kb_st = 0;   // row pairs: the K block (within its tile) next to be stored
     const uint32_t* cp = a.codes;
     // padded mode: this half block's first code, and channels left in its tap
     const int tap_blocks = (a.C + kBK - 1) / kBK;
@@ -1327,19 +1316,6 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
       uint32_t v0[16], v1[16];
       decode(q0, v0, pm);
       decode(q1, v1, pm);
-      if constexpr (kRowPair) {
-        // warp-uniform: a whole half's K block is taps or zeros
-        const auto zero = [&](uint32_t* v) {
-          const int kb = kb_st - behind;
-          if (kb < 0 || kb >= kb_taps) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0u;
-          }
-          if (++kb_st == KB) kb_st = 0;
-        };
-        zero(v0);
-        if (two) zero(v1);
-      }
       q0 = q2;
       q1 = q3;
       q2 = next_codes();
@@ -1482,27 +1458,6 @@ __global__ void __launch_bounds__(threads_for<kMode>(), 1)
             } else {
               tc_fence_before_sync();
               mbar_arrive(&ctl->acc_empty[ab]);
-            }
-            if constexpr (kRowPair) {
-              // a zero weight times an infinite or NaN input of the other row's
-              // taps is NaN: such sums are recomputed from their own taps
-              uint64_t z2[2] = {0, 0};
-#pragma unroll
-              for (int i = 0; i < 8; ++i)
-                z2[i & 1] = fma_f32x2(f32x2(v[lg][2 * i], v[lg][2 * i + 1]), 0ull, z2[i & 1]);
-              z2[0] = add_f32x2(z2[0], z2[1]);
-              if (__uint_as_float(static_cast<uint32_t>(z2[0])) != 0.0f ||
-                  __uint_as_float(static_cast<uint32_t>(z2[0] >> 32)) != 0.0f) {   // NaN
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                  const int mm = sub * 32 + lg * 16 + ((e >> 1) & 1) * 8 + fr;
-                  const int px = 32 * j + 8 * (e >> 2) + 2 * (lane & 3) + (e & 1);
-                  const int f = tc.p0 * a.Q + px;   // pixel of the row pairs
-                  if ((mm & 63) < a.K && px < a.bw * a.bh && f < a.P * a.Q &&
-                      !(fabsf(__uint_as_float(v[lg][e])) <= 3.402823466e38f))
-                    v[lg][e] = __float_as_uint(rowpair_sum(a, mm, f));
-                }
-              }
             }
             uint32_t pk[8];
             uint32_t addr[2];
@@ -1845,9 +1800,10 @@ inline bool use_tma_store(const ConvProblem& p) {
 // stride 1 down the rows, an even number of output rows of at most a tile's
 // width, whole 64-channel boxes, and the staged bf16 epilogue.  It pays for
 // filters of several rows: 3 x 3 over 64 channels takes 12 K blocks for two
-// output rows instead of 18 (56 x 56 with shortcut, 64 filters, batch 64: 27.5 ->
-// 24.5 us; the ResNet-18 step at batch 128: 602 -> 574); plan_cost decides by
-// the K blocks.
+// output rows instead of 18 (56 x 56 with shortcut, 64 filters, batch 64: 27.5
+// us one row at a time, 22.2 in pairs; 24.6 when zero weights stood for the
+// tap row that a half does not have and the epilogue looked for sums that an
+// infinite input times those made NaN); plan_cost decides by the K blocks.
 inline bool rowpair_ok(const ConvProblem& p) {
   return p.C % kBK == 0 && p.K <= kBM / 2 && p.sh == 1 && p.sw <= 2 && p.P % 2 == 0 && p.R >= 2 &&
          p.R < 128 && p.Q <= kMaxTileN && !p.pool && p.wq == nullptr && use_tma_store(p);

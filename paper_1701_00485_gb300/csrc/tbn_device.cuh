@@ -370,6 +370,38 @@ __device__ __forceinline__ void tc_mma_ts_block(uint32_t d_tmem, uint32_t a_tmem
       : "memory");
 }
 
+// The same four MMAs (kB1 = 2 and so on: 32 bytes apart) with whole halves of
+// D's 128 lanes left as they are: `no_low` and `no_high` are ~0 to disable
+// lanes 0-63 and 64-127, `no_high0` the latter in the first MMA.  Where
+// no_high0 differs from no_high, the upper half begins with this block: the
+// first MMA is issued for it once more, without accumulating.
+__device__ __forceinline__ void tc_mma_ts_block_halves(uint32_t d_tmem, uint32_t a_tmem,
+                                                       uint64_t b_desc, uint32_t idesc,
+                                                       uint32_t accumulate, uint32_t no_low,
+                                                       uint32_t no_high0, uint32_t no_high,
+                                                       uint64_t* done, uint64_t* done2) {
+  asm volatile(
+      "{\n\t.reg .pred e, ex, ec, p, t, f;\n\t"
+      ".reg .b32 a1, a2, a3, all, none;\n\t.reg .b64 b1, b2, b3;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, 0, 0;\n\tsetp.ne.b32 f, 0, 0;\n\t"
+      "setp.ne.and.b32 ex, %6, %7, e;\n\tsetp.ne.and.b32 ec, %9, 0, e;\n\t"
+      "mov.b32 all, -1;\n\tmov.b32 none, 0;\n\t"
+      "add.u32 a1, %1, 8;\n\tadd.u32 a2, %1, 16;\n\tadd.u32 a3, %1, 24;\n\t"
+      "add.u64 b1, %2, 2;\n\tadd.u64 b2, %2, 4;\n\tadd.u64 b3, %2, 6;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %5, %6, %6}, p;\n\t"
+      "@ex tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {all, all, none, none}, f;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, {%5, %5, %7, %7}, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a2], b2, %3, {%5, %5, %7, %7}, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a3], b3, %3, {%5, %5, %7, %7}, t;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%8];\n\t"
+      "@ec tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%9];\n\t}" ::"r"(
+          d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(no_low), "r"(no_high0),
+      "r"(no_high), "r"(smem_addr(done)), "r"(done2 != nullptr ? smem_addr(done2) : 0u)
+      : "memory");
+}
+
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
