@@ -11,6 +11,9 @@
 // one per tap.  Where the result is not finite (an infinite or NaN input or
 // weight, or an overflow) it is recomputed tap by tap in fp32, as the
 // CUDA-core kernel does, because the split's zero terms times infinity are NaN.
+// What that costs (32 images of 3 x 224 x 224, 37 us when finite, some 220 on
+// the CUDA cores): 195 us for a batch of NaN, 297 of infinities, 2.6 ms where
+// every sum overflows or most hold an infinity.
 //
 // GEMM view of a tile: D[128 pixels x 192] = A[128 x k] B[k x 192], where the
 // 192 columns are 64 filters x {h, m, l} (one read of A serves all three) and
@@ -104,21 +107,46 @@ struct alignas(16) Ctl {
   int abort;
 };
 
-// One output tap by tap, for results that are not finite.
-__device__ __noinline__ float dense_by_taps(const Args& a, int n, int k, int pix) {
+// Results that are not finite, tap by tap in fp32: bit i of `bad` is filter
+// k + i of this lane's pixel `pix` of image n, staged in `row_s` (the pixel's
+// 64 filters, 16-byte chunks permuted by `swz`) from chunk `chunk` on.  By the
+// whole warp, eight filters at a time, so that a tap's weights are one load for
+// all lanes and its input one load for eight filters; ends early when every
+// sum that is needed is NaN.
+__device__ __noinline__ void repair_by_taps(const Args& a, int n, int k, int pix, uint32_t bad,
+                                            uint8_t* row_s, int chunk, int swz) {
   const int p = pix / a.Q, q = pix - p * a.Q;
-  float acc = 0.0f;
-  for (int c = 0; c < a.C; ++c)
-    for (int r = 0; r < a.R; ++r)
+  const int h0 = p * a.sh - a.ph, w0 = q * a.sw - a.pw, wstep = a.nch * a.S;
+  for (int g = 0; g < 4; ++g, bad >>= 8, k += 8) {   // K % 8 == 0
+    const bool need = (bad & 0xFFu) != 0u;
+    if (!__any_sync(0xffffffffu, need)) continue;
+    const float* wk = a.w + static_cast<int64_t>(k) * wstep;
+    float acc[8] = {};
+    for (int cr = 0; cr < a.nch; ++cr) {
+      const int c = cr / a.R, h = h0 + cr - c * a.R;
+      const __nv_bfloat16* xr = a.x + ((static_cast<int64_t>(n) * a.C + c) * a.H + h) * a.W + w0;
+      const bool hv = h >= 0 && h < a.H;
+#pragma unroll 4
       for (int s = 0; s < a.S; ++s) {
-        const int h = p * a.sh - a.ph + r, w = q * a.sw - a.pw + s;
-        float xv = 0.0f;
-        if (h >= 0 && h < a.H && w >= 0 && w < a.W)
-          xv = __bfloat162float(
-              a.x[((static_cast<int64_t>(n) * a.C + c) * a.H + h) * a.W + w]);
-        acc = fmaf(xv, __ldg(a.w + ((static_cast<int64_t>(k) * a.C + c) * a.R + r) * a.S + s), acc);
+        const float xv = hv && w0 + s >= 0 && w0 + s < a.W ? __bfloat162float(xr[s]) : 0.0f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          acc[j] = fmaf(xv, __ldg(wk + j * wstep + cr * a.S + s), acc[j]);
       }
-  return acc;
+      bool done = true;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) done &= acc[j] != acc[j];
+      if (__all_sync(0xffffffffu, done || !need)) break;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if ((bad >> j) & 1u) {
+        const float v = a.relu ? fmaxf(acc[j], 0.0f) : acc[j];   // NaN gives 0 there
+        reinterpret_cast<__nv_bfloat16*>(row_s + (((chunk + g) ^ swz) << 4))[j] =
+            __float2bfloat16_rn(v);
+      }
+  }
+  __syncwarp();
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -322,6 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int n = a.by_img(t), f0 = (t - n * a.tiles_img) * kPix;
       if (ok) {
         tc_fence_after_sync();
+        uint32_t bad = 0;   // results that are not finite
 #pragma unroll
         for (int cc = 0; cc < 2; ++cc) {
           uint32_t vh[16], vm[16], vl[16];
@@ -352,15 +381,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           const float z = __uint_as_float(static_cast<uint32_t>(zero)) +
                           __uint_as_float(static_cast<uint32_t>(zero >> 32));
-          if (z != 0.0f && f0 + row < a.PQ) {   // NaN != 0
+          // one decision for the warp: collective instructions follow
+          if (__any_sync(0xffffffffu, z != 0.0f)) {   // NaN != 0
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int k = k0 + 32 * half + 16 * cc + j;
-              if (k < a.K && !(fabsf(o[j]) <= 3.402823466e38f)) {
-                o[j] = dense_by_taps(a, n, k, f0 + row);
-                if (a.relu) o[j] = fmaxf(o[j], 0.0f);   // NaN gives 0 there too
-              }
-            }
+            for (int j = 0; j < 16; ++j)
+              bad |= (fabsf(o[j]) <= 3.402823466e38f ? 0u : 1u) << (16 * cc + j);
           }
           uint32_t pk[8];
 #pragma unroll
@@ -373,6 +398,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                                       (((4 * half + 2 * cc + u) ^ (row & 7)) << 4)) =
                 make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
         }
+        const int k = k0 + 32 * half;
+        bad = f0 + row < a.PQ && k < a.K ? bad & (0xFFFFFFFFu >> max(0, k + 32 - a.K)) : 0u;
+        if (__any_sync(0xffffffffu, bad != 0u))
+          repair_by_taps(a, n, k, min(f0 + row, a.PQ - 1), bad, stage + row * 128, 4 * half,
+                         row & 7);
       }
       fence_proxy_async_smem();
       named_barrier_sync(1, 32 * kEpWarps);

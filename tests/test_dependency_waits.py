@@ -1,4 +1,6 @@
-"""Programmatic dependent launches read nothing of the previous kernel before
+"""Orders that no run can show to be wrong, checked in the kernels' source.
+
+Programmatic dependent launches read nothing of the previous kernel before
 griddepcontrol.wait: only behind it are that kernel's writes visible, and any
 input may be one (codes come from a quantizer or from the backward pass's
 transposition).  A race of this kind cannot be provoked at will, so the order
@@ -41,3 +43,19 @@ def test_wait_precedes_the_first_read(name, begin, end):
     first = READS.search(body)
     assert wait >= 0 and first is not None
     assert wait < first.start(), "%s: %r reads global memory before its wait" % (name, begin)
+
+
+def test_rare_recomputation_is_decided_by_the_whole_warp():
+    """The fp32 first layer recomputes results that are not finite and then goes
+    on to warp-collective instructions (tensor-memory loads, named barriers), so
+    no lane may leave the others: a vote decides, and the function that takes
+    the detour ends converged."""
+    text = open(os.path.join(CSRC, "tbn_dense_tc.cu")).read()
+    calls = [m.start() for m in re.finditer(r"_by_taps\(", text)]
+    definition, uses = calls[0], calls[1:]
+    assert uses
+    for u in uses:
+        before = text[:u].rstrip().rsplit("\n", 2)[-2]
+        assert re.search(r"if \(__any_sync\(0xffffffffu, ", before), before
+    body = text[definition:text.index("\n}\n", definition)]
+    assert body.rstrip().endswith("__syncwarp();")

@@ -78,6 +78,53 @@ def test_dense_tc_not_finite(value):
     assert np.all(np.abs(y[fin] - ref[fin]) <= 2.0 ** -6 * np.abs(ref[fin]) + 1e-4)
 
 
+@pytest.mark.parametrize("relu", [False, True])
+def test_dense_tc_not_finite_spread(relu):
+    """Several such inputs in every tile, over two filter groups and a ragged
+    last tile: each output is what fp32 products and sums give."""
+    g = inputs.generator(5)
+    x = torch.randn(3, 3, 30, 40, generator=g)
+    at = torch.rand(x.shape, generator=g)
+    x[at < 0.004] = float("inf")
+    x[at > 0.997] = float("-inf")
+    x[(at > 0.5) & (at < 0.501)] = float("nan")
+    x = x.to(torch.bfloat16)
+    w = inputs.he_normal(72, 3, 7, 7, g)
+    y = _run(x, w, (2, 2), (3, 3), relu)
+    ref = torch.nn.functional.conv2d(x.double(), w.double(), stride=2, padding=3)
+    if relu:
+        ref = torch.where(ref > 0, ref, 0.0)   # NaN gives 0, as fmaxf does
+    ref = ref.float().to(torch.bfloat16).float().numpy()
+    fin = np.isfinite(ref)
+    assert 0.1 < fin.mean() < 0.9
+    assert np.array_equal(np.isnan(y), np.isnan(ref))
+    assert np.array_equal(y[~fin & ~np.isnan(ref)], ref[~fin & ~np.isnan(ref)])
+    assert np.all(np.abs(y[fin] - ref[fin]) <= 2.0 ** -6 * np.abs(ref[fin]) + 1e-4)
+
+
+def test_dense_tc_cost_of_not_finite_input():
+    """A batch of NaN or infinities (a diverged run) costs several times a
+    finite one, not hundreds: the sums end at the first NaN."""
+    x = torch.randn(16, 3, 224, 224, generator=inputs.generator(6)).to(torch.bfloat16).cuda()
+    w = inputs.he_normal(64, 3, 7, 7, inputs.generator(7)).cuda()
+    us = []
+    for xs in (x, torch.full_like(x, float("nan")), torch.full_like(x, float("inf"))):
+        best = float("inf")
+        for _ in range(6):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                y = tbn.tbn_dense_conv2d_fwd(xs, w, (2, 2), (3, 3), layout=tbn.TBN_NCHW_NHWC,
+                                             out_dtype=torch.bfloat16)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 250.0)
+        us.append(best)
+    assert tbn.tbn_device_error() == 0
+    # measured 5 and 8 times; the limit allows for other clocks and drivers
+    assert max(us[1:]) <= 25.0 * us[0], us
+
+
 @pytest.mark.parametrize("B,K_in,K_out", [(33, 128, 31), (1, 4, 1), (32, 129, 32), (65, 516, 100),
                                           (31, 252, 1000)])
 def test_dense_linear_tile_edges(B, K_in, K_out):
