@@ -84,6 +84,8 @@ _lock = threading.Lock()
 _lib = None
 
 
+# exports of this binding's own, not declared in tbn.h
+_PRIVATE = ["tbn_packed_call"]
 ABI_VERSION = 9  # must match TBN_ABI_VERSION in include/tbn.h
 
 
@@ -101,6 +103,7 @@ def lib():
             raise RuntimeError("libtbn.so not found at %s: build it with "
                                "`python -m paper_1701_00485_gb300.build`" % _LIB_PATH)
         L = ctypes.CDLL(_LIB_PATH)
+        _check_version(L)
         P, I64, I32, U32P = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_void_p
         sig = {
             "tbn_abi_version": ([], I32),
@@ -155,10 +158,20 @@ def lib():
             fn.restype = res
         L.tbn_packed_call.argtypes = [I32, ctypes.c_char_p]
         L.tbn_packed_call.restype = I32
-        if L.tbn_abi_version() != ABI_VERSION:
-            raise RuntimeError("libtbn ABI version mismatch")
         _lib = L
         return L
+
+
+def _check_version(L):
+    """Raise unless the library is the one that this binding was written for:
+    the version of tbn.h, and the private exports, which have none."""
+    version = L.tbn_abi_version() if hasattr(L, "tbn_abi_version") else None
+    missing = [n for n in EXPORTED + _PRIVATE if not hasattr(L, n)]
+    if version != ABI_VERSION or missing:
+        raise RuntimeError("libtbn ABI version mismatch: the library has version %s%s, the "
+                           "binding needs %d; rebuild it" %
+                           (version, " without " + ", ".join(missing) if missing else "",
+                            ABI_VERSION))
 
 
 # The calls that a program issues once per layer pass their arguments as one

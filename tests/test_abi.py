@@ -4,6 +4,7 @@ arguments on the host before launching anything."""
 import ctypes
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -43,6 +44,22 @@ def test_abi_version_and_sizes(L):
     assert L.tbn_packed_words(0) == -1
     assert L.tbn_status_string(0) == b"ok"
     assert L.tbn_status_string(2) == b"unsupported"
+
+
+@pytest.mark.parametrize("version,body", [
+    (8, ""),                      # an older library
+    (9, "int tbn_quantize_pack(void) { return 0; }"),   # this version, exports missing
+])
+def test_other_libraries_are_refused_by_version(tmp_path, monkeypatch, version, body):
+    """Before any symbol is looked up: an older library is named as what it is."""
+    src = tmp_path / "stub.c"
+    src.write_text("int tbn_abi_version(void) { return %d; }\n%s\n" % (version, body))
+    so = tmp_path / ("libstub%d.so" % version)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
+    monkeypatch.setattr(tbn, "_LIB_PATH", str(so))
+    monkeypatch.setattr(tbn, "_lib", None)
+    with pytest.raises(RuntimeError, match="version mismatch.*tbn_packed_call"):
+        tbn.lib()
 
 
 def test_quantize_rejects_bad_arguments(L):
