@@ -1093,10 +1093,19 @@ tbn_status launch_bwd_data(const BwdConvShape& p, const void* dy, const uint32_t
     const int64_t blocks = std::min<int64_t>((threads + 255) / 256,
                                              static_cast<int64_t>(device_sm_count()) * 16);
     const unsigned grid = static_cast<unsigned>(a.code_blocks + blocks);
-    const cudaError_t e = launch_dependent(
-        unit ? bwd_data_prep_kernel<true> : bwd_data_prep_kernel<false>, dim3(grid), dim3(256), 0,
-        s, a);
-    if (e != cudaSuccess) return cuda_fail(e, "bwd_data_prep_kernel");
+    const auto kern = unit ? bwd_data_prep_kernel<true> : bwd_data_prep_kernel<false>;
+    // As a dependent its blocks are placed while the previous kernel still
+    // holds its SMs, so they gather on the idle ones, up to eight on each:
+    // worth 0.7 us where they are few and short (64 -> 64 channels, 8 x 8: 8.0
+    // us a call, launched plainly 9.3), a loss where they fill the machine
+    // (512 -> 512, 2 x 14 x 14: 44.2 and 32.3) or each runs long (65 -> 33
+    // channels, 64 x 32 x 32, pixel by pixel: 190 and 96).
+    if (a.vec && grid <= static_cast<unsigned>(device_sm_count())) {
+      const cudaError_t e = launch_dependent(kern, dim3(grid), dim3(256), 0, s, a);
+      if (e != cudaSuccess) return cuda_fail(e, "bwd_data_prep_kernel");
+    } else {
+      kern<<<grid, 256, 0, s>>>(a);
+    }
     const tbn_status st = check_launch("bwd_data_prep_kernel");
     if (st != TBN_OK) return st;
   }

@@ -185,3 +185,39 @@ def test_bwd_tma_filter_and_prep(case):
     dx_orc, bx = oracle.conv2d_bwd_data(dy.float().numpy(), wt, al, (H, W), st, pd)
     assert_within(dx.float().cpu().permute(0, 3, 1, 2).numpy(), dx_orc, bx, out_bf16=True,
                   extra=BF16_TERM, what="bwd data %s" % (case,))
+
+
+@pytest.mark.parametrize("case", [
+    (64, 33, 32, 32, 65, 1, 1, (1, 1), (0, 0)),    # few long blocks of the preparation
+    (2, 512, 14, 14, 512, 3, 3, (2, 2), (1, 1)),   # more blocks than SMs
+])
+def test_bwd_data_calls_in_a_row_cost_no_more_than_alone(case):
+    """What a call starts early must not crowd the SMs that the one before it
+    leaves idle: in a row calls are at least as fast as one at a time."""
+    N, C, H, W, K, R, S, st, pd = case
+    P, Q = tbn.conv_out_hw(H, W, R, S, st, pd)
+    g = inputs.generator(C)
+    codes, alpha = tbn.tbn_quantize_pack(inputs.normal((K, C * R * S), 1.2, g).cuda())
+    dy = torch.randn(N, P, Q, K, generator=g).to(torch.bfloat16).cuda()
+    n = tbn.lib().tbn_conv2d_bwd_data_workspace_bytes(N, C, H, W, K, R, S, *st, *pd)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    s = torch.cuda.Stream()
+    us = {}
+    with torch.cuda.stream(s):
+        for calls in (1, 8):
+            tbn.tbn_conv2d_bwd_data(dy, codes, alpha, C, (H, W), R, S, st, pd, workspace=ws)
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s):
+                for _ in range(calls):
+                    tbn.tbn_conv2d_bwd_data(dy, codes, alpha, C, (H, W), R, S, st, pd,
+                                            workspace=ws)
+            us[calls] = float("inf")
+            for _ in range(8):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record(s)
+                graph.replay()
+                b.record(s)
+                torch.cuda.synchronize()
+                us[calls] = min(us[calls], a.elapsed_time(b) * 1e3 / calls)
+    assert us[8] <= 1.1 * us[1], us
