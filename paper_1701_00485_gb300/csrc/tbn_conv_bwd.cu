@@ -905,21 +905,10 @@ int bwd_filter_slices(const BwdConvShape& p) {
   return static_cast<int>(std::min<int64_t>(s, 1024));
 }
 
-// The TMA-fed kernel: what limits an im2col tensor map (32-bit pixel indices,
-// 8-bit corner and tap offsets, strides up to 8), whole 16-byte rows, and at
-// least 40 channels, so that its 64-channel boxes are mostly channels.  Below
-// that, and for unaligned pointers, the kernels above (32 images of 28 x 28 x
-// 40 -> 72 at stride 2: 10.2 us against 11.7; equal at one small image).
-bool bwd_filter_tma_shape(const BwdConvShape& p) {
-  return p.K % 8 == 0 && p.C % 8 == 0 && p.C >= 40 && p.sh <= 8 && p.sw <= 8 && p.R <= 128 &&
-         p.S <= 128 && p.ph <= 127 && p.pw <= 127 && p.N * p.P * p.Q <= (int64_t(1) << 30) &&
-         p.N < (int64_t(1) << 30) && p.N * p.H * p.W * p.C * 2 >= 131072 &&
-         p.N * p.P * p.Q * p.K * 2 >= 131072;
-}
-
-// Its tiles (column units per CTA) and pixel slices, from the shape alone so
-// that the workspace query agrees with the launch.  A chunk costs a CTA about
-// 300 + 150 units cycles (its boxes' bytes); slices fill the machine once.
+// The TMA-fed kernel's tiles (column units per CTA) and pixel slices, from the
+// shape alone so that the workspace query agrees with the launch.  A chunk
+// costs a CTA about 300 + 150 units cycles (its boxes' bytes); slices fill the
+// machine once.
 struct BwdTmaPlan {
   int units, per_cta, cblocks, chunks, per_slice, slices;
 };
@@ -943,6 +932,53 @@ BwdTmaPlan plan_bwd_tma(const BwdConvShape& p) {
   t.per_slice = static_cast<int>((t.chunks + s - 1) / s);
   t.slices = (t.chunks + t.per_slice - 1) / t.per_slice;
   return t;
+}
+
+// Cycles that a box of 64 rows takes beyond the usual 150 when its rows end 8,
+// 24 or 40 channels into it (measured: 16, 48 or 80 valid bytes of 128 slow the
+// copy down, 112 and the multiples of 32 do not).
+int slow_rows(int64_t channels) {
+  switch (channels % 64) {
+    case 8: return 250;
+    case 24: return 300;
+    case 40: return 420;
+  }
+  return 0;
+}
+
+// The TMA-fed kernel: what limits an im2col tensor map (32-bit pixel indices,
+// 8-bit corner and tap offsets, strides up to 8), whole 16-byte rows, and at
+// least 40 channels, so that its 64-channel boxes are mostly channels.  Below
+// that, and for unaligned pointers, the kernels above (32 images of 28 x 28 x
+// 40 -> 72 at stride 2: 10.2 us against 11.7; equal at one small image).
+// Where boxes of x or dy have slow rows the estimates decide, with a tenth in
+// favour of TMA (in us): its chunks of 200 + 160 units cycles and the slow
+// boxes', against 1.08 a chunk of the cp.async kernel, both with their slices'
+// sum at 1.5 TB/s.  (TMA and cp.async, batch 64, 32 x 32: 40 -> 40 channels 3 x 3
+// 35 and 21 us, 5 x 5 82 and 38; 72 -> 128 5 x 5 80 and 76, 3 x 3 33 and 38.)
+bool bwd_filter_tma_shape(const BwdConvShape& p) {
+  if (p.K % 8 != 0 || p.C % 8 != 0 || p.C < 40 || p.sh > 8 || p.sw > 8 || p.R > 128 ||
+      p.S > 128 || p.ph > 127 || p.pw > 127 || p.N * p.P * p.Q > (int64_t(1) << 30) ||
+      p.N >= (int64_t(1) << 30) || p.N * p.H * p.W * p.C * 2 < 131072 ||
+      p.N * p.P * p.Q * p.K * 2 < 131072)
+    return false;
+  const int x_slow = slow_rows(p.C), dy_slow = slow_rows(p.K);
+  if (x_slow == 0 && dy_slow == 0) return true;
+  const BwdTmaPlan t = plan_bwd_tma(p);
+  const int64_t ktiles = (p.K + 127) / 128, rsc = p.R * p.S * p.C, sms = device_sm_count();
+  const double sum = static_cast<double>(p.K * rsc) * 4.0 / 1.5e6;   // us a slice
+  const int64_t ctas = ktiles * ((t.units + t.per_cta - 1) / t.per_cta) * t.slices;
+  const double cycles = 200.0 + 160.0 * t.per_cta +
+                        static_cast<double>(x_slow) * t.per_cta / t.cblocks +
+                        1.3 * static_cast<double>(dy_slow) / static_cast<double>(ktiles);
+  const double tma = static_cast<double>((ctas + sms - 1) / sms * t.per_slice) * cycles / 1900.0 +
+                     t.slices * sum;
+  const int64_t slices = bwd_filter_slices(p);
+  const int64_t chunks = (t.chunks + slices - 1) / slices;
+  const int64_t tiles = ktiles * ((rsc + kTileNA - 1) / kTileNA) * slices;
+  const double other = static_cast<double>((tiles + 2 * sms - 1) / (2 * sms) * chunks) * 1.08 +
+                       static_cast<double>(slices) * sum;
+  return tma + 6.0 <= 1.1 * (other + 6.0);
 }
 
 tbn_status launch_bwd_filter_tma(const BwdConvShape& p, const void* x, const void* dy, float* dw,

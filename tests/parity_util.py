@@ -134,3 +134,25 @@ def random_sites(shape, count, seed):
                     corners.append((b, k, p, q))
     s = np.stack(cols, axis=1)
     return np.concatenate([np.array(corners, dtype=np.int64), s.astype(np.int64)], axis=0)
+
+
+def device_us(call, calls=8, repeats=8):
+    """Device time of `call` in microseconds: the least of `repeats` replays of a
+    CUDA graph of `calls` calls in a row."""
+    s = torch.cuda.Stream()
+    best = float("inf")
+    with torch.cuda.stream(s):
+        call()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            for _ in range(calls):
+                call()
+        for _ in range(repeats):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(s)
+            graph.replay()
+            b.record(s)
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3 / calls)
+    return best

@@ -11,7 +11,7 @@ import torch
 import oracle
 import paper_1701_00485_gb300 as tbn
 from paper_1701_00485_gb300 import inputs
-from parity_util import assert_within
+from parity_util import assert_within, device_us
 
 pytestmark = pytest.mark.gpu
 
@@ -201,23 +201,27 @@ def test_bwd_data_calls_in_a_row_cost_no_more_than_alone(case):
     dy = torch.randn(N, P, Q, K, generator=g).to(torch.bfloat16).cuda()
     n = tbn.lib().tbn_conv2d_bwd_data_workspace_bytes(N, C, H, W, K, R, S, *st, *pd)
     ws = torch.empty(n, dtype=torch.uint8, device="cuda")
-    s = torch.cuda.Stream()
-    us = {}
-    with torch.cuda.stream(s):
-        for calls in (1, 8):
-            tbn.tbn_conv2d_bwd_data(dy, codes, alpha, C, (H, W), R, S, st, pd, workspace=ws)
-            torch.cuda.synchronize()
-            graph = torch.cuda.CUDAGraph()
-            with torch.cuda.graph(graph, stream=s):
-                for _ in range(calls):
-                    tbn.tbn_conv2d_bwd_data(dy, codes, alpha, C, (H, W), R, S, st, pd,
-                                            workspace=ws)
-            us[calls] = float("inf")
-            for _ in range(8):
-                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                a.record(s)
-                graph.replay()
-                b.record(s)
-                torch.cuda.synchronize()
-                us[calls] = min(us[calls], a.elapsed_time(b) * 1e3 / calls)
+
+    def call():
+        tbn.tbn_conv2d_bwd_data(dy, codes, alpha, C, (H, W), R, S, st, pd, workspace=ws)
+
+    us = {calls: device_us(call, calls) for calls in (1, 8)}
     assert us[8] <= 1.1 * us[1], us
+
+
+@pytest.mark.parametrize("C,K,R", [(40, 40, 5), (72, 40, 5), (48, 104, 3)])
+def test_bwd_filter_cost_of_slow_rows(C, K, R):
+    """Channel counts whose TMA rows are copied slowly go to the kernel that
+    does without them where that is the quicker one, so none costs much more
+    than the next multiple of 16."""
+    us = {}
+    for c, k in ((C, K), ((C + 15) // 16 * 16, (K + 15) // 16 * 16)):
+        g = inputs.generator(c + k)
+        x = torch.randn(64, 32, 32, c, generator=g).to(torch.bfloat16).cuda()
+        dy = torch.randn(64, 32, 32, k, generator=g).to(torch.bfloat16).cuda()
+        n = tbn.lib().tbn_conv2d_bwd_filter_workspace_bytes(64, c, 32, 32, k, R, R, 1, 1, R // 2,
+                                                            R // 2)
+        ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+        us[c, k] = device_us(lambda: tbn.tbn_conv2d_bwd_filter(x, dy, R, R, (1, 1),
+                                                               (R // 2, R // 2), workspace=ws), 4)
+    assert us[C, K] <= 1.5 * us[(C + 15) // 16 * 16, (K + 15) // 16 * 16], us
