@@ -100,21 +100,8 @@ bool tap_pairs_pay(const ConvProblem& p, const TilePlan& t) {
   return p.C > kBK && t.tile_n > 224 && p.R * p.S > 1;
 }
 
-// Patch mode (gathered activations staged per tile in shared memory) when a
-// tile is whole output rows of one image, the filter spans at most
-// kPatchMaxKBlocks K blocks and two patches fit beside the ring.
 int patch_cap_bytes(const ConvProblem& p, const TilePlan& t) {
-  if (tma_fed(p) || t.tiles_q != 1 || t.bn != 1) return 0;
-  const int64_t kblocks = (p.C * p.R * p.S + kBK - 1) / kBK;
-  if (kblocks > kPatchMaxKBlocks) return 0;
-  const int64_t rows = static_cast<int64_t>(t.bh - 1) * p.sh + p.R;
-  const int64_t elems = rows * (p.W + 2 * p.pw) * p.C;
-  const int64_t cap = ((2 * elems + 32) + 15) / 16 * 16;
-  if (cap > (int64_t(1) << 20)) return 0;
-  if (smem_bytes_for(kModePatch, static_cast<size_t>(cap), static_cast<int>(kblocks)) >
-      static_cast<size_t>(kSmemLimit))
-    return 0;
-  return static_cast<int>(cap);
+  return tma_fed(p) ? 0 : patch_bytes_of(p, t);
 }
 
 }  // namespace

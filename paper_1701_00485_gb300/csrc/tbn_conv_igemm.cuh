@@ -1704,24 +1704,14 @@ inline int ceil_div(int64_t a, int64_t b) { return static_cast<int>((a + b - 1) 
 // TMA activations: whole 64-channel boxes, or 32-channel boxes in pairs.
 inline bool use_tma(const ConvProblem& p) { return p.C % (kBK / 2) == 0 && p.sh <= 2 && p.sw <= 2; }
 inline bool use_ch32(const ConvProblem& p) { return p.C % kBK != 0; }
-// Other multiples of 8 channels: 64-channel boxes, each tap's last one padded.
-inline bool use_tma_pad(const ConvProblem& p) {
-  return !use_tma(p) && p.C % 8 == 0 && p.sh <= 2 && p.sw <= 2 && p.ph <= p.R && p.pw <= p.S;
-}
-inline bool tma_fed(const ConvProblem& p) { return use_tma(p) || use_tma_pad(p); }
-inline int64_t kblocks_of(const ConvProblem& p) {
-  return use_tma_pad(p) ? p.R * p.S * ((p.C + kBK - 1) / kBK)
-                        : (p.C * p.R * p.S + kBK - 1) / kBK;
-}
-
 // Output pixels per tile: whole rows of the output (so one TMA box per tap
 // covers the tile), balanced so the last tile along each axis is not a
 // sliver, at most 256 pixels.  With a fused 2x2 pool a tile holds whole
 // output rows and an even number of them per image.
-inline TilePlan plan_tiles(const ConvProblem& p) {
+inline TilePlan plan_tiles(const ConvProblem& p, bool tma) {
   TilePlan t{};
-  const int stride_w = tma_fed(p) ? static_cast<int>(p.sw) : 1;
-  const int stride_h = tma_fed(p) ? static_cast<int>(p.sh) : 1;
+  const int stride_w = tma ? static_cast<int>(p.sw) : 1;
+  const int stride_h = tma ? static_cast<int>(p.sh) : 1;
   const int bw_max = static_cast<int>(std::min<int64_t>(p.Q, kMaxTileN / stride_w));
   t.tiles_q = ceil_div(p.Q, bw_max);
   t.bw = ceil_div(p.Q, t.tiles_q);
@@ -1753,6 +1743,68 @@ inline TilePlan plan_tiles(const ConvProblem& p) {
   t.oQ = p.Q;
   return t;
 }
+
+// Patch mode (gathered activations staged per tile in shared memory) when a
+// tile is whole output rows of one image, the filter spans at most
+// kPatchMaxKBlocks K blocks and two patches fit beside the ring: the bytes of
+// a patch buffer, else 0.
+inline int patch_bytes_of(const ConvProblem& p, const TilePlan& t) {
+  if (t.tiles_q != 1 || t.bn != 1) return 0;
+  const int64_t kblocks = (p.C * p.R * p.S + kBK - 1) / kBK;
+  if (kblocks > kPatchMaxKBlocks) return 0;
+  const int64_t rows = static_cast<int64_t>(t.bh - 1) * p.sh + p.R;
+  const int64_t elems = rows * (p.W + 2 * p.pw) * p.C;
+  const int64_t cap = ((2 * elems + 32) + 15) / 16 * 16;
+  if (cap > (int64_t(1) << 20)) return 0;
+  if (smem_bytes_for(kModePatch, static_cast<size_t>(cap), static_cast<int>(kblocks)) >
+      static_cast<size_t>(kSmemLimit))
+    return 0;
+  return static_cast<int>(cap);
+}
+
+// Whether padded boxes beat the modes whose threads build the operand.  They do
+// at every channel count but 8 and 24: a tap's box is a K block of its own
+// there, where 64 codes hold eight or nearly three taps, and rows of 16 or 48
+// bytes are copied slowly (2.6 and 3.3 ns a pixel).  For those two the
+// estimates decide, in ns and fitted to 58 layers: a gathered K block 1250 (700
+// up to 128 pixels), a patch 4750 a tile and stride and 600 + 120 C a K block
+// of 256 pixels.  (Batch 64, 32 x 32, 64 filters, padded and else: 8 channels 3
+// x 3 16.4 and 16.4 us, 5 x 5 37.1 and 21.9; 24 channels 5 x 5 32 and 45, 7 x 7
+// 60 and 48.)
+inline bool pad_boxes_pay(const ConvProblem& p) {
+  if ((p.C != 8 && p.C != 24) || p.R * p.S == 1) return true;
+  const TilePlan t = plan_tiles(p, false);
+  // only these widths pool without boxes
+  if (p.pool && (t.tiles_q != 1 || t.T > kMaxTileN || (t.bh & 1) ||
+                 (t.bw != 8 && t.bw != 16 && t.bw != 32)))
+    return true;
+  const int64_t sms = device_sm_count(), tk = ceil_div(p.K, kBM), px = p.N * p.P * p.Q;
+  const int64_t kb = (p.C * p.R * p.S + kBK - 1) / kBK;
+  const int64_t tiles = static_cast<int64_t>(t.tiles_q) * t.tiles_p * t.tiles_n * tk;
+  const double built =
+      patch_bytes_of(p, t) > 0
+          ? 4750.0 * static_cast<double>(p.sh) +
+                static_cast<double>(kb) * (600.0 + 120.0 * static_cast<double>(p.C)) * t.tile_n / kMaxTileN
+          : 1500.0 + static_cast<double>(kb) * (t.tile_n > 128 ? 1250.0 : 700.0);
+  const int64_t T = std::min<int64_t>(kMaxTileN, std::max<int64_t>(16, ((px * tk + sms - 1) / sms + 15) / 16 * 16));
+  const double row = (p.C == 8 ? 2.6 : 3.3) * (p.sh == 1 ? 1.0 : 0.86);
+  const double boxes = static_cast<double>(p.R * p.S) * std::max(250.0, row * static_cast<double>(T)) + 1500.0;
+  return static_cast<double>(((px + T - 1) / T * tk + sms - 1) / sms) * boxes <=
+         static_cast<double>((tiles + sms - 1) / sms) * built;
+}
+
+// Other multiples of 8 channels: 64-channel boxes, each tap's last one padded.
+inline bool use_tma_pad(const ConvProblem& p) {
+  return !use_tma(p) && p.C % 8 == 0 && p.sh <= 2 && p.sw <= 2 && p.ph <= p.R && p.pw <= p.S &&
+         pad_boxes_pay(p);
+}
+inline bool tma_fed(const ConvProblem& p) { return use_tma(p) || use_tma_pad(p); }
+inline int64_t kblocks_of(const ConvProblem& p) {
+  return use_tma_pad(p) ? p.R * p.S * ((p.C + kBK - 1) / kBK)
+                        : (p.C * p.R * p.S + kBK - 1) / kBK;
+}
+
+inline TilePlan plan_tiles(const ConvProblem& p) { return plan_tiles(p, tma_fed(p)); }
 
 // The kernel's kPoolBW for a plan: -1 where a tile cannot pool (whole rows,
 // an even number of them); 1 for rows of other widths than 8, 16 and 32,

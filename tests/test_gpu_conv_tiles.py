@@ -7,7 +7,7 @@ import torch
 import oracle
 import paper_1701_00485_gb300 as tbn
 from paper_1701_00485_gb300 import inputs
-from parity_util import ConvCase, assert_within, random_sites
+from parity_util import ConvCase, assert_within, device_us, random_sites
 
 pytestmark = pytest.mark.gpu
 
@@ -105,6 +105,40 @@ def test_padded_channel_blocks(case):
                       residual=res)
         assert_within(y, want, bound, out_bf16=dt == torch.bfloat16, epilogue=True,
                       what="padded epi %s" % (case,))
+
+
+FEW_CHANNELS = [
+    # few channels under large filters: the modes whose threads build the operand
+    (8, 8, 40, 36, 40, 7, 7, (1, 1), (3, 3)),
+    (4, 24, 33, 40, 72, 9, 9, (1, 1), (4, 4)),
+    (2, 8, 45, 50, 16, 11, 11, (2, 2), (5, 5)),
+]
+
+
+@pytest.mark.parametrize("case", FEW_CHANNELS)
+def test_few_channels(case):
+    c = _case(*case, seed=sum(case[:7]))
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    for dt in (torch.float32, torch.bfloat16):
+        y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, dt)
+        assert_within(y, y_orc, bound, out_bf16=dt == torch.bfloat16,
+                      what="few channels %s" % (case,))
+    assert tbn.tbn_device_error() == 0
+
+
+@pytest.mark.parametrize("R", [7, 11])
+def test_few_channels_cost_no_more_than_more(R):
+    """A K block holds eight taps of 8 channels; a box of each tap's own would
+    make such layers slower than those of 16 channels."""
+    us = {}
+    for C in (8, 16):
+        g = inputs.generator(C)
+        x = torch.randn(64, 32, 32, C, generator=g).to(torch.bfloat16).cuda()
+        codes, alpha = tbn.tbn_quantize_pack(inputs.normal((64, R * R * C), 1.2, g).cuda())
+        out = torch.empty(64, 32, 32, 64, dtype=torch.bfloat16, device="cuda")
+        us[C] = device_us(lambda: tbn.tbn_conv2d_fwd(x, codes, alpha, 64, R, R, (1, 1),
+                                                     (R // 2, R // 2), out=out))
+    assert us[8] <= 1.3 * us[16], us
 
 
 @pytest.mark.parametrize("B,K_in,K_out", [(9, 1000, 70), (64, 2008, 130), (2, 520, 33)])
