@@ -141,6 +141,20 @@ def test_few_channels_cost_no_more_than_more(R):
     assert us[8] <= 1.3 * us[16], us
 
 
+def test_direct_stores_without_a_residual_cost_less_than_with_one():
+    """Outputs that no TMA store takes, stored by a gathering mode: what the
+    residual's requests ahead keep in registers is not paid without one."""
+    g = inputs.generator(65)
+    x = torch.randn(64, 32, 32, 12, generator=g).to(torch.bfloat16).cuda()
+    codes, alpha = tbn.tbn_quantize_pack(inputs.normal((33, 9 * 12), 1.2, g).cuda())
+    out = torch.empty(64, 32, 32, 33, device="cuda")
+    res = torch.randn(64, 32, 32, 33, generator=g).cuda()
+    us = [device_us(lambda: tbn.tbn_conv2d_fwd(x, codes, alpha, 33, 3, 3, (1, 1), (1, 1), out=out,
+                                               out_dtype=torch.float32, residual=r))
+          for r in (None, res)]
+    assert us[0] <= 0.8 * us[1], us
+
+
 @pytest.mark.parametrize("B,K_in,K_out", [(9, 1000, 70), (64, 2008, 130), (2, 520, 33)])
 def test_padded_linear(B, K_in, K_out):
     """Fully-connected layers whose K_in is a multiple of 8 only, with the
