@@ -260,10 +260,13 @@ tbn_status launch_dense_conv_l(const DenseConvArgs& a, size_t smem, bool xn, boo
 
 // ---------------------------------------------------------------- avg pool
 // The mean over H*W in fp32, pixels added in order.  A thread owns kVec
-// adjacent channels of one image and keeps kAvgAhead pixels' loads in flight:
-// the sum is a chain, but its loads are not, and one load per addition made
-// the 128 x 7 x 7 x 512 bf16 pool 14 us of latency for 6.4 MB.
-constexpr int kAvgAhead = 16;
+// adjacent channels of one image and keeps kAhead pixels' loads in flight: the
+// sum is a chain, but its loads are not, and one load per addition made the 128
+// x 7 x 7 x 512 bf16 pool 5.7 us of latency for 6.4 MB (4.2 now).  Few threads
+// keep 16 in flight (32 x 56 x 56 x 64 fp32: 56 us, with eight 83); where they
+// fill the machine eight do, and 16 only crowd the memory (256 x 8 x 8 x 2048
+// bf16: 12.0 us, with 16 15.6).
+constexpr int64_t kAvgManyThreads = 32768;
 
 template <typename TX, int kVec>
 __device__ __forceinline__ void ld_channels(const TX* p, float (&v)[kVec]) {
@@ -280,7 +283,7 @@ __device__ __forceinline__ void ld_channels(const TX* p, float (&v)[kVec]) {
   }
 }
 
-template <typename TX, typename TY, int kVec>
+template <typename TX, typename TY, int kVec, int kAhead>
 __global__ void __launch_bounds__(128) avgpool_global_nhwc_kernel(const TX* __restrict__ x,
                                                                   int64_t N, int64_t HW,
                                                                   int64_t C, float inv,
@@ -290,14 +293,14 @@ __global__ void __launch_bounds__(128) avgpool_global_nhwc_kernel(const TX* __re
   const int64_t b = i / C, c = i - b * C;
   const TX* p = x + b * HW * C + c;
   float acc[kVec] = {};
-  for (int64_t j0 = 0; j0 < HW; j0 += kAvgAhead) {
-    const int n = static_cast<int>(HW - j0 < kAvgAhead ? HW - j0 : kAvgAhead);
-    float v[kAvgAhead][kVec];
+  for (int64_t j0 = 0; j0 < HW; j0 += kAhead) {
+    const int n = static_cast<int>(HW - j0 < kAhead ? HW - j0 : kAhead);
+    float v[kAhead][kVec];
 #pragma unroll
-    for (int j = 0; j < kAvgAhead; ++j)
+    for (int j = 0; j < kAhead; ++j)
       if (j < n) ld_channels<TX, kVec>(p + (j0 + j) * C, v[j]);
 #pragma unroll
-    for (int j = 0; j < kAvgAhead; ++j)
+    for (int j = 0; j < kAhead; ++j)
       if (j < n)
 #pragma unroll
         for (int e = 0; e < kVec; ++e) acc[e] += v[j][e];
@@ -424,21 +427,25 @@ __global__ void __launch_bounds__(256) dense_linear_kernel(const float* __restri
   }
 }
 
+template <typename TX, typename TY, int kVec>
+tbn_status launch_avgpool_v(const void* x, int64_t N, int64_t HW, int64_t C, void* y,
+                            cudaStream_t s) {
+  const float inv = 1.0f / static_cast<float>(HW);
+  const int64_t threads = N * C / kVec;
+  const unsigned blocks = static_cast<unsigned>((threads + 127) / 128);
+  const auto kern = threads >= kAvgManyThreads ? avgpool_global_nhwc_kernel<TX, TY, kVec, 8>
+                                               : avgpool_global_nhwc_kernel<TX, TY, kVec, 16>;
+  kern<<<blocks, 128, 0, s>>>(static_cast<const TX*>(x), N, HW, C, inv, static_cast<TY*>(y));
+  return check_launch("avgpool_global_nhwc_kernel");
+}
+
 template <typename TX, typename TY>
 tbn_status launch_avgpool_t(const void* x, int64_t N, int64_t HW, int64_t C, void* y,
                             cudaStream_t s) {
-  const float inv = 1.0f / static_cast<float>(HW);
   // two channels per load where every pixel's are aligned for it
-  const bool two = C % 2 == 0 && is_aligned(x, 2 * sizeof(TX));
-  const int64_t threads = N * C / (two ? 2 : 1);
-  const unsigned blocks = static_cast<unsigned>((threads + 127) / 128);
-  if (two)
-    avgpool_global_nhwc_kernel<TX, TY, 2><<<blocks, 128, 0, s>>>(
-        static_cast<const TX*>(x), N, HW, C, inv, static_cast<TY*>(y));
-  else
-    avgpool_global_nhwc_kernel<TX, TY, 1><<<blocks, 128, 0, s>>>(
-        static_cast<const TX*>(x), N, HW, C, inv, static_cast<TY*>(y));
-  return check_launch("avgpool_global_nhwc_kernel");
+  return C % 2 == 0 && is_aligned(x, 2 * sizeof(TX))
+             ? launch_avgpool_v<TX, TY, 2>(x, N, HW, C, y, s)
+             : launch_avgpool_v<TX, TY, 1>(x, N, HW, C, y, s);
 }
 
 template <typename TY>
