@@ -127,7 +127,8 @@ def test_dense_tc_cost_of_not_finite_input():
 
 
 @pytest.mark.parametrize("B,K_in,K_out", [(33, 128, 31), (1, 4, 1), (32, 129, 32), (65, 516, 100),
-                                          (31, 252, 1000)])
+                                          (31, 252, 1000), (70, 1, 3), (40, 20, 33),
+                                          (33, 145, 31), (9, 31, 64)])
 def test_dense_linear_tile_edges(B, K_in, K_out):
     """Rows, columns and input chunks at the edges of their tiles, with
     vector (K_in % 4 == 0) and scalar loads.  fp32 sums: K_in 2^-24 sum|x w|."""
@@ -138,6 +139,14 @@ def test_dense_linear_tile_edges(B, K_in, K_out):
     torch.cuda.synchronize()
     want, bound = oracle.dense_linear(x.numpy(), w.numpy())
     assert np.all(np.abs(y.cpu().numpy() - want) <= K_in * 2.0 ** -24 * bound)
+
+
+def test_dense_linear_pays_for_the_inputs_there_are():
+    """16 inputs cost clearly less than a whole chunk of 128."""
+    us = [device_us(lambda: tbn.tbn_dense_linear_fwd(x, w)) for x, w in
+          ((torch.randn(10000, k, device="cuda"), torch.randn(16, k, device="cuda"))
+           for k in (16, 128))]
+    assert us[0] <= 0.85 * us[1], us
 
 
 def test_avgpool_of_many_channels():
