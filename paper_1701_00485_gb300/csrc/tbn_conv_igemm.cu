@@ -57,16 +57,19 @@ __global__ void __launch_bounds__(256) splitk_reduce_kernel(const float* __restr
 // p.ksplit ranges that the caller's workspace holds, and clusters in whole
 // waves of those that the device runs at once (GB300: 36 of four CTAs, 15 of
 // eight).  Costs in ns: a K block as in plan_cost; start, exchange and end,
-// fitted, 3.5 us + 12 ns a pixel in a cluster; two launches 4.5 us + 12 ns a
-// pixel + 80 ns a range, whose sums one thread adds in turn.  Measured, two
-// launches and clusters: 256 x 9216 -> 4096 21.0 and 19.2 us, 256 x 4096 ->
-// 4096 15.6 and 13.8, 256 x 4096 -> 1000 11.4 and 9.3 (two tiles of 128
-// images, six ranges), 64 x 2048 -> 300 7.9 and 5.4; even at 64 x 25088 -> 128
-// (98 ranges of four K blocks), beyond which two launches win.
+// fitted, 3.5 us + 12 ns a pixel in a cluster (24 where K is no multiple of four
+// and the sums go one by one); two launches 4.5 us + 12 ns a pixel + 80 ns a
+// range (60), whose sums one thread adds in turn.  Measured, two launches and
+// clusters: 256 x 9216 -> 4096 21.0 and 19.2 us, 256 x 4096 -> 4096 15.6 and
+// 13.8, 256 x 4096 -> 1000 11.4 and 9.3 (two tiles of 128 images, six ranges), 64
+// x 2048 -> 300 7.9 and 5.4; even at 64 x 25088 -> 128 (98 ranges of four K
+// blocks), beyond which two launches win; 256 x 25088 -> 10 14.4 and 17.4, 64 x
+// 16384 -> 10 10.0 and 12.6, 128 x 4096 -> 1001 9.5 and 10.8.
 int cluster_split(const ConvProblem& p, TilePlan& t) {
   const int64_t kb = kblocks_of(p), tk = ceil_div(p.K, kBM);
   const auto block = [](int64_t bn) { return 215.0 + 0.25 * bn; };
-  double cost = ceil_div(kb, p.ksplit) * block(t.bn) + 4500.0 + 12.0 * t.bn + 80.0 * p.ksplit;
+  const bool vec = p.K % 4 == 0;
+  double cost = ceil_div(kb, p.ksplit) * block(t.bn) + 4500.0 + 12.0 * t.bn + (vec ? 80.0 : 60.0) * p.ksplit;
   const int parts0 = t.tiles_n;
   int best = 1;
   for (int parts = parts0; parts <= 4 * parts0; ++parts) {
@@ -75,7 +78,7 @@ int cluster_split(const ConvProblem& p, TilePlan& t) {
     for (int S = 2; S <= std::min(kMaxCluster, p.ksplit); ++S) {
       const int per = ceil_div(kb, S), fit = igemm_max_clusters(S);
       if ((S - 1) * per >= kb || fit < 1) continue;
-      const double c = ceil_div(parts * tk, fit) * (per * block(bn) + 3500.0 + 12.0 * bn);
+      const double c = ceil_div(parts * tk, fit) * (per * block(bn) + 3500.0 + (vec ? 12.0 : 24.0) * bn);
       // narrower tiles only for a clear gain
       if (c >= (parts > t.tiles_n && best > 1 ? 0.95 : 1.0) * cost) continue;
       cost = c;

@@ -239,6 +239,20 @@ def test_linear_split_in_clusters(B, K_in, K_out, dtype, res):
     assert tbn.tbn_device_error() == 0
 
 
+def test_linear_split_of_many_ranges_and_few_outputs():
+    """Very long filters and a count of outputs that is no multiple of four: the
+    two launches, whose many ranges a cluster's eight cannot match."""
+    us = {}
+    for K_out in (10, 12):
+        x = torch.randn(64, 16384, device="cuda").to(torch.bfloat16)
+        codes, alpha = tbn.tbn_quantize_pack(torch.randn(K_out, 16384, device="cuda"))
+        ws = torch.empty(tbn.tbn_linear_workspace_bytes(64, 16384, K_out), dtype=torch.uint8,
+                         device="cuda")
+        out = torch.empty(64, K_out, dtype=torch.bfloat16, device="cuda")
+        us[K_out] = device_us(lambda: tbn.tbn_linear_fwd_ws(x, codes, alpha, K_out, ws, out=out))
+    assert us[10] <= 0.92 * us[12], us
+
+
 @pytest.mark.parametrize("case", [
     (3, 64, 28, 28, 72, 3, 3, (1, 1), (1, 1)),      # even map: runs of row pairs
     (2, 64, 13, 11, 136, 3, 3, (1, 1), (1, 1)),     # odd: the last row and column drop
