@@ -85,7 +85,7 @@ _lib = None
 
 
 # exports of this binding's own, not declared in tbn.h
-_PRIVATE = ["tbn_packed_call"]
+_PRIVATE = ["tbn_packed_call", "tbn_conv_mode"]
 ABI_VERSION = 9  # must match TBN_ABI_VERSION in include/tbn.h
 
 
@@ -158,6 +158,8 @@ def lib():
             fn.restype = res
         L.tbn_packed_call.argtypes = [I32, ctypes.c_char_p]
         L.tbn_packed_call.restype = I32
+        L.tbn_conv_mode.argtypes = [ctypes.c_char_p]
+        L.tbn_conv_mode.restype = I32
         _lib = L
         return L
 
@@ -416,6 +418,21 @@ def tbn_space_to_depth(x: torch.Tensor, R: int, S: int, stride=(4, 4), pad=(0, 0
 
 def _bwd_shape(N, C, H, W, K, R, S, stride, pad):
     return (N, C, H, W, K, R, S, stride[0], stride[1], pad[0], pad[1])
+
+
+_CONV_MODES = ("tma64", "tma32", "gather", "patch", "s2d", "pad", "rowpair", "tappair")
+
+
+def _conv_mode(N, C, H, W, K, R, S, stride=(1, 1), pad=(0, 0), out_dtype=torch.bfloat16,
+               residual: bool = False, pool: int = 0, layout: int = TBN_NHWC,
+               algo: int = TBN_CONV_AUTO) -> str | None:
+    """How the implicit GEMM would feed this bf16 convolution of aligned tensors
+    (csrc/tbn_conv_igemm.cuh), None where another algorithm would take it."""
+    ydt = TBN_F32 if out_dtype == torch.float32 else TBN_BF16
+    a = 256   # stands in for every pointer: only alignment counts
+    mode = lib().tbn_conv_mode(_PACK[23](a, TBN_BF16, layout, N, C, H, W, a, a, K, R, S, *stride,
+                                         *pad, a, ydt, 0, a if residual else 0, pool, algo, 0))
+    return _CONV_MODES[mode] if mode >= 0 else None
 
 
 def tbn_conv2d_bwd_data(dy: torch.Tensor, codes: torch.Tensor, alpha: torch.Tensor, C: int,

@@ -833,3 +833,24 @@ extern "C" tbn_status tbn_packed_call(int op, const int64_t* v) {
   }
   return fail(TBN_ERR_INVALID_ARG, "packed call: unknown operation %d", op);
 }
+
+// The implicit GEMM's activation mode for a convolution (arguments as in
+// operation 1 above; nothing is launched), or -1 where its algorithm is another
+// or the call would be refused.  The tests ask, so that a case meant for one
+// mode cannot silently run in another.
+extern "C" int tbn_conv_mode(const int64_t* v) {
+  const auto ptr = [&](int i) { return reinterpret_cast<void*>(static_cast<uintptr_t>(v[i])); };
+  const tbn_epilogue e{static_cast<int>(v[18]), ptr(19), static_cast<int>(v[20])};
+  ConvProblem p{};
+  if (validate_conv(ptr(0), static_cast<tbn_dtype>(v[1]), static_cast<tbn_layout>(v[2]), v[3],
+                    v[4], v[5], v[6], static_cast<uint32_t*>(ptr(7)), static_cast<float*>(ptr(8)),
+                    v[9], v[10], v[11], v[12], v[13], v[14], v[15], ptr(16),
+                    static_cast<tbn_dtype>(v[17]), &e, &p) != TBN_OK)
+    return -1;
+  const auto algo = static_cast<tbn_conv_algo>(v[21]);
+  const bool igemm =
+      algo == TBN_CONV_AUTO
+          ? conv_igemm_pools_any_width(p) || pick_algo(p) == TBN_CONV_IMPLICIT_GEMM
+          : algo == TBN_CONV_IMPLICIT_GEMM && conv_igemm_unsupported_reason(p)[0] == '\0';
+  return igemm ? conv_igemm_mode(p) : -1;
+}

@@ -111,6 +111,27 @@ int patch_cap_bytes(const ConvProblem& p, const TilePlan& t) {
 
 bool conv_igemm_uses_tma(const ConvProblem& p) { return use_tma(p); }
 
+namespace {
+
+// How the activations of a planned launch reach the ring (kMode...).
+int mode_of(const ConvProblem& p, const TilePlan& t, bool s2d) {
+  if (s2d) return kModeS2d;
+  if (t.rowpair) return kModeRowPair;
+  if (use_tma(p)) {
+    if (!use_ch32(p)) return kModeTma64;
+    return tap_pairs_pay(p, t) ? kModeTapPair : kModeTma32;
+  }
+  if (use_tma_pad(p)) return kModeTmaPad;
+  return patch_cap_bytes(p, t) > 0 ? kModePatch : kModeGather;
+}
+
+// Tensor-memory columns of each resident K block (space-to-depth mode).
+int resident_cols(const ConvProblem& p) {
+  return p.layout == TBN_S2D_NHWC ? 8 * ceil_div(p.sh * p.sh * p.C, 16) : 0;
+}
+
+}  // namespace
+
 // Split K when the output tiles fill fewer than half the SMs and the filter
 // has at least 8 K blocks.  The tensor core's time per K block is
 // proportional to the tile's pixels, but a CTA's time per K block is not
@@ -208,10 +229,16 @@ bool conv_igemm_pools_any_width(const ConvProblem& p) {
   return pool_width(p, plan_tiles(p)) == 1;
 }
 
+int conv_igemm_mode(const ConvProblem& p0) {
+  const bool s2d = p0.layout == TBN_S2D_NHWC;
+  const ConvProblem p = s2d ? s2d_problem(p0) : p0;
+  return mode_of(p, plan_conv(p, resident_cols(p0)), s2d);
+}
+
 tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
   const bool s2d = p0.layout == TBN_S2D_NHWC;
   const ConvProblem p = s2d ? s2d_problem(p0) : p0;
-  const int resident = s2d ? 8 * ceil_div(p0.sh * p0.sh * p0.C, 16) : 0;
+  const int resident = resident_cols(p0);
   TilePlan t = plan_conv(p, resident);
   const bool split = p.ksplit > 1 && p.partial != nullptr;
   const int cluster = split && is_aligned(p.partial, 16) ? cluster_split(p, t) : 1;
@@ -301,29 +328,24 @@ tbn_status launch_conv_igemm(const ConvProblem& p0, cudaStream_t s) {
           p.ydt == TBN_BF16 ? 1 : 0);
     return check_launch("splitk_reduce_kernel");
   }
-  if (s2d) {
-    return tst ? launch_t<kModeS2d, 0, true, false>(p, t, a, s)
-               : launch_t<kModeS2d, 0, false, false>(p, t, a, s);
-  }
-  if (t.rowpair) return launch_igemm_rowpair(p, t, a, s);
-  if (use_tma(p) && use_ch32(p) && tap_pairs_pay(p, t))
-    return launch_igemm_tappair(p, t, a, pw, tst, a.wq != nullptr, s);
-  if (use_tma(p) && use_ch32(p)) {
-    return launch_igemm_tma32(p, t, a, pw, tst, a.wq != nullptr, s);
-  }
-  if (use_tma(p)) {
-    return launch_igemm_tma64(p, t, a, pw, tst, a.wq != nullptr, s);
-  }
-  if (use_tma_pad(p)) return launch_igemm_pad(p, t, a, pw, tst, s);
-  const int cap = patch_cap_bytes(p, t);
-  if (cap > 0) {
-    a.PR = (t.bh - 1) * a.sh + a.R;
-    a.PW = a.W + 2 * a.pw;
-    a.patch_cap = cap;
-    a.patch_bulk = a.pw == 0 ? 1 : 0;
-    a.x_bytes = static_cast<long long>(p.N) * p.H * p.W * p.C * 2;
-    return tst ? launch_pool<kModePatch, true, false>(p, t, a, pw, s)
-               : launch_pool<kModePatch, false, false>(p, t, a, pw, s);
+  const bool fuse = a.wq != nullptr;
+  switch (mode_of(p, t, s2d)) {
+    case kModeS2d:
+      return tst ? launch_t<kModeS2d, 0, true, false>(p, t, a, s)
+                 : launch_t<kModeS2d, 0, false, false>(p, t, a, s);
+    case kModeRowPair: return launch_igemm_rowpair(p, t, a, s);
+    case kModeTapPair: return launch_igemm_tappair(p, t, a, pw, tst, fuse, s);
+    case kModeTma32: return launch_igemm_tma32(p, t, a, pw, tst, fuse, s);
+    case kModeTma64: return launch_igemm_tma64(p, t, a, pw, tst, fuse, s);
+    case kModeTmaPad: return launch_igemm_pad(p, t, a, pw, tst, s);
+    case kModePatch:
+      a.PR = (t.bh - 1) * a.sh + a.R;
+      a.PW = a.W + 2 * a.pw;
+      a.patch_cap = patch_cap_bytes(p, t);
+      a.patch_bulk = a.pw == 0 ? 1 : 0;
+      a.x_bytes = static_cast<long long>(p.N) * p.H * p.W * p.C * 2;
+      return tst ? launch_pool<kModePatch, true, false>(p, t, a, pw, s)
+                 : launch_pool<kModePatch, false, false>(p, t, a, pw, s);
   }
   return tst ? launch_pool<kModeGather, true, false>(p, t, a, pw, s)
              : launch_pool<kModeGather, false, false>(p, t, a, pw, s);

@@ -140,6 +140,8 @@ tbn_status launch_conv_direct(const ConvProblem& p, cudaStream_t s);
 // Empty string when the implicit-GEMM kernel can run `p`, else the reason.
 const char* conv_igemm_unsupported_reason(const ConvProblem& p);
 tbn_status launch_conv_igemm(const ConvProblem& p, cudaStream_t s);
+// The activation mode (kMode... of tbn_conv_igemm.cuh) that `p` is launched in.
+int conv_igemm_mode(const ConvProblem& p);
 // True for a fused pool that only AUTO sends to the implicit GEMM.
 bool conv_igemm_pools_any_width(const ConvProblem& p);
 // Space-to-depth layout change of a bf16 NCHW or NHWC input for the

@@ -54,6 +54,7 @@ def test_fused_quant_conv_equals_separate(case):
 def test_fused_quant_conv_equals_separate_on_paired_blocks(case):
     N, C, H, W, K, R, S, st, pd, wscale = case
     W = W + S - 1 if pd == 0 else W
+    assert tbn._conv_mode(N, C, H, W, K, R, S, (st, st), (pd, pd)) in ("tappair", "rowpair")
     test_fused_quant_conv_equals_separate((N, C, H, W, K, R, S, st, pd, wscale))
 
 

@@ -93,6 +93,7 @@ PADDED = [
 
 @pytest.mark.parametrize("case", PADDED)
 def test_padded_channel_blocks(case):
+    assert tbn._conv_mode(*case) == "pad"
     c = _case(*case, seed=sum(case[:7]))
     y_orc, bound = c.oracle_full(torch.bfloat16)
     y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.float32,
@@ -109,14 +110,17 @@ def test_padded_channel_blocks(case):
 
 FEW_CHANNELS = [
     # few channels under large filters: the modes whose threads build the operand
-    (8, 8, 40, 36, 40, 7, 7, (1, 1), (3, 3)),
-    (4, 24, 33, 40, 72, 9, 9, (1, 1), (4, 4)),
-    (2, 8, 45, 50, 16, 11, 11, (2, 2), (5, 5)),
+    (64, 8, 32, 31, 40, 7, 7, (1, 1), (3, 3), "patch"),
+    (64, 24, 30, 32, 72, 9, 9, (1, 1), (4, 4), "gather"),
+    (2, 8, 45, 50, 16, 11, 11, (2, 2), (5, 5), "patch"),
+    (8, 8, 40, 36, 40, 7, 7, (1, 1), (3, 3), "pad"),    # one wave: boxes cut finer
 ]
 
 
 @pytest.mark.parametrize("case", FEW_CHANNELS)
 def test_few_channels(case):
+    *case, mode = case
+    assert tbn._conv_mode(*case) == mode
     c = _case(*case, seed=sum(case[:7]))
     y_orc, bound = c.oracle_full(torch.bfloat16)
     for dt in (torch.float32, torch.bfloat16):
@@ -188,6 +192,7 @@ def test_tap_pairs(case, pool):
     Wl, codes, alpha = c.quantize_gpu(tbn.TBN_NHWC)
     x = c.x.to(torch.bfloat16).permute(0, 2, 3, 1).contiguous().cuda()
     for dt in (torch.float32, torch.bfloat16):
+        assert tbn._conv_mode(*case, out_dtype=dt, pool=pool) == "tappair"
         y = tbn.tbn_conv2d_fwd(x, codes, alpha, K, R, S, st, pad, out_dtype=dt, relu=bool(pool),
                                pool=pool)
         assert tbn.tbn_device_error() == 0
@@ -285,16 +290,20 @@ def test_pool_of_any_width(case):
 
 ROW_PAIRS = [
     # N, C, H, W, K, R, S, stride, pad: at most 64 filters, an even number of
-    # output rows, inputs of at least 128 KiB
-    (6, 64, 56, 56, 64, 3, 3, (1, 1), (1, 1)),      # 64 filters, several tiles per CTA
-    (9, 128, 14, 17, 40, 3, 3, (1, 1), (1, 1)),     # ragged filters, odd width
-    (5, 64, 21, 24, 8, 2, 3, (1, 2), (0, 1)),       # R = 2, column stride 2
-    (3, 64, 18, 60, 64, 5, 5, (1, 1), (2, 2)),
+    # output rows, and work for two waves of tiles, so that pairs pay
+    (64, 64, 28, 28, 64, 3, 3, (1, 1), (1, 1)),     # 64 filters, several tiles per CTA
+    (64, 128, 28, 27, 40, 3, 3, (1, 1), (1, 1)),    # ragged filters, odd width, 128 channels
+    (48, 64, 33, 56, 8, 2, 3, (1, 2), (0, 1)),      # R = 2, column stride 2
+    (64, 64, 30, 31, 56, 5, 5, (1, 1), (2, 2)),
+    (90, 64, 41, 27, 64, 2, 2, (1, 1), (0, 0)),     # no padding
+    (300, 64, 12, 28, 24, 3, 3, (1, 2), (1, 1)),    # a tile holds two images
 ]
 
 
 @pytest.mark.parametrize("case", ROW_PAIRS)
 def test_row_pairs(case):
+    for residual in (False, True):
+        assert tbn._conv_mode(*case, residual=residual) == "rowpair"
     c = _case(*case, seed=sum(case[:7]))
     y_orc, bound = c.oracle_full(torch.bfloat16)
     assert y_orc.shape[2] % 2 == 0
@@ -307,23 +316,31 @@ def test_row_pairs(case):
 
 
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
-def test_row_pairs_not_finite(value):
+@pytest.mark.parametrize("case", [
+    (64, 64, 28, 28, 48, 3, 3, (1, 1), (1, 1)),
+    (48, 64, 33, 56, 8, 2, 3, (1, 2), (0, 1)),
+    (64, 64, 30, 31, 56, 5, 5, (1, 1), (2, 2)),
+])
+def test_row_pairs_not_finite(case, value):
     """An infinite or NaN input reaches the outputs whose taps read it and no
-    others, although both rows of a pair multiply it."""
+    others, although both rows of a pair are computed from the same boxes."""
+    assert tbn._conv_mode(*case) == "rowpair"
+    N, C, H, W, K, R, S, st, pd = case
     g = inputs.generator(11)
-    x = torch.randn(64, 64, 28, 28, generator=g)
+    x = torch.randn(N, C, H, W, generator=g)
     x[2, 5, 7, 9] = value       # an odd row: the first tap row of one pair, the last of another
     x[4, 60, 0, 0] = value
-    x[33, 1, 14, 27] = value
-    x[63, 63, 27, 3] = value
-    c = ConvCase(x, inputs.normal((48, 64, 3, 3), 1.2, g), (1, 1), (1, 1))
+    x[33, 1, 14, W - 1] = value
+    x[N - 1, 63, H - 1, 3] = value
+    c = ConvCase(x, inputs.normal((K, C, R, S), 1.2, g), st, pd)
     y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16)
     assert tbn.tbn_device_error() == 0
-    wt, al = oracle.quantize(c.W.reshape(48, -1).numpy())
+    wt, al = oracle.quantize(c.W.reshape(K, -1).numpy())
     w = torch.from_numpy((wt * al[:, None]).reshape(c.W.shape))
-    ref = torch.nn.functional.conv2d(x.to(torch.bfloat16).double(), w.double(), padding=1).numpy()
+    ref = torch.nn.functional.conv2d(x.to(torch.bfloat16).double(), w.double(), stride=st,
+                                     padding=pd).numpy()
     fin = torch.isfinite(torch.from_numpy(ref)).numpy()
-    assert 48 * 20 < (~fin).sum() < 48 * 40
+    assert K * 4 <= (~fin).sum() <= K * 4 * R * S
     assert (torch.isnan(torch.from_numpy(y)).numpy() == torch.isnan(torch.from_numpy(ref)).numpy()).all()
     inf = ~fin & ~torch.isnan(torch.from_numpy(ref)).numpy()
     assert (y[inf] == ref[inf]).all()
