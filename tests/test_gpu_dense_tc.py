@@ -51,14 +51,59 @@ def test_dense_tc_matches_oracle(case):
 
 
 def test_dense_tc_weight_terms():
-    """Weights that need all three terms: one tap, so each output is a single
-    product rounded once to bf16, at most half an ulp away."""
+    """Weights that need all three terms: two taps cancel to a few units of the
+    24th bit, which the result holds exactly; without the third term, or with it
+    in the wrong place, it is 0 or a multiple of 2^-15."""
     g = inputs.generator(9)
     x = torch.ones(1, 1, 8, 8, dtype=torch.bfloat16)
-    w = (torch.rand(64, 1, 1, 1, generator=g) + 1) * (1 + 2.0 ** -23)
+    x[..., 1::2] = -1.0
+    w0 = torch.randint(1 << 23, (1 << 24) - 8, (64,), generator=g)   # 24 bits, [1, 2)
+    d = torch.randint(1, 8, (64,), generator=g)
+    w = torch.stack((w0 + d, w0), 1).float().reshape(64, 1, 1, 2) * 2.0 ** -23
+    assert torch.equal(w.double() * 2.0 ** 23, torch.stack((w0 + d, w0), 1).reshape(w.shape).double())
     y = _run(x, w, (1, 2), (0, 0))
-    want = w.reshape(1, 64, 1, 1).double().numpy() * np.ones(y.shape)
-    assert np.array_equal(y, torch.from_numpy(want).to(torch.bfloat16).float().numpy())
+    want = (d.double() * 2.0 ** -23).reshape(1, 64, 1, 1).numpy() * np.ones(y.shape)
+    assert np.array_equal(y.astype(np.float64), want)
+
+
+@pytest.mark.parametrize("case", [
+    (8, 3, 64, 64, 7, 7, (2, 2), (3, 3)),     # the stem's filter, three weight blocks and two more
+    (8, 1, 64, 64, 3, 3, (2, 2), (1, 1)),
+    (8, 4, 64, 64, 5, 7, (2, 2), (2, 3)),
+])
+def test_dense_tc_sums_in_fp32(case):
+    """The sums' own error: two further channels, one tap each, take the exact
+    result away from the first filter's outputs (rounded to bf16, then what that
+    leaves), so what remains is the rounding of the sums, and the output's bf16
+    hides none of it.  At most n additions of half a unit of sum|x w| each; the
+    rms is below that of fp32 sums tap by tap."""
+    N, C, H, W, R, S, st, pd = case
+    g = inputs.generator(sum(case[:6]))
+    x = torch.randn(N, C, H, W, generator=g).to(torch.bfloat16)
+    w = inputs.he_normal(8, C, R, S, g)
+    conv = torch.nn.functional.conv2d
+    ref = conv(x.double(), w[:1].double(), stride=st, padding=pd)[:, 0]
+    mag = conv(x.double().abs(), w[:1].double().abs(), stride=st, padding=pd)[:, 0].numpy()
+    P, Q = ref.shape[1:]
+    xe = torch.zeros(N, C + 2, H, W, dtype=torch.bfloat16)
+    xe[:, :C] = x
+    left = ref
+    for i in range(2):
+        xe[:, C + i, :P * st[0]:st[0], :Q * st[1]:st[1]] = (-left).to(torch.bfloat16)
+        left = left + (-left).to(torch.bfloat16).double()
+    we = torch.zeros(8, C + 2, R, S)
+    we[:, :C] = w
+    we[:, C:, pd[0], pd[1]] = 1.0
+    err = {}
+    for dt in (torch.bfloat16, torch.float32):    # tensor cores; CUDA cores, tap by tap
+        y = tbn.tbn_dense_conv2d_fwd(xe.cuda(), we.cuda(), st, pd, layout=tbn.TBN_NCHW_NHWC,
+                                     out_dtype=dt)
+        torch.cuda.synchronize()
+        err[dt] = (y[..., 0].double().cpu() - left).numpy()
+    e = err[torch.bfloat16]
+    assert np.all(np.abs(e) <= C * R * S * 2.0 ** -24 * mag + 2.0 ** -8 * np.abs(left.numpy()))
+    rms = {dt: float(np.sqrt(np.mean(v ** 2))) for dt, v in err.items()}
+    assert rms[torch.bfloat16] <= rms[torch.float32], rms
 
 
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.3e38])
