@@ -392,9 +392,6 @@ __device__ __forceinline__ void add_cluster_sums(const IgArgs& a) {
   }
 }
 
-// kPoolBW: 0 = no pool; 8, 16, 32 = fused 2x2/2 max pool for tiles of whole
-// output rows of that width; 1 = of any width (a.bw).  kTmaStore: bf16 output
-// through the staging tile and TMA stores (else direct global stores).
 // Fused quantization prologue: CTA b quantizes filters [b K / G, (b + 1) K / G)
 // exactly as the quantize kernel does (the same per-word fields and sums,
 // reduced per filter in the same order: bitwise the same codes and alpha),
@@ -524,8 +521,11 @@ struct TapPairs {
   }
 };
 
-// kMode: how activations reach the ring (kModeTma64 / kModeTma32 /
-// kModeGather / kModePatch).
+// kMode: how activations reach the ring (one of the eight kMode... above).
+// kPoolBW: 0 = no pool; 8, 16, 32 = fused 2x2/2 max pool for tiles of whole
+// output rows of that width; 1 = of any width (a.bw).  kTmaStore: bf16 output
+// through the staging tile and TMA stores (else direct global stores).  kFuse:
+// with the quantization prologue.
 template <int kMode, int kPoolBW, bool kTmaStore, bool kFuse>
 __global__ void __launch_bounds__(threads_for<kMode>(), 1)
     conv_igemm_kernel(const __grid_constant__ CUtensorMap tmap_x,
