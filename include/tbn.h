@@ -116,7 +116,8 @@ typedef enum {
   TBN_CONV_DIRECT = 1,        /* CUDA-core direct convolution, any layout/dtype   */
   TBN_CONV_IMPLICIT_GEMM = 2, /* tcgen05 implicit GEMM, NHWC bf16 x; activations
                                  by TMA when C % 8 == 0 and the strides are 1 or
-                                 2, else gathered by threads; a fused pool over
+                                 2 (at 8 and 24 channels where that is estimated
+                                 quicker), else gathered by threads; a fused pool over
                                  rows of 8, 16 or 32 (AUTO also sends TMA-fed
                                  layers with other rows of up to 128 here) */
   TBN_CONV_SMALL_TAPS = 3     /* tensor-core convolution for short filters,

@@ -41,7 +41,8 @@
 //                   the last box of a tap reaches past C and arrives
 //                   zero-filled there, so whatever codes stand in those
 //                   columns add zero, and whole steps of 16 past C are
-//                   skipped.  Otherwise gather warps assemble the rows from
+//                   skipped (8 and 24 channels: see pad_boxes_pay).
+//                   Otherwise gather warps assemble the rows from
 //                   a per-K-block table of (tap, channel) offsets.
 //   D               fp32 in tensor memory (256 columns).  Epilogue warps read
 //                   lane = filter, column = pixel, multiply by 2 * alpha (Eq. 1
