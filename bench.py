@@ -87,7 +87,7 @@ WORKLOADS = {
 CONV_TRAFFIC = {"sources": ["paper_1701_00485_gb300/csrc/tbn_conv_igemm.cuh",
                             "paper_1701_00485_gb300/csrc/tbn_conv_igemm.cu",
                             "paper_1701_00485_gb300/csrc/tbn_device.cuh"],
-                "sha256_16": "903afa2b252578e8", "bytes_per_launch": 47.82e6}
+                "sha256_16": "91f7e3d7c974b8d8", "bytes_per_launch": 47.87e6}
 
 
 def measured_traffic(rec):
