@@ -34,11 +34,12 @@
 //
 // The kernel is launched as a programmatic dependent of the previous kernel
 // on the stream.  Codes, inputs and residual may be that kernel's output, so
-// all are read behind griddepcontrol.wait; before it the first ring of code
-// boxes is asked for in L2, so in a chain of layers the weight stream of one
-// starts while the previous one finishes (batch 1, weights not in L2: 4096
-// square 5.1 us a call, 5.4 without; 8192 square 9.0; batch 8, 1024 square 3.3
-// and 3.6).
+// all are read behind griddepcontrol.wait; before it the first ring of stages is
+// announced to its barriers and its code boxes are asked for in L2, so that
+// behind the wait only copies are issued.  Batch 1, weights not in L2, in a
+// chain of layers: 4096 square 4.2 us a call, 8192 square 8.7 (5.4 and 9.0 with
+// all of it behind the wait; 5.3 and 10.3 with the codes read ahead of it);
+// batch 2, 9216 -> 300 in L2: 5.4, 7.0 and 5.7.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -250,16 +251,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     // strided) code matrix instead of one.  Consumers do not depend on the
     // order: a stage's data position only enters through these coordinates.
     const int k_start = static_cast<int>((static_cast<int64_t>(blockIdx.x) * a.nks) / gridDim.x);
-    int it = 0;                      // stages issued so far
-    int slot = 0;                    // it % stages
-    uint32_t empty_parity = 1;       // parity of the release before use it / stages
     // Codes and inputs may come from the previous kernel, so nothing is read
-    // before the wait.  The first ring of code boxes is only asked for in L2
-    // until then (a hint).
-    if (elected && static_cast<int>(blockIdx.x) * a.n_t < a.T)
-      for (int i = 0, kc = k_start; i < min(a.stages, a.nks); ++i) {
+    // before the wait.  Until then the first ring is only announced to its
+    // barriers and its code boxes asked for in L2 (a hint).
+    const int first = static_cast<int>(blockIdx.x) * a.n_t < a.T ? min(a.stages, a.nks) : 0;
+    const auto next = [&](int kc) { return kc + 1 == a.nks ? 0 : kc + 1; };
+    if (elected)
+      for (int i = 0, kc = k_start; i < first; ++i, kc = next(kc)) {
+        mbar_arrive_expect_tx(&full_bar[i], a.stage_bytes);
         tma_prefetch_2d(&tmap_w, kc * kWordsPerStage, static_cast<int>(blockIdx.x) * a.n_t * 16);
-        if (++kc == a.nks) kc = 0;
       }
     __syncwarp();
     grid_dependency_wait();
@@ -274,25 +274,35 @@ __global__ void __launch_bounds__(kThreads, 1)
         tma_load_3d(st + a.w_bytes, &tmap_x, &full_bar[sl], 0, 0, kc * (kCodesPerStage / 8));
       }
     };
+    const auto load_stage = [&](int sl, int kc, int band) {
+      tma_load_2d(ring_ptr + static_cast<size_t>(sl) * a.stage_bytes, &tmap_w, &full_bar[sl],
+                  kc * kWordsPerStage, band * a.n_t * 16);
+      load_x(sl, kc);
+    };
+    if (elected)
+      for (int i = 0, kc = k_start; i < first; ++i, kc = next(kc))
+        load_stage(i, kc, static_cast<int>(blockIdx.x));
+    __syncwarp();
+    int it = first;                          // stages issued so far
+    int slot = first == a.stages ? 0 : first;   // it % stages
+    uint32_t empty_parity = first == a.stages ? 0u : 1u;   // of the release before use it / stages
     for (int r = 0; r < a.rounds; ++r) {
       const int band = blockIdx.x + r * gridDim.x;
       if (band * a.n_t >= a.T) break;
-      int kc = k_start;
-      for (int ks = 0; ks < a.nks; ++ks) {
+      int kc = r == 0 ? (k_start + first) % a.nks : k_start;
+      for (int ks = r == 0 ? first : 0; ks < a.nks; ++ks) {
         bool ok = true;
         if (it >= a.stages)
           ok = mbar_wait_sleep(&empty_bar[slot], empty_parity, &abort_flag, a.err, kWaitLimitNs);
         // one decision for the whole warp (lane 0's)
         if (!__shfl_sync(0xffffffffu, ok && !abort_flag, 0)) break;
         if (elected) {
-          uint8_t* st = ring_ptr + static_cast<size_t>(slot) * a.stage_bytes;
           mbar_arrive_expect_tx(&full_bar[slot], a.stage_bytes);
-          tma_load_2d(st, &tmap_w, &full_bar[slot], kc * kWordsPerStage, band * a.n_t * 16);
-          load_x(slot, kc);
+          load_stage(slot, kc, band);
         }
         __syncwarp();
         ++it;
-        if (++kc == a.nks) kc = 0;
+        kc = next(kc);
         if (++slot == a.stages) {
           slot = 0;
           empty_parity ^= 1u;
