@@ -288,6 +288,34 @@ def test_pool_of_any_width(case):
         tbn.tbn_conv2d_fwd(*args, relu=True, pool=2, algo=tbn.TBN_CONV_IMPLICIT_GEMM)
 
 
+FEW_FILTERS = [
+    # at most 64 filters and an even number of output rows, but work for one wave
+    # of tiles only: runs of pixels
+    (6, 64, 56, 56, 64, 3, 3, (1, 1), (1, 1)),
+    (9, 128, 14, 17, 40, 3, 3, (1, 1), (1, 1)),     # ragged filters, odd width
+    (5, 64, 21, 24, 8, 2, 3, (1, 2), (0, 1)),       # R = 2, column stride 2
+    (3, 64, 18, 60, 64, 5, 5, (1, 1), (2, 2)),
+]
+
+
+@pytest.mark.parametrize("case", FEW_FILTERS)
+def test_few_filters(case):
+    assert tbn._conv_mode(*case) == "tma64"
+    _check_staged_outputs(case, "few filters")
+
+
+def _check_staged_outputs(case, what):
+    c = _case(*case, seed=sum(case[:7]))
+    y_orc, bound = c.oracle_full(torch.bfloat16)
+    assert y_orc.shape[2] % 2 == 0
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16)
+    assert_within(y, y_orc, bound, out_bf16=True, what="%s %s" % (what, case))
+    res = torch.randn(*y_orc.shape, generator=inputs.generator(3)).to(torch.bfloat16)
+    want = oracle.epilogue(y_orc, res.float().numpy(), relu=True)
+    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16, relu=True, residual=res)
+    assert_within(y, want, bound, out_bf16=True, epilogue=True, what="%s epi %s" % (what, case))
+
+
 ROW_PAIRS = [
     # N, C, H, W, K, R, S, stride, pad: at most 64 filters, an even number of
     # output rows, and work for two waves of tiles, so that pairs pay
@@ -304,27 +332,20 @@ ROW_PAIRS = [
 def test_row_pairs(case):
     for residual in (False, True):
         assert tbn._conv_mode(*case, residual=residual) == "rowpair"
-    c = _case(*case, seed=sum(case[:7]))
-    y_orc, bound = c.oracle_full(torch.bfloat16)
-    assert y_orc.shape[2] % 2 == 0
-    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16)
-    assert_within(y, y_orc, bound, out_bf16=True, what="row pairs %s" % (case,))
-    res = torch.randn(*y_orc.shape, generator=inputs.generator(3)).to(torch.bfloat16)
-    want = oracle.epilogue(y_orc, res.float().numpy(), relu=True)
-    y = c.run_gpu(tbn.TBN_NHWC, torch.bfloat16, torch.bfloat16, relu=True, residual=res)
-    assert_within(y, want, bound, out_bf16=True, epilogue=True, what="row pairs epi %s" % (case,))
+    _check_staged_outputs(case, "row pairs")
 
 
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
-@pytest.mark.parametrize("case", [
-    (64, 64, 28, 28, 48, 3, 3, (1, 1), (1, 1)),
-    (48, 64, 33, 56, 8, 2, 3, (1, 2), (0, 1)),
-    (64, 64, 30, 31, 56, 5, 5, (1, 1), (2, 2)),
+@pytest.mark.parametrize("case,mode", [
+    ((64, 64, 28, 28, 48, 3, 3, (1, 1), (1, 1)), "rowpair"),
+    ((48, 64, 33, 56, 8, 2, 3, (1, 2), (0, 1)), "rowpair"),
+    ((64, 64, 30, 31, 56, 5, 5, (1, 1), (2, 2)), "rowpair"),
+    ((34, 64, 16, 16, 48, 3, 3, (1, 1), (1, 1)), "tma64"),
 ])
-def test_row_pairs_not_finite(case, value):
+def test_row_pairs_not_finite(case, mode, value):
     """An infinite or NaN input reaches the outputs whose taps read it and no
     others, although both rows of a pair are computed from the same boxes."""
-    assert tbn._conv_mode(*case) == "rowpair"
+    assert tbn._conv_mode(*case) == mode
     N, C, H, W, K, R, S, st, pd = case
     g = inputs.generator(11)
     x = torch.randn(N, C, H, W, generator=g)

@@ -50,6 +50,17 @@ def test_dense_tc_matches_oracle(case):
         assert np.all(err <= tol), float(np.max(err - tol))
 
 
+def test_dense_tc_single_products():
+    """One tap, 24-bit weights: each output is a single product rounded once to
+    bf16, at most half an ulp away."""
+    g = inputs.generator(9)
+    x = torch.ones(1, 1, 8, 8, dtype=torch.bfloat16)
+    w = (torch.rand(64, 1, 1, 1, generator=g) + 1) * (1 + 2.0 ** -23)
+    y = _run(x, w, (1, 2), (0, 0))
+    want = w.reshape(1, 64, 1, 1).double().numpy() * np.ones(y.shape)
+    assert np.array_equal(y, torch.from_numpy(want).to(torch.bfloat16).float().numpy())
+
+
 def test_dense_tc_weight_terms():
     """Weights that need all three terms: two taps cancel to a few units of the
     24th bit, which the result holds exactly; without the third term, or with it
